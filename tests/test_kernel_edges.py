@@ -1,0 +1,69 @@
+"""Kernels at the sizes where they can go wrong: edges of tiles, remainders, smallest and largest
+of a dispatch's range, against 64-bit references of the same operation.
+
+Solves are judged by their backward error ||D - Q X|| / (||Q|| ||X||), which a stable FP32 solve
+keeps at a small multiple of the unit roundoff (6e-8) whatever the condition of Q; 2e-6 leaves
+room for the growth with the matrix size (n u at n = 33) and for the transform in front of it
+(bf16x3, about 1e-5 of the right-hand side, does not enter: the residual is taken against the
+spectra the library itself computed for a unit-diagonal set).
+"""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+def _hpd(rng, nf, n):
+    A = rng.standard_normal((nf, n, n + 4)) + 1j * rng.standard_normal((nf, n, n + 4))
+    Q = A @ A.conj().transpose(0, 2, 1) / (n + 4) + 0.05 * np.eye(n)
+    return (0.5 * (Q + Q.conj().transpose(0, 2, 1))).astype(np.complex64)
+
+
+def _line_ctx(n, nf, nt, precision):
+    """A context on a small grid with n receivers (two may share a column when n is large)."""
+    from paper_2512_16642_gb300 import egh
+
+    nx = max(64, n)
+    return egh.Context(4, nx, 10.0, 10.0, 0, 0.5, 1e-3, nt, np.zeros(n, np.int32),
+                       np.arange(n, dtype=np.int32) % nx, np.linspace(5.0, 40.0, nf), precision=precision)
+
+
+def _load_set(ctx, Q, tmp_path):
+    """Puts given Hessians into a context through the set-file format (egh_save / egh_load)."""
+    import json
+    import struct
+
+    nf, n, _ = Q.shape
+    h = json.dumps({"format": "egh Hessian set", "version": 1, "nrec": n, "nfreq": nf,
+                    "freq_hz": [float(f) for f in ctx.freqs], "dt": 1e-3, "nt": ctx.nt,
+                    "precision": ctx.prec_for_test, "mu": 0.05, "rec_iz": [0] * n,
+                    "rec_ix": [int(i) % max(64, n) for i in range(n)]}).encode()
+    p = tmp_path / "set.bin"
+    p.write_bytes(b"EGHQSET1" + struct.pack("<Q", len(h)) + h + Q.tobytes() + Q.tobytes())
+    ctx.load(str(p))
+
+
+@pytest.mark.parametrize("precision", [0, 1, 2])
+@pytest.mark.parametrize("n,ns", [(1, 1), (2, 3), (31, 16), (32, 17), (33, 4), (64, 5), (65, 33), (161, 57),
+                                  (230, 1), (345, 40)])
+def test_solve_backward_error(n, ns, precision, tmp_path):
+    """X of egh_deblur_freq against the spectra D (the same transform with Q = I): Q X = D."""
+    import torch
+
+    rng = np.random.default_rng(100 * n + ns)
+    nf, nt = 3, 200
+    Q = _hpd(rng, nf, n)
+    r = torch.from_numpy(rng.standard_normal((ns, n, nt)).astype(np.float32)).cuda()
+    out = {}
+    for name, M in (("D", np.broadcast_to(np.eye(n, dtype=np.complex64), Q.shape).copy()), ("X", Q)):
+        with _line_ctx(n, nf, nt, precision) as ctx:
+            ctx.prec_for_test = precision
+            _load_set(ctx, M, tmp_path)
+            x = torch.zeros((nf, n, ns, 2), device="cuda")
+            ctx.deblur_freq(r, x)
+            torch.cuda.synchronize()
+            out[name] = torch.view_as_complex(x).cpu().numpy().astype(np.complex128)
+    for k in range(nf):
+        q = Q[k].astype(np.complex128)
+        res = np.linalg.norm(out["D"][k] - q @ out["X"][k])
+        assert res <= 2e-6 * np.linalg.norm(q, 2) * np.linalg.norm(out["X"][k]), (k, res)
