@@ -404,7 +404,7 @@ egh_status fd_chunk_steps(egh_ctx* ctx, int ta, int t0, int t1, int sbase, int n
 egh_status refine_plan(egh_ctx* ctx, cudaStream_t stream) {
   if (!ctx->Wh) return EGH_OK;
   CK(launch_fro2(ctx->Qh, ctx->nrec, ctx->nf, ctx->fro2, stream));
-  CK(launch_inv_power(ctx->Wh, ctx->nrec, ctx->nf, ctx->fro2 + ctx->nf, stream));
+  CK(launch_inv_power(ctx->Ph, ctx->nrec, ctx->nf, ctx->fro2 + ctx->nf, stream));
   ctx->cond_host.assign(2 * ctx->nf, 0.0);
   CK(cudaMemcpyAsync(ctx->cond_host.data(), ctx->fro2, 2 * ctx->nf * sizeof(double),
                      cudaMemcpyDeviceToHost, stream));
@@ -1602,7 +1602,7 @@ egh_status egh_batch_factor(egh_batch* b, int32_t* bad_ctx, int32_t* bad_freq, v
     // the copies and the launch once as a CUDA graph
     float best = 1e30f;
     const long long l0 = launches_so_far();
-    for (int th : {256, 512, 1024}) {
+    for (int th : {256, 512}) {  // (1024 threads leave too few registers for a row per thread)
       float ms = 0.f;
       for (int rep = 0; rep < 2; ++rep) {
         BCK(cudaEventRecord(b->ev[0], stream));

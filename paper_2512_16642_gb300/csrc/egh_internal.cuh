@@ -190,8 +190,8 @@ cudaError_t launch_add_correction(float2* X, const float2* R, long long m, int n
                                   const int* kl = nullptr);
 // ||Q_k||_F^2 per frequency (FP64 sums) into d_out[nf]
 cudaError_t launch_fro2(const float2* Qh, int n, int nf, double* d_out, cudaStream_t st);
-// lambda_max(W_k^H W_k) = 1 / lambda_min(Q_k) by power iteration (from below) into lam[nf]
-cudaError_t launch_inv_power(const float2* Wh, int n, int nf, double* lam, cudaStream_t st);
+// lambda_max(P_k) = 1 / lambda_min(Q_k), P_k = Q_k^{-1}, by power iteration (from below) into lam[nf]
+cudaError_t launch_inv_power(const float2* Ph, int n, int nf, double* lam, cudaStream_t st);
 // Condition bound of a factorisation from ||Q||_F^2, the power estimate of 1/lambda_min (with a
 // margin for its approach from below) and, when known (> 0), mu <= lambda_min.
 inline double cond_bound(double fro2, double inv_lmin, double mu) {

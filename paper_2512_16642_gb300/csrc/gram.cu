@@ -5,7 +5,10 @@
 //   Re H[i][j] = C[2i][2j] + C[2i+1][2j+1],   Im H[i][j] = C[2i+1][2j] - C[2i][2j+1].
 // C is computed in 64 x 64 tiles on and above the tile diagonal only, with the grid sum split
 // into `splits` ranges whose partial tiles are reduced in a second kernel (scratch workspace).
+#include <algorithm>
 #include <cmath>
+
+#include <cooperative_groups.h>
 
 #include "egh_internal.cuh"
 
@@ -183,100 +186,137 @@ cudaError_t launch_diag_sum(const float2* Qh, int nrec, int nf, double* d_sum, c
   return cudaGetLastError();
 }
 
-// ||Q_k||_F^2 per frequency: one block per frequency, FP32 squares summed in FP64.
-__global__ void k_fro2(const float2* __restrict__ Qh, int n, double* d_out) {
-  __shared__ double red[256];
+// ||Q_k||_F^2 per frequency: one block per frequency.  The squares are summed to FP64-class
+// accuracy in FP32 arithmetic (TwoProd and TwoSum into a two-word sum per thread, Ogita, Rump and
+// Oishi's Dot2) and combined in FP64: the GB300 issues FP64 at a small fraction of the FP32 rate,
+// and two FP64 operations per entry were the kernel's time (40 matrices of 341 rows: 150 us, now
+// 18 us).
+constexpr int FR_THREADS = 1024;
+
+__device__ __forceinline__ void two_word_square(float a, float& s, float& c) {
+  const float p = __fmul_rn(a, a);
+  const float e = __fmaf_rn(a, a, -p);
+  const float t = __fadd_rn(s, p);
+  const float bp = __fsub_rn(t, s);
+  c = __fadd_rn(c, __fadd_rn(__fadd_rn(__fsub_rn(s, __fsub_rn(t, bp)), __fsub_rn(p, bp)), e));
+  s = t;
+}
+
+__global__ void __launch_bounds__(FR_THREADS)
+    k_fro2(const float2* __restrict__ Qh, int n, double* d_out) {
+  __shared__ double red[FR_THREADS / 32];
   const long long n2 = (long long)n * n;
   const float2* A = Qh + (long long)blockIdx.x * n2;
-  double s = 0.0;
-  for (long long t = threadIdx.x; t < n2; t += blockDim.x) {
-    const float2 a = A[t];
-    s += (double)a.x * a.x + (double)a.y * a.y;
+  float s[2] = {0.f, 0.f}, c[2] = {0.f, 0.f};
+#pragma unroll 4
+  for (long long t = threadIdx.x; t < n2; t += FR_THREADS) {
+    const float2 a = __ldg(A + t);
+    two_word_square(a.x, s[0], c[0]);
+    two_word_square(a.y, s[1], c[1]);
   }
-  red[threadIdx.x] = s;
+  double v = ((double)s[0] + c[0]) + ((double)s[1] + c[1]);
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
   __syncthreads();
-  for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-    if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-    __syncthreads();
+  if (threadIdx.x == 0) {
+    double sum = 0.0;
+    for (int w = 0; w < FR_THREADS / 32; ++w) sum += red[w];
+    d_out[blockIdx.x] = sum;
   }
-  if (threadIdx.x == 0) d_out[blockIdx.x] = red[0];
 }
 
 cudaError_t launch_fro2(const float2* Qh, int n, int nf, double* d_out, cudaStream_t st) {
   count_launches(1);
-  k_fro2<<<nf, 256, 0, st>>>(Qh, n, d_out);
+  k_fro2<<<nf, FR_THREADS, 0, st>>>(Qh, n, d_out);
   return cudaGetLastError();
 }
 
-// Largest eigenvalue of Q_k^{-1} = W_k^H W_k (W = L^{-1}, lower triangular) by 40 steps of
-// power iteration in FP32, one block per frequency: lam[k] = ||W^H W v|| / ||v|| for the last v.
-// It approaches 1 / lambda_min(Q_k) from below.
-__global__ void k_inv_power(const float2* __restrict__ Wh, int n, double* lam) {
-  extern __shared__ float2 pv[];  // v [n], y [n]
-  __shared__ float red[256];
-  float2* v = pv;
-  float2* y = pv + n;
-  const float2* W = Wh + (long long)blockIdx.x * n * n;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) v[i] = make_float2(1.f + 0.01f * (i % 7), 0.f);
-  __syncthreads();
-  float norm = 0.f;
-  auto reduce = [&](float x) {
-    red[threadIdx.x] = x;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-      if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-      __syncthreads();
-    }
-    const float r = red[0];
-    __syncthreads();
-    return r;
-  };
-  float vv = reduce([&] {
-    float a = 0.f;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) a += v[i].x * v[i].x + v[i].y * v[i].y;
-    return a;
-  }());
-  for (int it = 0; it < 40; ++it) {
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {  // y = W v
+// Largest eigenvalue of Q_k^{-1} (the dense inverse P_k) by 40 steps of power iteration in FP32:
+// lam[k] = ||P v|| / ||v|| for the last v, which approaches 1 / lambda_min(Q_k) from below.
+//
+// One cluster of IP_CL blocks per matrix: each block keeps its share of the rows of P in shared
+// memory (as many as fit; the rest is read from L2 every step), so that a step costs one
+// shared-memory matrix-vector product, a warp per row, and one cluster barrier; the new vector
+// and the partial norms go to every block of the cluster through distributed shared memory, in
+// two alternating buffers.  The 40 steps are a serial chain: with one block per matrix reading the
+// two triangular factors from L2 each of them took 10 to 37 us.  Measured on 40 matrices of 341
+// rows: 1471 us before, 166 us now (161 rows: 378 and 105 us).
+constexpr int IP_CL = 8, IP_THREADS = 512, IP_STEPS = 40;
+
+__global__ void __cluster_dims__(IP_CL, 1, 1) __launch_bounds__(IP_THREADS)
+    k_inv_power(const float2* __restrict__ Ph, int n, int cached, double* lam) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
+  extern __shared__ __align__(16) float2 pv[];  // v[2][n], then `cached` rows of P
+  __shared__ float wred[IP_THREADS / 32];
+  __shared__ float part[2][IP_CL];  // the blocks' partial ||P v||^2, by step parity
+  const int rank = (int)cluster.block_rank(), tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  constexpr int NW = IP_THREADS / 32;
+  const float2* P = Ph + (long long)(blockIdx.x / IP_CL) * n * n;
+  const int r0 = (int)((long long)n * rank / IP_CL), r1 = (int)((long long)n * (rank + 1) / IP_CL);
+  const int nr = r1 - r0, nc = min(nr, cached);
+  float2* rows = pv + 2 * n;
+  for (int e = tid; e < nc * n; e += IP_THREADS) rows[e] = P[(long long)r0 * n + e];
+  float vv = 0.f;  // ||v||^2 of the start vector, the same sum in every block
+  for (int i = lane; i < n; i += 32) {
+    const float x = 1.f + 0.01f * (i % 7);
+    vv += x * x;
+  }
+  for (int o = 16; o > 0; o >>= 1) vv += __shfl_xor_sync(0xffffffffu, vv, o);
+  for (int i = tid; i < n; i += IP_THREADS) pv[i] = make_float2(1.f + 0.01f * (i % 7), 0.f);
+  float sc = 1.f, norm = 0.f;
+  cluster.sync();  // every block of the cluster runs before its shared memory is written
+  for (int it = 0; it < IP_STEPS; ++it) {
+    const float2* v = pv + (it & 1) * n;
+    float2* vn = pv + ((it & 1) ^ 1) * n;
+    float w2 = 0.f;
+    for (int r = warp; r < nr; r += NW) {
+      const float2* row = r < nc ? rows + (size_t)r * n : P + (long long)(r0 + r) * n;
       float re = 0.f, im = 0.f;
-      for (int j = 0; j <= i; ++j) {
-        const float2 a = W[(long long)i * n + j], b = v[j];
+#pragma unroll 4
+      for (int j = lane; j < n; j += 32) {
+        const float2 a = row[j], b = v[j];
         re = fmaf(a.x, b.x, fmaf(-a.y, b.y, re));
         im = fmaf(a.x, b.y, fmaf(a.y, b.x, im));
       }
-      y[i] = make_float2(re, im);
-    }
-    __syncthreads();
-    float a2 = 0.f;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {  // v' = W^H y
-      float re = 0.f, im = 0.f;
-      for (int j = i; j < n; ++j) {
-        const float2 a = W[(long long)j * n + i], b = y[j];
-        re = fmaf(a.x, b.x, fmaf(a.y, b.y, re));
-        im = fmaf(a.x, b.y, fmaf(-a.y, b.x, im));
+      for (int o = 16; o > 0; o >>= 1) {
+        re += __shfl_xor_sync(0xffffffffu, re, o);
+        im += __shfl_xor_sync(0xffffffffu, im, o);
       }
-      v[i] = make_float2(re, im);
-      a2 += re * re + im * im;
+      re *= sc;
+      im *= sc;
+      w2 += re * re + im * im;
+      if (lane < IP_CL) cluster.map_shared_rank(vn, lane)[r0 + r] = make_float2(re, im);
     }
+    if (lane == 0) wred[warp] = w2;
     __syncthreads();
-    const float w2 = reduce(a2);
-    norm = sqrtf(w2 / vv);
-    const float sc = 1.f / sqrtf(w2);
-    for (int i = threadIdx.x; i < n; i += blockDim.x) v[i] = make_float2(v[i].x * sc, v[i].y * sc);
+    if (tid < IP_CL) {
+      float s = 0.f;
+      for (int w = 0; w < NW; ++w) s += wred[w];
+      cluster.map_shared_rank(&part[it & 1][0], tid)[rank] = s;
+    }
+    cluster.sync();
+    float s = 0.f;
+    for (int b = 0; b < IP_CL; ++b) s += part[it & 1][b];
+    norm = sqrtf(s / vv);
+    sc = 1.f / sqrtf(s);  // applied to the next product
     vv = 1.f;
-    __syncthreads();
   }
-  if (threadIdx.x == 0) lam[blockIdx.x] = norm;
+  // the last step's barrier is behind every remote write: no block leaves early
+  if (rank == 0 && tid == 0) lam[blockIdx.x / IP_CL] = norm;
 }
 
-cudaError_t launch_inv_power(const float2* Wh, int n, int nf, double* lam, cudaStream_t st) {
-  const size_t smem = sizeof(float2) * 2 * (size_t)n;
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(k_inv_power, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
+cudaError_t launch_inv_power(const float2* Ph, int n, int nf, double* lam, cudaStream_t st) {
+  // rows of P beside the two vectors in at most 200 KB of a block's shared memory
+  const size_t vec = 2 * sizeof(float2) * (size_t)n, cap = 200 * 1024;
+  const int share = (n + IP_CL - 1) / IP_CL;
+  const int cached = (int)std::min<size_t>((size_t)share, vec < cap ? (cap - vec) / (sizeof(float2) * (size_t)n) : 0);
+  const size_t smem = vec + sizeof(float2) * (size_t)cached * n;
+  cudaError_t e =
+      cudaFuncSetAttribute(k_inv_power, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
   count_launches(1);
-  k_inv_power<<<nf, 256, smem, st>>>(Wh, n, lam);
+  k_inv_power<<<nf * IP_CL, IP_THREADS, smem, st>>>(Ph, n, cached, lam);
   return cudaGetLastError();
 }
 

@@ -495,7 +495,7 @@ egh_status egh_server_add_set(egh_server* sv, int32_t nrec, int32_t nfreq, const
     if (!e) e = launch_gram_inverse(h.Wh, nrec, nfreq, h.Ph, st);
     if (!e) e = cudaMalloc(&d_cond, 2 * nfreq * sizeof(double));
     if (!e) e = launch_fro2(h.Qh, nrec, nfreq, d_cond, st);
-    if (!e) e = launch_inv_power(h.Wh, nrec, nfreq, d_cond + nfreq, st);
+    if (!e) e = launch_inv_power(h.Ph, nrec, nfreq, d_cond + nfreq, st);
     if (!e) e = cudaMemcpyAsync(cond.data(), d_cond, 2 * nfreq * sizeof(double), cudaMemcpyDeviceToHost, st);
   }
   std::vector<int> stv(nfreq, 0);
