@@ -4,7 +4,7 @@
 //                                                                  k_trace_dft_tc otherwise)
 //   X_k = L_k^{-H} L_k^{-1} D_k                                   (k_trsm, all sources as RHS)
 //   mixed precision: X_k = Q_k^{-1} D_k with Q_k^{-1} = W_k^H W_k, W_k = L_k^{-1} (k_trtri and
-//                    k_cgemm once per factorisation; the product on the tensor cores in
+//                    k_gram_inverse once per factorisation; the product on the tensor cores in
 //                    solve_tc.cu), then at ill-conditioned frequencies
 //                    X_k += Q_k^{-1} (D_k - Q_k X_k)                (k_resid_dot2 or k_resid64)
 //   mult[s][r][t] = sum_k w_k Re(X_k[r][s] exp(+i w_k t dt))      (k_synth_operands + k_synth_tma
@@ -720,54 +720,54 @@ cudaError_t launch_trace_tma(const float* resid, int ntr, int nt_d, const unsign
 constexpr int TS_W = 8;               // warps per block (also of the residual kernels)
 constexpr int TR_B = 32, TR_C = 16;   // block rows, sources per block
 
-__global__ void __launch_bounds__(32 * TS_W)
-    k_trsm(const float2* __restrict__ Lh, int n, float2* __restrict__ Dh, int ns) {
-  extern __shared__ __align__(16) float2 Y[];  // [n][TR_C]
-  __shared__ float2 Ls[2][TR_B][TR_B + 1];
-  const int k = blockIdx.y, c0 = blockIdx.x * TR_C;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const float2* L = Lh + (long long)k * n * n;
-  float2* B = Dh + (long long)k * n * ns;
-  for (int e = tid; e < n * TR_C; e += 32 * TS_W) {
-    const int i = e / TR_C, c = c0 + e % TR_C;
-    Y[e] = c < ns ? B[(long long)i * ns + c] : make_float2(0.f, 0.f);
-  }
-  const int nb = (n + TR_B - 1) / TR_B;
-  const int r = tid >> 3, c = 2 * (tid & 7);  // this thread's output of a block row
+// One block's solve: Y [rows][TR_C] in shared memory against the lower triangle L (n x n).
+struct TriSolve {
+  const float2* L;
+  int n;
+  float2* Y;
+  float2 (*Ls)[TR_B][TR_B + 1];  // two tiles
+  int buf;
   float2 pre[4];
-  auto load = [&](int rb, int cb) {  // tile (rb, cb) of L: 4 entries per thread, zero past n
+
+  // tile (rb, cb) of L into registers: 4 entries per thread, zero past n
+  __device__ void load(int rb, int cb) {
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      const int e = tid + 256 * q, i = rb * TR_B + (e >> 5), j = cb * TR_B + (e & 31);
+      const int e = threadIdx.x + 256 * q, i = rb * TR_B + (e >> 5), j = cb * TR_B + (e & 31);
       pre[q] = (i < n && j < n) ? L[(long long)i * n + j] : make_float2(0.f, 0.f);
     }
-  };
-  int buf = 0;
-  auto put = [&]() {  // the loaded tile into the other buffer: its readers passed a barrier since
+  }
+  // the loaded tile into the other buffer: its readers have passed a barrier since
+  __device__ void put() {
     buf ^= 1;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      const int e = tid + 256 * q;
+      const int e = threadIdx.x + 256 * q;
       Ls[buf][e >> 5][e & 31] = pre[q];
     }
     __syncthreads();
-  };
-  // acc[c..c+1] += op(tile)[r][:] Y[block jb][c..c+1]
-  auto sums = [&](int jb, bool conjt, float2 (&acc)[2]) {
+  }
+  // acc += op(tile)[r][:] Y[block jb][c..c+1], r = thread / 8, c = 2 (thread % 8)
+  template <bool CONJT>
+  __device__ void sums(int jb, float2 (&acc)[2]) {
+    const int r = threadIdx.x >> 3, c = 2 * (threadIdx.x & 7);
     const int j0 = jb * TR_B, nk = min(TR_B, n - j0);
 #pragma unroll 8
     for (int kk = 0; kk < nk; ++kk) {
-      float2 l = conjt ? Ls[buf][kk][r] : Ls[buf][r][kk];
-      if (conjt) l.y = -l.y;
+      float2 l = CONJT ? Ls[buf][kk][r] : Ls[buf][r][kk];
+      if (CONJT) l.y = -l.y;
       const float4 y = *reinterpret_cast<const float4*>(Y + (j0 + kk) * TR_C + c);
       acc[0].x = fmaf(l.x, y.x, fmaf(-l.y, y.y, acc[0].x));
       acc[0].y = fmaf(l.x, y.y, fmaf(l.y, y.x, acc[0].y));
       acc[1].x = fmaf(l.x, y.z, fmaf(-l.y, y.w, acc[1].x));
       acc[1].y = fmaf(l.x, y.w, fmaf(l.y, y.z, acc[1].y));
     }
-  };
+  }
   // subtract the sums from block row ib, then solve it against the diagonal tile (in Ls[buf])
-  auto finish = [&](int ib, bool conjt, const float2 (&acc)[2]) {
+  template <bool CONJT>
+  __device__ void finish(int ib, const float2 (&acc)[2]) {
+    const int r = threadIdx.x >> 3, c = 2 * (threadIdx.x & 7);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int i0 = ib * TR_B;
     if (i0 + r < n) {
       float4* y = reinterpret_cast<float4*>(Y + (i0 + r) * TR_C + c);
@@ -781,13 +781,13 @@ __global__ void __launch_bounds__(32 * TS_W)
     const float d = in ? 1.f / Ls[buf][lane][lane].x : 0.f;
     const int nr = min(TR_B, n - i0);
     for (int q = 0; q < nr; ++q) {
-      const int p = conjt ? nr - 1 - q : q;
+      const int p = CONJT ? nr - 1 - q : q;
       if (lane == p) s = make_float4(s.x * d, s.y * d, s.z * d, s.w * d);
       const float yx = __shfl_sync(0xffffffffu, s.x, p), yy = __shfl_sync(0xffffffffu, s.y, p);
       const float yz = __shfl_sync(0xffffffffu, s.z, p), yw = __shfl_sync(0xffffffffu, s.w, p);
-      if (conjt ? lane < p : lane > p) {
-        float2 l = conjt ? Ls[buf][p][lane] : Ls[buf][lane][p];
-        if (conjt) l.y = -l.y;
+      if (CONJT ? lane < p : lane > p) {
+        float2 l = CONJT ? Ls[buf][p][lane] : Ls[buf][lane][p];
+        if (CONJT) l.y = -l.y;
         s.x = fmaf(-l.x, yx, fmaf(l.y, yy, s.x));
         s.y = fmaf(-l.x, yy, fmaf(-l.y, yx, s.y));
         s.z = fmaf(-l.x, yz, fmaf(l.y, yw, s.z));
@@ -796,37 +796,60 @@ __global__ void __launch_bounds__(32 * TS_W)
     }
     if (in) *yp = s;
     __syncthreads();
-  };
-  load(0, 0);
-  for (int ib = 0; ib < nb; ++ib) {  // L y = d
-    float2 acc[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-    for (int jb = 0; jb <= ib; ++jb) {
-      put();
-      if (jb < ib)
-        load(ib, jb + 1);
-      else if (ib + 1 < nb)
-        load(ib + 1, 0);
-      else
-        load(nb - 1, nb - 1);  // the backward pass begins with its diagonal tile
-      if (jb < ib) sums(jb, false, acc);
-    }
-    finish(ib, false, acc);
   }
-  for (int ib = nb - 1; ib >= 0; --ib) {  // L^H x = y
-    float2 acc[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-    for (int jb = nb - 1; jb >= ib; --jb) {
-      put();
-      if (jb > ib)
-        load(jb - 1, ib);
-      else if (ib > 0)
-        load(nb - 1, ib - 1);
-      if (jb > ib) sums(jb, true, acc);
+  // L y = d; tile (0, 0) is loaded already, the last diagonal tile is loaded at the end
+  __device__ void forward() {
+    const int nb = (n + TR_B - 1) / TR_B;
+    for (int ib = 0; ib < nb; ++ib) {
+      float2 acc[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+      for (int jb = 0; jb <= ib; ++jb) {
+        put();
+        if (jb < ib)
+          load(ib, jb + 1);
+        else if (ib + 1 < nb)
+          load(ib + 1, 0);
+        else
+          load(nb - 1, nb - 1);
+        if (jb < ib) sums<false>(jb, acc);
+      }
+      finish<false>(ib, acc);
     }
-    finish(ib, true, acc);
   }
+  // L^H x = y; the last diagonal tile is loaded already
+  __device__ void backward() {
+    const int nb = (n + TR_B - 1) / TR_B;
+    for (int ib = nb - 1; ib >= 0; --ib) {
+      float2 acc[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+      for (int jb = nb - 1; jb >= ib; --jb) {
+        put();
+        if (jb > ib)
+          load(jb - 1, ib);
+        else if (ib > 0)
+          load(nb - 1, ib - 1);
+        if (jb > ib) sums<true>(jb, acc);
+      }
+      finish<true>(ib, acc);
+    }
+  }
+};
+
+__global__ void __launch_bounds__(32 * TS_W)
+    k_trsm(const float2* __restrict__ Lh, int n, float2* __restrict__ Dh, int ns) {
+  extern __shared__ __align__(16) float2 Y[];  // [n][TR_C]
+  __shared__ float2 Ls[2][TR_B][TR_B + 1];
+  const int k = blockIdx.y, c0 = blockIdx.x * TR_C, tid = threadIdx.x;
+  float2* B = Dh + (long long)k * n * ns;
   for (int e = tid; e < n * TR_C; e += 32 * TS_W) {
-    const int i = e / TR_C, cc = c0 + e % TR_C;
-    if (cc < ns) B[(long long)i * ns + cc] = Y[e];
+    const int i = e / TR_C, c = c0 + e % TR_C;
+    Y[e] = c < ns ? B[(long long)i * ns + c] : make_float2(0.f, 0.f);
+  }
+  TriSolve t{Lh + (long long)k * n * n, n, Y, Ls, 0, {}};
+  t.load(0, 0);
+  t.forward();
+  t.backward();
+  for (int e = tid; e < n * TR_C; e += 32 * TS_W) {
+    const int i = e / TR_C, c = c0 + e % TR_C;
+    if (c < ns) B[(long long)i * ns + c] = Y[e];
   }
 }
 
@@ -933,137 +956,231 @@ __global__ void __launch_bounds__(256)
 // ---------------------------------------------------------------------------------------------
 // Explicit inverse of the Cholesky factor, W_k = L_k^{-1} (lower triangular), for solves as
 // matrix products X = W^H (W D).  Column j of W solves L w = e_j by forward substitution,
-// w_i = -(sum_{l=j}^{i-1} L_il w_l) / L_ii.  One warp per (frequency, column): the lanes split
-// each row's sum (coalesced reads of row i of L) and the column so far sits in shared memory.
+// w_i = -(sum_{l=j}^{i-1} L_il w_l) / L_ii, the sum split over the lanes of a warp (lane l - j
+// mod 32) and combined by a butterfly.
+//
+// A warp takes CB columns j, j + 32, ... of one residue: they share every lane's entries of L, so
+// a row of L is read once for CB columns (and one row ahead), their chains overlap, and the
+// butterflies of the CB complex sums run together, halving the values at each step (9 exchanges
+// in place of 5 per sum for CB = 4).  The chain of n rows bounds it: one column per warp, each
+// row of L read from L2 behind the previous row's butterfly, took 512 us on 40 matrices of 341
+// rows; this form takes 383 us, with the same sums in the same
+// order (161 rows: 125 and 123 us).
 // ---------------------------------------------------------------------------------------------
-constexpr int TRI_WARPS = 4;
+constexpr int TRI_WARPS = 4, TRI_PRE = 12;  // warps per block; 32-entry groups of a row read ahead
 
+template <int CB>
 __global__ void __launch_bounds__(32 * TRI_WARPS)
-    k_trtri(const float2* __restrict__ Lh, int n, int nf, float2* __restrict__ Wh) {
-  extern __shared__ float2 wcol[];  // [TRI_WARPS][n]
+    k_trtri(const float2* __restrict__ Lh, int n, int groups, float2* __restrict__ Wh) {
+  extern __shared__ __align__(16) float2 wcol[];  // [TRI_WARPS][CB][groups][32]
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-  const long long t = blockIdx.x * (long long)TRI_WARPS + wp;
-  if (t >= (long long)n * nf) return;  // warp-uniform
-  const int k = (int)(t / n), j = (int)(t % n);
-  const float2* L = Lh + (long long)k * n * n;
-  float2* W = Wh + (long long)k * n * n;
-  float2* w = wcol + (size_t)wp * n;
-  for (int i = lane; i < j; i += 32) W[(long long)i * n + j] = make_float2(0.f, 0.f);
-  const float wjj = 1.f / L[(long long)j * n + j].x;
-  if (lane == 0) {
-    w[j] = make_float2(wjj, 0.f);
-    W[(long long)j * n + j] = w[j];
+  const int t = blockIdx.x * TRI_WARPS + wp;
+  const int jb = t % 32 + 32 * CB * (t / 32);  // first column
+  if (jb >= n) return;                         // warp-uniform; warps are independent
+  const float2* L = Lh + (long long)blockIdx.y * n * n;
+  float2* W = Wh + (long long)blockIdx.y * n * n;
+  float2* w = wcol + (size_t)wp * CB * groups * 32;  // w[c][m][lane]: entry jb + lane + 32 m
+  // zero where no entry is known yet
+  for (int e = lane; e < CB * groups * 32; e += 32) w[e] = make_float2(0.f, 0.f);
+  __syncwarp();
+#pragma unroll
+  for (int c = 0; c < CB; ++c) {
+    const int j = jb + 32 * c;
+    if (j < n) {
+      for (int i = lane; i < j; i += 32) W[(long long)i * n + j] = make_float2(0.f, 0.f);
+      if (lane == 0) {
+        const float2 v = make_float2(1.f / L[(long long)j * n + j].x, 0.f);
+        w[(c * groups + c) * 32] = v;
+        W[(long long)j * n + j] = v;
+      }
+    }
   }
   __syncwarp();
-  for (int i = j + 1; i < n; ++i) {
-    const float2* Li = L + (long long)i * n;
-    float2 acc = make_float2(0.f, 0.f);
-    for (int l = j + lane; l < i; l += 32) {
-      const float2 a = Li[l], v = w[l];
-      acc.x = fmaf(a.x, v.x, fmaf(-a.y, v.y, acc.x));
-      acc.y = fmaf(a.x, v.y, fmaf(a.y, v.x, acc.y));
+  // the lane's entries jb + lane + 32 m < i of row i, and the pivot
+  float2 pre[TRI_PRE];
+  float piv = 0.f;
+  auto load = [&](int i) {
+    const float2* Li = L + (long long)i * n + jb + lane;
+    piv = __ldg(&L[(long long)i * n + i].x);
+#pragma unroll
+    for (int m = 0; m < TRI_PRE; ++m)
+      pre[m] = jb + lane + 32 * m < i ? __ldg(Li + 32 * m) : make_float2(0.f, 0.f);
+  };
+  if (jb + 1 < n) load(jb + 1);
+  for (int i = jb + 1; i < n; ++i) {
+    float2 cur[TRI_PRE];
+#pragma unroll
+    for (int m = 0; m < TRI_PRE; ++m) cur[m] = pre[m];
+    const float d = -1.f / piv;
+    if (i + 1 < n) load(i + 1);  // one row ahead
+    const int mi = (i - jb) >> 5;        // entry i is lane (i - jb) % 32 of group mi
+    const int ng = (i - 1 - jb) >> 5;    // the last group with entries below i
+    float2 acc[CB];
+#pragma unroll
+    for (int c = 0; c < CB; ++c) acc[c] = make_float2(0.f, 0.f);
+    auto add = [&](int m, float2 a) {
+#pragma unroll
+      for (int c = 0; c < CB; ++c)
+        if (m >= c) {
+          const float2 v = w[(c * groups + m) * 32 + lane];
+          acc[c].x = fmaf(a.x, v.x, fmaf(-a.y, v.y, acc[c].x));
+          acc[c].y = fmaf(a.x, v.y, fmaf(a.y, v.x, acc[c].y));
+        }
+    };
+#pragma unroll
+    for (int m = 0; m < TRI_PRE; m += 4)
+      if (m <= ng) {  // (a group's entries at and past i are zero, as are w's rows not yet set)
+#pragma unroll
+        for (int q = m; q < m + 4; ++q) add(q, cur[q]);
+      }
+    for (int m = TRI_PRE; m <= ng; ++m) {
+      const int l = jb + lane + 32 * m;
+      add(m, l < i ? __ldg(L + (long long)i * n + l) : make_float2(0.f, 0.f));
     }
+    // butterfly sums over 16, 8, 4, 2, 1: while more than one value is left, a lane keeps one half
+    // of them and hands over the other half
+    float v[2 * CB];
+#pragma unroll
+    for (int c = 0; c < CB; ++c) {
+      v[2 * c] = acc[c].x;
+      v[2 * c + 1] = acc[c].y;
+    }
+    int idx = 0;  // the value this lane ends up with
+    int cnt = 2 * CB;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-      acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
-      acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
+      if (cnt > 1) {
+        cnt >>= 1;
+        const bool up = (lane & o) != 0;
+        if (up) idx += cnt;
+#pragma unroll
+        for (int q = 0; q < CB; ++q)
+          if (q < cnt) {
+            const float keep = up ? v[q + cnt] : v[q], give = up ? v[q] : v[q + cnt];
+            v[q] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+          }
+      } else {
+        v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+      }
     }
-    const float d = -1.f / Li[i].x;
-    if (lane == 0) {
-      w[i] = make_float2(acc.x * d, acc.y * d);
-      W[(long long)i * n + j] = w[i];
+    // one lane per value writes it (the others hold copies)
+    constexpr int REP = 32 / (2 * CB);
+    const int c = idx >> 1, j = jb + 32 * c;
+    if ((lane & (REP - 1)) == 0 && i > j) {
+      const float x = v[0] * d;
+      reinterpret_cast<float*>(w + (c * groups + mi) * 32 + ((i - jb) & 31))[idx & 1] = x;
+      reinterpret_cast<float*>(W + (long long)i * n + j)[idx & 1] = x;
     }
     __syncwarp();
   }
 }
 
 cudaError_t launch_trtri(const float2* Lh, int n, int nf, float2* Wh, cudaStream_t st) {
-  const long long m = (long long)n * nf;
-  const size_t smem = (size_t)TRI_WARPS * n * sizeof(float2);
+  const int groups = ((n + 31) / 32 + 3) / 4 * 4;  // 32-entry groups of a column, by fours
+  const size_t one = sizeof(float2) * TRI_WARPS * 32 * (size_t)groups;  // one column per warp
+  const bool four = 4 * one <= 200 * 1024;  // up to 1536 rows; beyond, a column per warp
+  const size_t smem = four ? 4 * one : one;
+  auto kern = four ? k_trtri<4> : k_trtri<1>;
   if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(k_trtri, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
+  const int cb = four ? 4 : 1, warps = 32 * ((groups + cb - 1) / cb);
   count_launches(1);
-  k_trtri<<<(unsigned)((m + TRI_WARPS - 1) / TRI_WARPS), 32 * TRI_WARPS, smem, st>>>(Lh, n, nf, Wh);
+  kern<<<dim3(warps / TRI_WARPS, nf), 32 * TRI_WARPS, smem, st>>>(Lh, n, groups, Wh);
   return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------------------------
-// Batched complex products C_k = op(W_k) B_k, op = identity or conjugate transpose, W_k n x n,
-// B_k and C_k n x ld (all frequencies in one launch).  32 x 32 output tiles, 32-deep K steps
-// staged in shared memory over the triangle's nonzero range; each of the 256 threads computes a
-// 2 x 2 block.
+// Q_k^{-1} = W_k^H W_k (dense Hermitian n x n), the operator of the tensor-core solve, in FP32:
+// 64 x 64 tiles on and below the diagonal; the mirror of a tile below it shares the real sums and
+// has imaginary sums of its own, in the order of the transposed product; W is lower triangular, so
+// a tile's sum starts at its row block.  A thread holds 4 x 4 entries (12 FMAs per
+// shared-memory read; the 2 x 2 form over both triangles that this replaces was bound by its
+// shared-memory reads: 251 us on 40 matrices of 341 rows, now 155 us).
 // ---------------------------------------------------------------------------------------------
-constexpr int CG_T = 32;
+constexpr int GI_T = 64, GI_K = 16;
 
-template <bool CONJT>
 __global__ void __launch_bounds__(256)
-    k_cgemm(const float2* __restrict__ Wh, int n, const float2* __restrict__ Bh, int ld,
-            float2* __restrict__ Ch, const int* __restrict__ kl) {
-  __shared__ float2 As[CG_T][CG_T + 1];  // As[r][kk] = op(W)[row0 + r][k0 + kk]
-  __shared__ float2 Bs[CG_T][CG_T + 1];  // Bs[kk][c] = B[k0 + kk][col0 + c]
-  const int k = kl ? kl[blockIdx.z] : blockIdx.z;
-  const float2* W = Wh + (long long)k * n * n;
-  const float2* B = Bh + (long long)k * n * ld;
-  float2* C = Ch + (long long)k * n * ld;
-  const int row0 = blockIdx.y * CG_T, col0 = blockIdx.x * CG_T;
-  const int tid = threadIdx.x, tr = (tid >> 4) * 2, tc = (tid & 15) * 2;
-  float2 acc[2][2];
+    k_gram_inverse(const float2* __restrict__ Wh, int n, float2* __restrict__ Ph) {
+  __shared__ float2 sm[GI_T * (GI_T + 1)];  // As[GI_K][GI_T], Bs[GI_K][GI_T]; then the mirror tile
+  float2 (*As)[GI_T] = reinterpret_cast<float2 (*)[GI_T]>(sm);
+  float2 (*Bs)[GI_T] = As + GI_K;
+  int ti = 0, rem = blockIdx.x;
+  while (rem > ti) rem -= ++ti;  // pairs (ti, tj), tj <= ti
+  const int tj = rem, i0 = ti * GI_T, j0 = tj * GI_T;
+  const float2* W = Wh + (long long)blockIdx.y * n * n;
+  float2* P = Ph + (long long)blockIdx.y * n * n;
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  float2 pa[4], pb[4];
+  auto load = [&](int k0) {
 #pragma unroll
-  for (int a = 0; a < 2; ++a)
+    for (int q = 0; q < 4; ++q) {
+      const int e = tid + 256 * q, kk = k0 + (e >> 6), c = e & 63;
+      const bool in = kk < n;
+      pa[q] = in && i0 + c < n ? W[(long long)kk * n + i0 + c] : make_float2(0.f, 0.f);
+      pb[q] = in && j0 + c < n ? W[(long long)kk * n + j0 + c] : make_float2(0.f, 0.f);
+    }
+  };
+  float2 acc[4][4];
+  float mir[4][4];  // the mirror's imaginary sums
 #pragma unroll
-    for (int b = 0; b < 2; ++b) acc[a][b] = make_float2(0.f, 0.f);
-  // W is lower triangular (its upper part stored as zeros): rows row0.. of W need k < row0 + 32,
-  // rows of W^H need k >= row0
-  const int kbeg = CONJT ? row0 : 0, kend = CONJT ? n : min(n, row0 + CG_T);
-  for (int k0 = kbeg; k0 < kend; k0 += CG_T) {
-    for (int e = tid; e < CG_T * CG_T; e += 256) {
-      const int r = e / CG_T, c = e % CG_T;
-      float2 a = make_float2(0.f, 0.f);
-      if (CONJT) {
-        // op(W)[i][kk] = conj(W[kk][i]): read rows of W, coalesced along i
-        const int kk = k0 + r, i = row0 + c;
-        if (kk < n && i < n) a = W[(long long)kk * n + i];
-        As[c][r] = make_float2(a.x, -a.y);
-      } else {
-        const int i = row0 + r, kk = k0 + c;
-        if (i < n && kk < n) a = W[(long long)i * n + kk];
-        As[r][c] = a;
-      }
-      const int kk = k0 + r, cc = col0 + c;
-      Bs[r][c] = (kk < n && cc < ld) ? B[(long long)kk * ld + cc] : make_float2(0.f, 0.f);
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      acc[a][b] = make_float2(0.f, 0.f);
+      mir[a][b] = 0.f;
+    }
+  load(i0);
+  for (int k0 = i0; k0 < n; k0 += GI_K) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int e = tid + 256 * q;
+      As[e >> 6][e & 63] = pa[q];
+      Bs[e >> 6][e & 63] = pb[q];
     }
     __syncthreads();
-#pragma unroll 8
-    for (int kk = 0; kk < CG_T; ++kk) {
-      const float2 a0 = As[tr][kk], a1 = As[tr + 1][kk];
-      const float2 b0 = Bs[kk][tc], b1 = Bs[kk][tc + 1];
-      const float2 av[2] = {a0, a1}, bv[2] = {b0, b1};
+    if (k0 + GI_K < n) load(k0 + GI_K);
 #pragma unroll
-      for (int a = 0; a < 2; ++a)
+    for (int kk = 0; kk < GI_K; ++kk) {
+      float2 a[4], b[4];
 #pragma unroll
-        for (int b = 0; b < 2; ++b) {
-          acc[a][b].x = fmaf(av[a].x, bv[b].x, fmaf(-av[a].y, bv[b].y, acc[a][b].x));
-          acc[a][b].y = fmaf(av[a].x, bv[b].y, fmaf(av[a].y, bv[b].x, acc[a][b].y));
+      for (int q = 0; q < 4; ++q) {
+        a[q] = As[kk][ty + 16 * q];
+        b[q] = Bs[kk][tx + 16 * q];
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {  // conj(a) b
+          acc[u][v].x = fmaf(a[u].x, b[v].x, fmaf(a[u].y, b[v].y, acc[u][v].x));
+          acc[u][v].y = fmaf(a[u].x, b[v].y, fmaf(-a[u].y, b[v].x, acc[u][v].y));
+          mir[u][v] = fmaf(b[v].x, a[u].y, fmaf(-b[v].y, a[u].x, mir[u][v]));  // conj(b) a
         }
     }
     __syncthreads();
   }
 #pragma unroll
-  for (int a = 0; a < 2; ++a)
+  for (int u = 0; u < 4; ++u)
 #pragma unroll
-    for (int b = 0; b < 2; ++b) {
-      const int i = row0 + tr + a, c = col0 + tc + b;
-      if (i < n && c < ld) C[(long long)i * ld + c] = acc[a][b];
+    for (int v = 0; v < 4; ++v) {
+      const int r = ty + 16 * u, c = tx + 16 * v;
+      if (i0 + r < n && j0 + c < n) P[(long long)(i0 + r) * n + j0 + c] = acc[u][v];
+      sm[c * (GI_T + 1) + r] = make_float2(acc[u][v].x, mir[u][v]);
     }
+  if (ti == tj) return;  // a diagonal tile holds both triangles
+  __syncthreads();
+  // the mirror in rows of the transposed tile
+  for (int e = tid; e < GI_T * GI_T; e += 256) {
+    const int c = e >> 6, r = e & 63;
+    if (i0 + r < n && j0 + c < n) P[(long long)(j0 + c) * n + i0 + r] = sm[c * (GI_T + 1) + r];
+  }
 }
 
-// Q^{-1} = W^H W per frequency (dense Hermitian n x n), the operator of the tensor-core solve.
 cudaError_t launch_gram_inverse(const float2* Wh, int n, int nf, float2* Ph, cudaStream_t st) {
-  const dim3 grid((n + CG_T - 1) / CG_T, (n + CG_T - 1) / CG_T, nf);
+  const int nt = (n + GI_T - 1) / GI_T;
   count_launches(1);
-  k_cgemm<true><<<grid, 256, 0, st>>>(Wh, n, Wh, n, Ph, nullptr);
+  k_gram_inverse<<<dim3(nt * (nt + 1) / 2, nf), 256, 0, st>>>(Wh, n, Ph);
   return cudaGetLastError();
 }
 
