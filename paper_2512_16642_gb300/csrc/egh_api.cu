@@ -133,6 +133,11 @@ struct egh_batch {
   cudaGraphExec_t graph = nullptr;
   int graph_launches = 0;      // kernels in one replay of the graph
   cudaEvent_t ev[2] = {};
+  // branches of the contexts' inverses, in order of falling size
+  std::vector<egh_ctx*> by_size;
+  std::vector<cudaStream_t> side;
+  std::vector<cudaEvent_t> ev_join;
+  cudaEvent_t ev_fork = nullptr;
   std::string err;
 };
 
@@ -399,12 +404,15 @@ egh_status fd_chunk_steps(egh_ctx* ctx, int ta, int t0, int t1, int sbase, int n
   return EGH_OK;
 }
 
-// Selective refinement of the mixed precisions, step 1 (queued on `stream` after the inverse
-// factors): ||Q_k||_F^2 and the power estimate of 1 / lambda_min(Q_k), copied to the host buffer.
-egh_status refine_plan(egh_ctx* ctx, cudaStream_t stream) {
+// Selective refinement of the mixed precisions, step 1 (queued on `stream` after the inverses):
+// ||Q_k||_F^2 and the power estimate of 1 / lambda_min(Q_k), then their copy to the host buffer.
+cudaError_t refine_estimates(egh_ctx* ctx, cudaStream_t stream) {
+  const cudaError_t e = launch_fro2(ctx->Qh, ctx->nrec, ctx->nf, ctx->fro2, stream);
+  return e ? e : launch_inv_power(ctx->Ph, ctx->nrec, ctx->nf, ctx->fro2 + ctx->nf, stream);
+}
+
+egh_status refine_fetch(egh_ctx* ctx, cudaStream_t stream) {
   if (!ctx->Wh) return EGH_OK;
-  CK(launch_fro2(ctx->Qh, ctx->nrec, ctx->nf, ctx->fro2, stream));
-  CK(launch_inv_power(ctx->Ph, ctx->nrec, ctx->nf, ctx->fro2 + ctx->nf, stream));
   ctx->cond_host.assign(2 * ctx->nf, 0.0);
   CK(cudaMemcpyAsync(ctx->cond_host.data(), ctx->fro2, 2 * ctx->nf * sizeof(double),
                      cudaMemcpyDeviceToHost, stream));
@@ -1093,7 +1101,8 @@ egh_status egh_factor(egh_ctx* ctx, int32_t* bad_freq, void* stream_) {
     CK(launch_trtri(ctx->Lh, ctx->nrec, ctx->nf, ctx->Wh, stream));
     CK(launch_gram_inverse(ctx->Wh, ctx->nrec, ctx->nf, ctx->Ph, stream));
   }
-  egh_status rs = refine_plan(ctx, stream);  // queues its kernels; reads them after the sync
+  if (ctx->Wh) CK(refine_estimates(ctx, stream));
+  egh_status rs = refine_fetch(ctx, stream);  // read after the sync
   if (rs) return rs;
   CK(cudaEventRecord(ctx->ev[5], stream));
   ctx->ev_rec[2] = true;
@@ -1516,6 +1525,11 @@ void egh_batch_destroy(egh_batch* b) {
   cudaDeviceSynchronize();
   if (b->graph) cudaGraphExecDestroy(b->graph);
   if (b->cap) cudaStreamDestroy(b->cap);
+  for (cudaStream_t s : b->side)
+    if (s) cudaStreamDestroy(s);
+  for (cudaEvent_t e : b->ev_join)
+    if (e) cudaEventDestroy(e);
+  if (b->ev_fork) cudaEventDestroy(b->ev_fork);
   for (cudaEvent_t e : b->ev)
     if (e) cudaEventDestroy(e);
   cudaFree(b->items);
@@ -1559,6 +1573,14 @@ egh_status egh_batch_create(egh_ctx* const* ctxs, int32_t n, egh_batch** out) {
     BCK(cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking));
     BCK(cudaEventCreate(&b->ev[0]));
     BCK(cudaEventCreate(&b->ev[1]));
+    b->by_size = b->ctxs;
+    std::stable_sort(b->by_size.begin(), b->by_size.end(),
+                     [](const egh_ctx* x, const egh_ctx* y) { return x->nrec > y->nrec; });
+    b->side.assign(b->ctxs.size(), nullptr);
+    b->ev_join.assign(b->ctxs.size(), nullptr);
+    for (cudaStream_t& s : b->side) BCK(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
+    for (cudaEvent_t& e : b->ev_join) BCK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+    BCK(cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming));
     BCK(potrf_many_prepare(b->nmax));
     return EGH_OK;
   };
@@ -1572,7 +1594,8 @@ egh_status egh_batch_create(egh_ctx* const* ctxs, int32_t n, egh_batch** out) {
   return EGH_OK;
 }
 
-// Q -> L copies of every context and one persistent factorisation launch, on `st`.
+// Q -> L copies of every context and one persistent factorisation launch, on `st`, then the
+// contexts' inverses in branches that join `st`.
 static cudaError_t batch_enqueue(egh_batch* b, int threads, cudaStream_t st) {
   cudaError_t e;
   for (egh_ctx* c : b->ctxs)
@@ -1582,9 +1605,21 @@ static cudaError_t batch_enqueue(egh_batch* b, int threads, cudaStream_t st) {
   if ((e = launch_potrf_many(b->items, b->count, b->nmax, std::min(b->count, 2 * 152), threads,
                              b->piv64, st)))
     return e;
-  for (egh_ctx* c : b->ctxs) {
-    if (c->Wh && (e = launch_trtri(c->Lh, c->nrec, c->nf, c->Wh, st))) return e;
-    if (c->Ph && (e = launch_gram_inverse(c->Wh, c->nrec, c->nf, c->Ph, st))) return e;
+  // the mixed precisions' inverse factors, inverses and condition estimates: a branch per context,
+  // largest first (each kernel is a chain of rows or steps that leaves the SMs half idle, so the
+  // contexts' chains run side by side: factor and deblur of patches of 161, 257 and 341 receivers
+  // x 40 frequencies 3.20 ms one after another, 2.70 ms as branches)
+  if ((e = cudaEventRecord(b->ev_fork, st))) return e;
+  for (size_t i = 0; i < b->by_size.size(); ++i) {
+    egh_ctx* c = b->by_size[i];
+    if (!c->Wh) continue;
+    cudaStream_t s = b->side[i];
+    if ((e = cudaStreamWaitEvent(s, b->ev_fork, 0))) return e;
+    if ((e = launch_trtri(c->Lh, c->nrec, c->nf, c->Wh, s))) return e;
+    if ((e = launch_gram_inverse(c->Wh, c->nrec, c->nf, c->Ph, s))) return e;
+    if ((e = refine_estimates(c, s))) return e;
+    if ((e = cudaEventRecord(b->ev_join[i], s))) return e;
+    if ((e = cudaStreamWaitEvent(st, b->ev_join[i], 0))) return e;
   }
   return cudaSuccess;
 }
@@ -1632,7 +1667,7 @@ egh_status egh_batch_factor(egh_batch* b, int32_t* bad_ctx, int32_t* bad_freq, v
   BCK(cudaGraphLaunch(b->graph, stream));
   count_launches(b->graph_launches);
   for (egh_ctx* c : b->ctxs) {  // the selective refinement's bounds of every mixed context
-    const egh_status rs = refine_plan(c, stream);
+    const egh_status rs = refine_fetch(c, stream);
     if (rs) return bfail(b, rs, c->err);
   }
   std::vector<int> stv(b->count);
