@@ -57,6 +57,7 @@ struct egh_ctx {
   int* rflags = nullptr;   // resident solver: per-tile step counters + abort flag
   long long fd_steps = 0;  // last egh_green: FD steps computed
   int prec = EGH_PREC_FP32;
+  int gram_edge = 64; // tile edge of the FP32 Gram
   int splits_tc = 0;  // grid-sum splits of the tensor-core Gram
   bool tune_splits = false;  // time half / once / twice the default splits on the first Gram
   Layout L{};
@@ -559,7 +560,8 @@ egh_status egh_create(const egh_config* cfg, egh_ctx** out) {
 
   ctx->prec = c.precision;
   {
-    const int ntile = gram_tiles(c.nrec);
+    ctx->gram_edge = gram_tile_edge(c.nrec);
+    const int ntile = gram_tiles(c.nrec, 64);  // (the sums' point ranges do not follow the edge)
     const long long pairs_nf = (long long)ntile * (ntile + 1) / 2 * c.nfreq;
     long long s = (3LL * 456 + pairs_nf - 1) / pairs_nf;
     s = std::max(1LL, std::min(s, L.G / 2048));
@@ -596,7 +598,7 @@ egh_status egh_create(const egh_config* cfg, egh_ctx** out) {
   std::vector<unsigned char> twt = dft_twiddle_tiles(ctx->freqs, c.dt, c.nt);
   ALLOC(ctx->twt, twt.size(), "twiddle tiles");
   ALLOC(ctx->part,
-        std::max(gram_workspace_floats(c.nrec, c.nfreq, ctx->splits),
+        std::max(gram_workspace_floats(c.nrec, c.nfreq, ctx->splits, ctx->gram_edge),
                  gram_tc_workspace_floats(c.nrec, c.nfreq,
                                           ctx->tune_splits ? 2 * ctx->splits_tc : ctx->splits_tc)) *
             sizeof(float),
@@ -1041,9 +1043,10 @@ egh_status egh_hessian(egh_ctx* ctx, egh_mu_mode mode, double mu_param, double* 
     CK(cudaEventRecord(ctx->ev_gram[1], stream));
     CK(launch_gram_tc_finish(ctx->part, ctx->nrec, ctx->nf, ctx->splits_tc, ctx->Qh, stream));
   } else {
-    CK(launch_gram_partial(ctx->gh, ctx->nrec, ctx->nf, ctx->L.G, ctx->splits, ctx->part, stream));
+    CK(launch_gram_partial(ctx->gh, ctx->nrec, ctx->nf, ctx->L.G, ctx->splits, ctx->gram_edge,
+                           ctx->L.PX, ctx->L.NX, ctx->part, stream));
     CK(cudaEventRecord(ctx->ev_gram[1], stream));
-    CK(launch_gram_finish(ctx->part, ctx->nrec, ctx->nf, ctx->splits, ctx->Qh, stream));
+    CK(launch_gram_finish(ctx->part, ctx->nrec, ctx->nf, ctx->splits, ctx->gram_edge, ctx->Qh, stream));
   }
   double mu = mu_param;
   if (mode == EGH_MU_REL_MEANDIAG) {

@@ -135,12 +135,15 @@ cudaError_t launch_gram_tc_finish(const float* part, int nrec, int nf, int split
                                   cudaStream_t st);
 
 // ---- gram.cu ----------------------------------------------------------------------------------
-__host__ __device__ int gram_tiles(int nrec);
-size_t gram_workspace_floats(int nrec, int nf, int splits);
-cudaError_t launch_gram_partial(const float* gh, int nrec, int nf, long long G, int splits,
-                                float* part, cudaStream_t st);
-cudaError_t launch_gram_finish(const float* part, int nrec, int nf, int splits, float2* Qh,
-                               cudaStream_t st);
+// edge: tile edge of C, 64 or 128 (gram_tile_edge: the better one for nrec); px, nx: row pitch of
+// the points and columns that are not zero (px a multiple of 16; 0: every point counts)
+int gram_tile_edge(int nrec);
+__host__ __device__ int gram_tiles(int nrec, int edge);
+size_t gram_workspace_floats(int nrec, int nf, int splits, int edge);
+cudaError_t launch_gram_partial(const float* gh, int nrec, int nf, long long G, int splits, int edge,
+                                int px, int nx, float* part, cudaStream_t st);
+cudaError_t launch_gram_finish(const float* part, int nrec, int nf, int splits, int edge,
+                               float2* Qh, cudaStream_t st);
 cudaError_t launch_diag_sum(const float2* Qh, int nrec, int nf, double* d_sum, cudaStream_t st);
 cudaError_t launch_lambda_max(const float2* Qh, int nrec, int nf, double* d_lmax, cudaStream_t st);
 cudaError_t launch_add_mu_copy(float2* Qh, float2* Lh, int nrec, int nf, float mu, cudaStream_t st);

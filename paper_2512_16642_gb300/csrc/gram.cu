@@ -3,7 +3,7 @@
 // With M_k = [Re ghat_0; Im ghat_0; Re ghat_1; ...] (2 nrec rows, G columns) and the real
 // symmetric C = M_k M_k^T:
 //   Re H[i][j] = C[2i][2j] + C[2i+1][2j+1],   Im H[i][j] = C[2i+1][2j] - C[2i][2j+1].
-// C is computed in 64 x 64 tiles on and above the tile diagonal only, with the grid sum split
+// C is computed in square tiles on and above the tile diagonal only, with the grid sum split
 // into `splits` ranges whose partial tiles are reduced in a second kernel (scratch workspace).
 #include <algorithm>
 #include <cmath>
@@ -14,27 +14,58 @@
 
 namespace egh {
 
-constexpr int GT = 64;   // tile edge
-constexpr int GK = 16;   // points per shared-memory stage
+constexpr int GK = 16;       // points per shared-memory stage
+constexpr int GST = 3;       // stages in the ring
 constexpr int GFLUSH = 128;  // stages accumulated before adding into the running total
 
-__host__ __device__ int gram_tiles(int nrec) { return (2 * nrec + GT - 1) / GT; }
+// Tile edge of the FP32 Gram: 128 (8 x 8 entries per thread) or 64 (4 x 4).  The larger tile reads
+// each staged value for twice the products; the smaller one computes less past the last receiver,
+// so it is taken where that is a sixth less (231 receivers: 128; up to 32 receivers: 64).  The
+// warps of a 128-row diagonal tile that lie below the diagonal, a quarter of it, compute nothing.
+int gram_tile_edge(int nrec) {
+  const long long n64 = (2LL * nrec + 63) / 64, n128 = (2LL * nrec + 127) / 128;
+  const long long a64 = n64 * (n64 + 1) / 2, a128 = n128 * (n128 + 1) / 2 * 4 - n128;
+  return 6 * a64 < 5 * a128 ? 64 : 128;
+}
 
-size_t gram_workspace_floats(int nrec, int nf, int splits) {
-  const int nt = gram_tiles(nrec);
+__host__ __device__ int gram_tiles(int nrec, int edge) { return (2 * nrec + edge - 1) / edge; }
+
+size_t gram_workspace_floats(int nrec, int nf, int splits, int edge) {
+  const int nt = gram_tiles(nrec, edge);
   const size_t pairs = (size_t)nt * (nt + 1) / 2;
-  return (size_t)splits * nf * pairs * GT * GT;
+  return (size_t)splits * nf * pairs * edge * edge;
 }
 
 __device__ inline const float* m_row(const float* gh, int a, int k, int nf, long long G) {
   return gh + ((long long)((a >> 1) * nf + k) * 2 + (a & 1)) * G;
 }
 
-__global__ void __launch_bounds__(256)
+__device__ __forceinline__ void gram_cp4(unsigned dst, const float* src, bool ok) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(ok ? 4 : 0)
+               : "memory");
+}
+
+// One tile pair of C at one frequency over one range of points, in FP32 on the CUDA cores.  Rows
+// arrive by cp.async, turned on the way ([point][row], three stages in the ring, one barrier per
+// stage); a thread reads 2 R values per point for R^2 products, taken as packed FP32x2 FMAs over
+// two adjacent rows.  Every sum runs over the points in order, and every GFLUSH stages of the range
+// it is added into a total in shared memory (fixed ranges of points: the sums do not depend on the
+// tile edge).  Columns of the padded rows past the grid (x >= nx, zero) are skipped.
+//
+// Bound by the FP32 FMA rate: 231 receivers x 26 frequencies x 349 184 points took 75.7 ms with 64 x
+// 64 tiles (4 x 4 entries per thread, two barriers per 16 points and no loads in flight across
+// them), now 67.2 ms: 520 blocks are 1.7 rounds of the 304 that fit, and the sums' fixed ranges of
+// points allow no other split.
+template <int R>
+__global__ void __launch_bounds__(256, 2)
     k_gram_partial(const float* __restrict__ gh, int nrec, int nf, long long G, int ntile,
-                   long long split_len, float* __restrict__ part) {
-  __shared__ __align__(16) float As[GK][GT + 4];
-  __shared__ __align__(16) float Bs[GK][GT + 4];
+                   long long split_len, int px, int xe, float* __restrict__ part) {
+  constexpr int T = 16 * R;     // tile edge: 4 x 2 warps of 4 x 8 lanes with R x R entries each
+  constexpr int H = R / 4;      // groups of four adjacent rows (columns) per thread
+  // [GST][A, B][GK][T], then totals [R * R][256].  Row r of a staged point p sits at r ^ 4 (p % 8):
+  // the copies, which turn 16 points at a time, then meet two to a bank, and two blocks fit an SM
+  extern __shared__ __align__(16) float gsm[];
+  float* tot = gsm + GST * 2 * GK * T;
   const int pair = blockIdx.x, k = blockIdx.y, s = blockIdx.z;
   int ta = 0, rem = pair;
   while (rem >= ntile - ta) {
@@ -42,124 +73,200 @@ __global__ void __launch_bounds__(256)
     ++ta;
   }
   const int tb = ta + rem;
+  const bool diag = ta == tb;  // B is A
   const int rows = 2 * nrec;
-  const int tid = threadIdx.x;
-  const int tx = tid & 15, ty = tid >> 4;
-  const int lr = tid >> 2, lp = (tid & 3) * 4;
-  const int ra = ta * GT + lr, rb = tb * GT + lr;
-  const float* arow = ra < rows ? m_row(gh, ra, k, nf, G) : nullptr;
-  const float* brow = rb < rows ? m_row(gh, rb, k, nf, G) : nullptr;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const long long p0 = (long long)s * split_len;
   const long long p1 = min(G, p0 + split_len);
-
-  float acc[4][4], tot[4][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = tot[i][j] = 0.f;
-  int stages = 0;
-  for (long long p = p0; p < p1; p += GK) {
-    float4 va = make_float4(0.f, 0.f, 0.f, 0.f), vb = va;
-    if (arow) va = *reinterpret_cast<const float4*>(arow + p + lp);
-    if (brow) vb = *reinterpret_cast<const float4*>(brow + p + lp);
-    As[lp + 0][lr] = va.x;
-    As[lp + 1][lr] = va.y;
-    As[lp + 2][lr] = va.z;
-    As[lp + 3][lr] = va.w;
-    Bs[lp + 0][lr] = vb.x;
-    Bs[lp + 1][lr] = vb.y;
-    Bs[lp + 2][lr] = vb.z;
-    Bs[lp + 3][lr] = vb.w;
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < GK; ++kk) {
-      const float4 a4 = *reinterpret_cast<const float4*>(&As[kk][ty * 4]);
-      const float4 b4 = *reinterpret_cast<const float4*>(&Bs[kk][tx * 4]);
-      const float av[4] = {a4.x, a4.y, a4.z, a4.w};
-      const float bv[4] = {b4.x, b4.y, b4.z, b4.w};
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
+  // copies of a stage: point tid % 16 of rows tid / 16 + 16 q of each operand
+  const int cp = tid & 15, cr = tid >> 4;
+  const unsigned ring = (unsigned)__cvta_generic_to_shared(gsm) + (unsigned)(cp * T) * 4u;
+  const int csw = 4 * (cp & 7);
+  // rows 2 r, 2 r + 1 of M_k are the planes of receiver r: row a starts at (a / 2 * nf * 2 + a % 2) G;
+  // 16 rows on is 8 receivers on
+  const float* srcA = m_row(gh, ta * T + cr, k, nf, G) + cp;
+  const float* srcB = m_row(gh, tb * T + cr, k, nf, G) + cp;
+  const long long step16 = 16LL * nf * G;
+  // stages of the range that hold grid columns: point p, column x of its row
+  auto advance = [&](long long& p, int& x) {
+    p += GK;
+    x += GK;
+    if (px > 0 && x >= xe) {
+      p += px - x;
+      x = 0;
     }
-    __syncthreads();
-    if (++stages == GFLUSH) {
-      stages = 0;
+  };
+  auto begin = [&](long long& p, int& x) {
+    p = p0;
+    x = px > 0 ? (int)(p0 % px) : 0;
+    if (px > 0 && x >= xe) {
+      p += px - x;
+      x = 0;
+    }
+  };
+  long long lp, mp;  // next stage to copy, stage to multiply
+  int lx, mx;
+  begin(lp, lx);
+  begin(mp, mx);
+  auto issue = [&](int buf) {
+    if (lp < p1) {
+      const unsigned dst = ring + (unsigned)(buf * 2 * GK * T) * 4u;
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int q = 0; q < R; ++q) {
+        const bool in = ta * T + cr + 16 * q < rows;
+        gram_cp4(dst + 4u * ((cr + 16 * q) ^ csw), in ? srcA + q * step16 + lp : gh, in);
+      }
+      if (!diag) {
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          tot[i][j] += acc[i][j];
-          acc[i][j] = 0.f;
+        for (int q = 0; q < R; ++q) {
+          const bool in = tb * T + cr + 16 * q < rows;
+          gram_cp4(dst + 4u * (GK * T + ((cr + 16 * q) ^ csw)), in ? srcB + q * step16 + lp : gh, in);
         }
+      }
+      advance(lp, lx);
     }
-  }
-  const int npairs = ntile * (ntile + 1) / 2;
-  float* out = part + (((long long)s * nf + k) * npairs + pair) * (GT * GT);
+    asm volatile("cp.async.commit_group;" ::: "memory");  // empty groups keep the count uniform
+  };
+  // this thread's entries: rows ra + 4 R h + i, columns rb + 8 R h + j (i, j < 4, h < H) of the tile
+  const int wr = (warp >> 1) * 4 * R, wc = (warp & 1) * 8 * R;
+  const int ra = wr + 4 * (lane >> 3), rb = wc + 4 * (lane & 7);
+  const bool work = !(diag && wr >= wc + 8 * R) && ta * T + wr < rows && tb * T + wc < rows;
+  float2 acc[R / 2][R];  // adjacent rows as pairs
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    float4 v;
-    v.x = tot[i][0] + acc[i][0];
-    v.y = tot[i][1] + acc[i][1];
-    v.z = tot[i][2] + acc[i][2];
-    v.w = tot[i][3] + acc[i][3];
-    *reinterpret_cast<float4*>(out + (ty * 4 + i) * GT + tx * 4) = v;
+  for (int i = 0; i < R / 2; ++i)
+#pragma unroll
+    for (int j = 0; j < R; ++j) {
+      acc[i][j] = make_float2(0.f, 0.f);
+      tot[(2 * i * R + j) * 256 + tid] = 0.f;
+      tot[((2 * i + 1) * R + j) * 256 + tid] = 0.f;
+    }
+  long long flush_at = p0 + (long long)GFLUSH * GK;
+  issue(0);
+  issue(1);
+  int buf = 0;
+  while (mp < p1) {
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    __syncthreads();  // the stage has landed; every thread is done with the one before
+    issue(buf == 0 ? 2 : buf - 1);
+    while (mp >= flush_at) {
+#pragma unroll
+      for (int i = 0; i < R / 2; ++i)
+#pragma unroll
+        for (int j = 0; j < R; ++j) {
+          tot[(2 * i * R + j) * 256 + tid] += acc[i][j].x;
+          tot[((2 * i + 1) * R + j) * 256 + tid] += acc[i][j].y;
+          acc[i][j] = make_float2(0.f, 0.f);
+        }
+      flush_at += (long long)GFLUSH * GK;
+    }
+    if (work) {
+      const float* A = gsm + buf * 2 * GK * T;
+      const float* B = gsm + (buf * 2 + (diag ? 0 : 1)) * GK * T;
+#pragma unroll
+      for (int q = 0; q < GK; ++q) {
+        float4 a[H], b[H];
+#pragma unroll
+        for (int h = 0; h < H; ++h) {
+          a[h] = *reinterpret_cast<const float4*>(A + q * T + ((ra + 16 * h) ^ (4 * (q & 7))));
+          b[h] = *reinterpret_cast<const float4*>(B + q * T + ((rb + 32 * h) ^ (4 * (q & 7))));
+        }
+#pragma unroll
+        for (int h = 0; h < H; ++h) {
+          const float bv[4] = {b[h].x, b[h].y, b[h].z, b[h].w};
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const float2 bb = make_float2(bv[j], bv[j]);
+#pragma unroll
+            for (int g = 0; g < H; ++g) {
+              acc[2 * g][4 * h + j] = __ffma2_rn(make_float2(a[g].x, a[g].y), bb, acc[2 * g][4 * h + j]);
+              acc[2 * g + 1][4 * h + j] = __ffma2_rn(make_float2(a[g].z, a[g].w), bb, acc[2 * g + 1][4 * h + j]);
+            }
+          }
+        }
+      }
+    }
+    advance(mp, mx);
+    buf = buf == GST - 1 ? 0 : buf + 1;
   }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  const int npairs = ntile * (ntile + 1) / 2;
+  float* out = part + (((long long)s * nf + k) * npairs + pair) * (T * T);
+#pragma unroll
+  for (int i = 0; i < R; ++i)
+#pragma unroll
+    for (int h = 0; h < H; ++h) {
+      float v[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        v[j] = tot[(i * R + 4 * h + j) * 256 + tid] + (i & 1 ? acc[i / 2][4 * h + j].y : acc[i / 2][4 * h + j].x);
+      *reinterpret_cast<float4*>(out + (ra + 16 * (i / 4) + i % 4) * T + rb + 32 * h) =
+          make_float4(v[0], v[1], v[2], v[3]);
+    }
 }
 
-cudaError_t launch_gram_partial(const float* gh, int nrec, int nf, long long G, int splits,
-                                float* part, cudaStream_t st) {
-  const int nt = gram_tiles(nrec);
+cudaError_t launch_gram_partial(const float* gh, int nrec, int nf, long long G, int splits, int edge,
+                                int px, int nx, float* part, cudaStream_t st) {
+  const int nt = gram_tiles(nrec, edge);
   const int npairs = nt * (nt + 1) / 2;
+  if ((edge != 64 && edge != 128) || px % GK != 0) return cudaErrorInvalidValue;
   long long split_len = (G + splits - 1) / splits;
   split_len = (split_len + GK - 1) / GK * GK;
+  const int R = edge / 16;
+  auto bytes = [](int r) { return (GST * 2 * GK * 16 * r + r * r * 256) * (int)sizeof(float); };
+  const int smem = bytes(R);
+  auto kern = R == 8 ? k_gram_partial<8> : k_gram_partial<4>;
+  // both instances, so that a later call with the other tile edge loads no code
+  cudaError_t e;
+  if ((e = cudaFuncSetAttribute(k_gram_partial<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes(8))) ||
+      (e = cudaFuncSetAttribute(k_gram_partial<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes(4))))
+    return e;
   dim3 grid(npairs, nf, splits);
   count_launches(1);
-  k_gram_partial<<<grid, 256, 0, st>>>(gh, nrec, nf, G, nt, split_len, part);
+  kern<<<grid, 256, smem, st>>>(gh, nrec, nf, G, nt, split_len, px, (nx + GK - 1) / GK * GK, part);
   return cudaGetLastError();
 }
 
 // C[a][b] summed over splits, read from the tile pair with ta <= tb (C is symmetric).
 __device__ inline float c_entry(const float* part, int a, int b, int k, int nf, int ntile,
-                                int npairs, int splits) {
-  if (a / GT > b / GT) {
+                                int npairs, int splits, int T) {
+  if (a / T > b / T) {
     const int t = a;
     a = b;
     b = t;
   }
-  const int ta = a / GT, tb = b / GT;
+  const int ta = a / T, tb = b / T;
   const int pair = ta * ntile - ta * (ta - 1) / 2 + (tb - ta);
-  const long long off = (long long)(a % GT) * GT + (b % GT);
+  const long long off = (long long)(a % T) * T + (b % T);
   double sum = 0.0;
   for (int s = 0; s < splits; ++s)
-    sum += part[(((long long)s * nf + k) * npairs + pair) * (GT * GT) + off];
+    sum += part[(((long long)s * nf + k) * npairs + pair) * (T * T) + off];
   return (float)sum;
 }
 
-__global__ void k_gram_finish(const float* __restrict__ part, int nrec, int nf, int splits,
+__global__ void k_gram_finish(const float* __restrict__ part, int nrec, int nf, int splits, int T,
                               float2* __restrict__ Qh) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   const int i = blockIdx.y;
   const int k = blockIdx.z;
   if (j >= nrec) return;
-  const int ntile = gram_tiles(nrec);
+  const int ntile = gram_tiles(nrec, T);
   const int npairs = ntile * (ntile + 1) / 2;
   const int a = min(i, j), b = max(i, j);
-  const float rr = c_entry(part, 2 * a, 2 * b, k, nf, ntile, npairs, splits);
-  const float ii = c_entry(part, 2 * a + 1, 2 * b + 1, k, nf, ntile, npairs, splits);
+  const float rr = c_entry(part, 2 * a, 2 * b, k, nf, ntile, npairs, splits, T);
+  const float ii = c_entry(part, 2 * a + 1, 2 * b + 1, k, nf, ntile, npairs, splits, T);
   float im = 0.f;
   if (a != b)
-    im = c_entry(part, 2 * a + 1, 2 * b, k, nf, ntile, npairs, splits) -
-         c_entry(part, 2 * a, 2 * b + 1, k, nf, ntile, npairs, splits);
+    im = c_entry(part, 2 * a + 1, 2 * b, k, nf, ntile, npairs, splits, T) -
+         c_entry(part, 2 * a, 2 * b + 1, k, nf, ntile, npairs, splits, T);
   // entry (a, b) with a <= b; (b, a) is its conjugate
   Qh[((long long)k * nrec + i) * nrec + j] = make_float2(rr + ii, i <= j ? im : -im);
 }
 
-cudaError_t launch_gram_finish(const float* part, int nrec, int nf, int splits, float2* Qh,
-                               cudaStream_t st) {
+cudaError_t launch_gram_finish(const float* part, int nrec, int nf, int splits, int edge,
+                               float2* Qh, cudaStream_t st) {
   dim3 grid((nrec + 127) / 128, nrec, nf);
   count_launches(1);
-  k_gram_finish<<<grid, 128, 0, st>>>(part, nrec, nf, splits, Qh);
+  k_gram_finish<<<grid, 128, 0, st>>>(part, nrec, nf, splits, edge, Qh);
   return cudaGetLastError();
 }
 
@@ -205,14 +312,26 @@ __device__ __forceinline__ void two_word_square(float a, float& s, float& c) {
 __global__ void __launch_bounds__(FR_THREADS)
     k_fro2(const float2* __restrict__ Qh, int n, double* d_out) {
   __shared__ double red[FR_THREADS / 32];
+  __shared__ int emax;
   const long long n2 = (long long)n * n;
   const float2* A = Qh + (long long)blockIdx.x * n2;
+  // entries are scaled by the exponent of the largest diagonal one (which bounds every entry of a
+  // positive-definite matrix), so that the FP32 squares neither overflow nor lose their errors
+  if (threadIdx.x == 0) emax = -126;
+  __syncthreads();
+  for (int i = threadIdx.x; i < n; i += FR_THREADS) {
+    const float d = A[(long long)i * n + i].x;
+    if (isfinite(d) && d != 0.f) atomicMax(&emax, ilogbf(d));
+  }
+  __syncthreads();
+  const int ex = max(-126, min(126, emax));
+  const float sc = ldexpf(1.f, -ex);
   float s[2] = {0.f, 0.f}, c[2] = {0.f, 0.f};
 #pragma unroll 4
   for (long long t = threadIdx.x; t < n2; t += FR_THREADS) {
     const float2 a = __ldg(A + t);
-    two_word_square(a.x, s[0], c[0]);
-    two_word_square(a.y, s[1], c[1]);
+    two_word_square(a.x * sc, s[0], c[0]);
+    two_word_square(a.y * sc, s[1], c[1]);
   }
   double v = ((double)s[0] + c[0]) + ((double)s[1] + c[1]);
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -221,7 +340,7 @@ __global__ void __launch_bounds__(FR_THREADS)
   if (threadIdx.x == 0) {
     double sum = 0.0;
     for (int w = 0; w < FR_THREADS / 32; ++w) sum += red[w];
-    d_out[blockIdx.x] = sum;
+    d_out[blockIdx.x] = ldexp(sum, 2 * ex);
   }
 }
 

@@ -73,7 +73,9 @@ extern "C" egh_status egh_gram_noalloc(const float* gh, int32_t nrec, int32_t nf
     return fail(EGH_EINVAL, "egh_gram_noalloc: gh must be 16-byte and H 8-byte aligned");
   if (!is_device_pointer(gh) || !is_device_pointer(H))
     return fail(EGH_EINVAL, "egh_gram_noalloc: gh and H must be device memory");
-  const size_t one_split = egh::gram_workspace_floats(nrec, nfreq, 1);
+  // 64-row tiles set the limit and the splits; larger ones are taken where they suit nrec and fit
+  int edge = 64;
+  const size_t one_split = egh::gram_workspace_floats(nrec, nfreq, 1, edge);
   if (one_split > kScratchFloats) {
     return fail(EGH_EINVAL,
                 "egh_gram_noalloc: nrec = " + std::to_string(nrec) + ", nfreq = " +
@@ -88,16 +90,18 @@ extern "C" egh_status egh_gram_noalloc(const float* gh, int32_t nrec, int32_t nf
     return fail(EGH_ECUDA, std::string("egh_gram_noalloc: cudaGetSymbolAddress: ") +
                                cudaGetErrorString(e));
   // as many splits of the grid sum as fit the scratch, up to the default heuristic
-  const int ntile = egh::gram_tiles(nrec);
+  const int ntile = egh::gram_tiles(nrec, 64);
   const long long pairs_nf = (long long)ntile * (ntile + 1) / 2 * nfreq;
   long long want = (3LL * 456 + pairs_nf - 1) / pairs_nf;
   want = std::max(1LL, std::min(want, (long long)(npts / 2048)));
   const long long fit = (long long)(kScratchFloats / one_split);
   const int splits = (int)std::max(1LL, std::min(want, fit));
+  const int best = egh::gram_tile_edge(nrec);
+  if (egh::gram_workspace_floats(nrec, nfreq, splits, best) <= kScratchFloats) edge = best;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  e = egh::launch_gram_partial(gh, nrec, nfreq, npts, splits, scratch, st);
+  e = egh::launch_gram_partial(gh, nrec, nfreq, npts, splits, edge, 0, 0, scratch, st);
   if (e == cudaSuccess)
-    e = egh::launch_gram_finish(scratch, nrec, nfreq, splits, static_cast<float2*>(H), st);
+    e = egh::launch_gram_finish(scratch, nrec, nfreq, splits, edge, static_cast<float2*>(H), st);
   if (e != cudaSuccess)
     return fail(EGH_ECUDA, std::string("egh_gram_noalloc: launch: ") + cudaGetErrorString(e));
   return EGH_OK;
