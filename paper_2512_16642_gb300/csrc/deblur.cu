@@ -56,18 +56,19 @@ cudaError_t launch_trace_dft_tc(const float* resid, int ntr, int nt_d, const uns
 
 cudaError_t launch_trace_tma(const float* resid, int ntr, int nt_d, const unsigned char* twt,
                              int nf, int nrec, int ld, int s0, float2* Dh, int* err, int expire,
-                             cudaStream_t st);
+                             cudaStream_t st, void* scratch, size_t scratch_bytes);
 cudaError_t make_f32_tmap(CUtensorMap* tm, const void* base, long long rows, long long cols,
                           int box_cols, int box_rows, bool swizzle);
 
 cudaError_t launch_trace_dft(const float* resid, int ntr, int nt_d, int nf, int nrec, int ld,
                              int s0, float2* Dh, cudaStream_t st, const unsigned char* twt,
-                             int* err, int expire, bool dev_in) {
+                             int* err, int expire, bool dev_in, void* scratch, size_t scratch_bytes) {
   // N = 2 nf rounded up to 32 is at most 128 for nf <= 64
   if (nf < 1 || nf > NFMAX || !twt || !err) return cudaErrorInvalidValue;
   const bool vec = (nt_d & 3) == 0 && (reinterpret_cast<uintptr_t>(resid) & 15) == 0;
-  if (dev_in && vec && tt_ncomp(nf) <= 64 && ntr > 0)
-    return launch_trace_tma(resid, ntr, nt_d, twt, nf, nrec, ld, s0, Dh, err, expire, st);
+  if (dev_in && vec && tt_ncomp(nf) <= 96 && ntr > 0)  // (TP_NMAX)
+    return launch_trace_tma(resid, ntr, nt_d, twt, nf, nrec, ld, s0, Dh, err, expire, st, scratch,
+                            scratch_bytes);
   return launch_trace_dft_tc(resid, ntr, nt_d, twt, nf, nrec, ld, s0, Dh, err, expire, st);
 }
 
@@ -328,12 +329,21 @@ __global__ void __cluster_dims__(TD_S, 1, 1) __launch_bounds__(256)
 // and the parts depend on the trace length alone: a trace's spectrum does not depend on the
 // other traces of the call.  mbarriers carry every hand-off; every wait is bounded and gives up
 // early once another role has failed.
+//
+// A call with few trace tiles leaves most SMs idle with two parts (one source of 231 receivers: 4
+// units of 31 stages, 34 us, the time of 40 sources).  Given scratch memory, such a call takes a
+// TMEM block (TT_J stages of a part) as its unit: the blocks' sums go to the scratch and the last
+// unit of the tile to arrive adds them in the order in which one unit per part adds them, so the
+// spectra have the same bits in both forms.  Used where two parts leave half of the SMs without a
+// unit (34 us for that source before, 24 us now).
 // ---------------------------------------------------------------------------------------------
 constexpr int TP_EPI = 256;  // threads of warps 0-7
 constexpr int TP_A = 2;  // A tiles in TMEM (the converters fill one while the MMAs read another)
 constexpr int TP_B = 4;  // twiddle tiles in flight (loaded TP_B - 2 stages ahead)
 // fp32 ring stages: what shared memory holds beside the twiddle tiles
-__host__ __device__ constexpr int tp_ring(int N) { return N <= 32 ? 6 : 5; }
+__host__ __device__ constexpr int tp_ring(int N) { return N <= 32 ? 6 : N <= 64 ? 5 : 4; }
+// Tensor memory holds two block buffers of 2N columns and the A tiles up to N = 96
+constexpr int TP_NMAX = 96;
 // The MMA thread waits for the MMAs of stage g - 2 before reusing a twiddle tile; that phase is
 // still the latest one of its mbarrier (mdone of A tile (g - 2) % TP_A) only with two or more A
 // tiles: with one, stage g - 1's MMAs may already have completed the next phase.
@@ -345,27 +355,50 @@ size_t trace_tma_smem(int N) {
   return 1024 + (size_t)tp_ring(N) * TP_STAGE + TP_B * 2 * (size_t)N * 128;
 }
 
-// the stages of unit u (part u % H of tile u / H)
+// TMEM blocks of a part of nr stages, and of a tile's H parts
+__host__ __device__ inline int tp_blocks(int nr) { return (nr + TT_J - 1) / TT_J; }
+__host__ __device__ inline int tp_tile_blocks(int H, int nst) {
+  int b = 0;
+  for (int h = 0; h < H; ++h) b += tp_blocks((h + 1) * nst / H - h * nst / H);
+  return b;
+}
+
+// the stages of unit u: part u % H of tile u / H, or with BPT > 0 blocks per tile, block u % BPT of
+// tile u / BPT (counted over the tile's parts)
 struct TpUnit {
   int tile, sb, nr;
 };
-__device__ __forceinline__ TpUnit tp_unit(long long u, int H, int nst) {
-  const int half = (int)(u % H);
+__device__ __forceinline__ TpUnit tp_unit(long long u, int H, int nst, int BPT) {
   TpUnit r;
+  if (BPT > 0) {
+    r.tile = (int)(u / BPT);
+    int b = (int)(u % BPT), h = 0, nr = nst / H;
+    while (b >= tp_blocks(nr)) {
+      b -= tp_blocks(nr);
+      ++h;
+      nr = (h + 1) * nst / H - h * nst / H;
+    }
+    r.sb = h * nst / H + b * TT_J;
+    r.nr = min(TT_J, nr - b * TT_J);
+    return r;
+  }
+  const int half = (int)(u % H);
   r.tile = (int)(u / H);
   r.sb = half * nst / H;
   r.nr = (half + 1) * nst / H - r.sb;
   return r;
 }
 
-template <int N>
+template <int N, bool BLOCKS>
 __global__ void __launch_bounds__(TP_EPI + 64, 1)
     k_trace_tma(const __grid_constant__ CUtensorMap tm_in, int ntr, int nt_d,
                 const unsigned char* __restrict__ twt, int nf, int nrec, int ld, int s0, int H,
-                float2* __restrict__ Dh, int* __restrict__ err, int expire) {
+                int bpt, float2* __restrict__ Dh, float* __restrict__ part,
+                unsigned* __restrict__ arrived, int* __restrict__ err, int expire) {
   constexpr int R = tp_ring(N);
   constexpr unsigned BT = 2u * N * 128u;  // one twiddle tile (hi + lo)
   constexpr int NH = N / 2;
+  const int BPT = BLOCKS ? bpt : 0;  // (an instance of its own: the second form's sums cost registers)
   extern __shared__ __align__(1024) unsigned char tp_dsm[];
   unsigned char* sm = tp_dsm + ((1024 - (tc::smem_u32(tp_dsm) & 1023)) & 1023);
   constexpr int NB = TP_B, NA = TP_A;
@@ -376,7 +409,7 @@ __global__ void __launch_bounds__(TP_EPI + 64, 1)
   volatile int* fail = &fail_s;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int ntile = (ntr + TT_M - 1) / TT_M, nst = (nt_d + TT_K - 1) / TT_K;
-  const long long U = (long long)ntile * H;
+  const long long U = (long long)ntile * (BPT > 0 ? BPT : H);
   const long long u0 = U * blockIdx.x / gridDim.x;
   const int n = (int)(U * (blockIdx.x + 1) / gridDim.x - u0);  // units of this CTA
   const unsigned bar0 = tc::smem_u32(&bars[0]);
@@ -392,6 +425,7 @@ __global__ void __launch_bounds__(TP_EPI + 64, 1)
   // TMEM: two block buffers of 2N columns ([0, N) hi.hi + lo.hi, [N, 2N) hi.lo), then the A tiles
   // at column ACOL: per tile 32 columns of hi (64 samples, two bf16 each) and 32 of lo
   constexpr unsigned ACOL = 4 * N, TCOLS = 4 * N + 64 * TP_A <= 256 ? 256 : 512;
+  static_assert(4 * N + 64 * TP_A <= 512, "block buffers and A tiles in tensor memory");
   if (warp == 0) tc::tmem_alloc(&tslot, TCOLS);
   if (tid == 0) {
     for (int i = 0; i < R; ++i) {
@@ -425,19 +459,19 @@ __global__ void __launch_bounds__(TP_EPI + 64, 1)
   auto cur_init = [&](Cur& c) {
     c.i = 0;
     c.s = 0;
-    c.t = tp_unit(u0, H, nst);
+    c.t = tp_unit(u0, H, nst, BPT);
   };
   auto cur_next = [&](Cur& c) {
     if (++c.s == c.t.nr) {
       c.s = 0;
-      if (++c.i < n) c.t = tp_unit(u0 + c.i, H, nst);
+      if (++c.i < n) c.t = tp_unit(u0 + c.i, H, nst, BPT);
     }
   };
   bool ok = true;
   if (warp == 8) {
     if (lane == 0 && n > 0) {
       int G = 0;  // stages of this CTA
-      for (int i = 0; i < n; ++i) G += tp_unit(u0 + i, H, nst).nr;
+      for (int i = 0; i < n; ++i) G += tp_unit(u0 + i, H, nst, BPT).nr;
       Cur mc, bc;  // next MMA stage, next twiddle load
       cur_init(mc);
       cur_init(bc);
@@ -508,7 +542,7 @@ __global__ void __launch_bounds__(TP_EPI + 64, 1)
     // the ring: a slot is loaded again as soon as the converters have read it
     if (lane == 0 && n > 0) {
       int G = 0;
-      for (int i = 0; i < n; ++i) G += tp_unit(u0 + i, H, nst).nr;
+      for (int i = 0; i < n; ++i) G += tp_unit(u0 + i, H, nst, BPT).nr;
       Cur lc;
       cur_init(lc);
       int issued_r = 0;
@@ -591,9 +625,43 @@ __global__ void __launch_bounds__(TP_EPI + 64, 1)
       tc::mbar_arrive(tempty(b & 1));
       return true;
     };
-    auto emit = [&](int tile) {  // a unit's totals into the spectra: components 2 kk, 2 kk + 1
+    auto emit = [&](int tile, long long u) {  // a unit's totals into the spectra: 2 kk, 2 kk + 1
       const int q = tile * TT_M + row;
-      if (q < ntr) {
+      bool store = q < ntr;
+      if (BLOCKS) {
+        // the block's sums as [unit][component][row].  A warp's slice (32 rows, half of the
+        // components) is completed by that warp of the unit whose slice arrives last; nothing here
+        // waits for another warp
+#pragma unroll
+        for (int c = 0; c < NH; ++c) part[(u * N + hh * NH + c) * TT_M + row] = tot[c];
+        __threadfence();
+        __syncwarp();
+        unsigned before = 0;
+        if (lane == 0) before = atomicAdd(arrived + tile * (TP_EPI / 32) + warp, 1u);
+        const bool last = __shfl_sync(0xffffffffu, before, 0) == (unsigned)(BPT - 1);
+        store = store && last;
+        if (last) {
+          __threadfence();
+          // as the other form: each part's blocks in order from zero, then the parts
+          const float* pb = part + ((long long)tile * BPT * N + hh * NH) * TT_M + row;
+          float sum[NH];
+#pragma unroll
+          for (int c = 0; c < NH; ++c) sum[c] = 0.f;
+          for (int h = 0; h < H; ++h) {
+            const int nb = tp_blocks((h + 1) * nst / H - h * nst / H);
+#pragma unroll
+            for (int c = 0; c < NH; ++c) tot[c] = 0.f;
+            for (int b = 0; b < nb; ++b, pb += (long long)N * TT_M)
+#pragma unroll
+              for (int c = 0; c < NH; ++c) tot[c] += __ldcg(pb + c * TT_M);
+#pragma unroll
+            for (int c = 0; c < NH; ++c) sum[c] += tot[c];
+          }
+#pragma unroll
+          for (int c = 0; c < NH; ++c) tot[c] = sum[c];
+        }
+      }
+      if (store) {
         const int sidx = q / nrec, r = q % nrec;
 #pragma unroll
         for (int p = 0; p < NH / 2; ++p) {
@@ -601,7 +669,7 @@ __global__ void __launch_bounds__(TP_EPI + 64, 1)
           if (kk < nf) {
             float2* d = Dh + ((long long)kk * nrec + r) * ld + s0 + sidx;
             const float2 x = make_float2(tot[2 * p], tot[2 * p + 1]);
-            if (H == 1)
+            if (BLOCKS || H == 1)
               *d = x;
             else
               atomicAdd(d, x);
@@ -612,8 +680,9 @@ __global__ void __launch_bounds__(TP_EPI + 64, 1)
       for (int c = 0; c < NH; ++c) tot[c] = 0.f;
     };
     int g = 0, blk = 0, pend = -1, pend_tile = -1;
+    long long pend_unit = -1;
     for (int i = 0; i < n && ok; ++i) {
-      const TpUnit t = tp_unit(u0 + i, H, nst);
+      const TpUnit t = tp_unit(u0 + i, H, nst, BPT);
       for (int s = 0; s < t.nr; ++s) {
         if (!convert(g)) {
           ok = false;
@@ -626,18 +695,19 @@ __global__ void __launch_bounds__(TP_EPI + 64, 1)
             ok = false;
             break;
           }
-          if (pend_tile >= 0) emit(pend_tile);
+          if (pend_tile >= 0) emit(pend_tile, pend_unit);
           pend = -1;
         }
         if ((s + 1) % TT_J == 0 || s == t.nr - 1) {
           pend = blk++;
           pend_tile = s == t.nr - 1 ? t.tile : -1;
+          pend_unit = u0 + i;
         }
       }
     }
     if (ok && pend >= 0) {
       ok = drain(pend);
-      if (ok && pend_tile >= 0) emit(pend_tile);
+      if (ok && pend_tile >= 0) emit(pend_tile, pend_unit);
     }
     if (!ok) *fail = 1;
   }
@@ -675,31 +745,56 @@ cudaError_t launch_trace_dft_tc(const float* resid, int ntr, int nt_d, const uns
   return cudaErrorInvalidValue;
 }
 
+size_t trace_scratch_bytes(int nf, long long ntr, int nt_d) {
+  const int N = tt_ncomp(nf), nst = (nt_d + TT_K - 1) / TT_K;
+  const long long ntile = (ntr + TT_M - 1) / TT_M;
+  const int H = nst >= 2 ? 2 : 1;
+  int dev = 0, sms = 0;
+  if (N > TP_NMAX || (nt_d & 3) || cudaGetDevice(&dev) ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev))
+    return 0;
+  const int bpt = tp_tile_blocks(H, nst);
+  if (bpt <= H || 2 * ntile * H > sms) return 0;
+  return (size_t)ntile * bpt * N * TT_M * sizeof(float) + (size_t)ntile * (TP_EPI / 32) * sizeof(unsigned);
+}
+
 // Persistent transform: one CTA per SM, at most one per unit.  With two parts per tile the
 // spectra of the call's columns are zeroed first (the parts add into them).
 cudaError_t launch_trace_tma(const float* resid, int ntr, int nt_d, const unsigned char* twt,
                              int nf, int nrec, int ld, int s0, float2* Dh, int* err, int expire,
-                             cudaStream_t st) {
+                             cudaStream_t st, void* scratch, size_t scratch_bytes) {
   const int N = tt_ncomp(nf);
   const size_t smem = trace_tma_smem(N);
-  auto kern = N == 32 ? k_trace_tma<32> : k_trace_tma<64>;
   cudaError_t e;
   int dev = 0, sms = 0;
   if ((e = cudaGetDevice(&dev)) || (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)))
     return e;
-  if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)))
-    return e;
   const int ntile = (ntr + TT_M - 1) / TT_M, nst = (nt_d + TT_K - 1) / TT_K;
   const int H = nst >= 2 ? 2 : 1;
-  if (H == 2 &&
-      (e = cudaMemset2DAsync(Dh + s0, (size_t)ld * sizeof(float2), 0,
-                             (size_t)(ntr / nrec) * sizeof(float2), (size_t)nf * nrec, st)))
+  int bpt = 0;
+  float* part = nullptr;
+  unsigned* arrived = nullptr;
+  const size_t need = scratch ? trace_scratch_bytes(nf, ntr, nt_d) : 0;
+  if (need && need <= scratch_bytes) {
+    bpt = tp_tile_blocks(H, nst);
+    part = static_cast<float*>(scratch);
+    arrived = reinterpret_cast<unsigned*>(part + (size_t)ntile * bpt * N * TT_M);
+    if ((e = cudaMemsetAsync(arrived, 0, (size_t)ntile * (TP_EPI / 32) * sizeof(unsigned), st))) return e;
+  } else if (H == 2 &&
+             (e = cudaMemset2DAsync(Dh + s0, (size_t)ld * sizeof(float2), 0,
+                                    (size_t)(ntr / nrec) * sizeof(float2), (size_t)nf * nrec, st))) {
+    return e;
+  }
+  auto kern = bpt ? (N == 32 ? k_trace_tma<32, true> : N == 64 ? k_trace_tma<64, true> : k_trace_tma<96, true>)
+                  : (N == 32 ? k_trace_tma<32, false> : N == 64 ? k_trace_tma<64, false> : k_trace_tma<96, false>);
+  if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)))
     return e;
   CUtensorMap tm;
   if ((e = make_f32_tmap(&tm, resid, ntr, nt_d, 32, TT_M, true))) return e;
-  const int grid = (int)std::min<long long>((long long)ntile * H, sms);
+  const int grid = (int)std::min<long long>((long long)ntile * (bpt ? bpt : H), sms);
   count_launches(1);
-  kern<<<grid, TP_EPI + 64, smem, st>>>(tm, ntr, nt_d, twt, nf, nrec, ld, s0, H, Dh, err, expire);
+  kern<<<grid, TP_EPI + 64, smem, st>>>(tm, ntr, nt_d, twt, nf, nrec, ld, s0, H, bpt, Dh, part, arrived,
+                                        err, expire);
   return cudaGetLastError();
 }
 
@@ -1228,95 +1323,148 @@ __global__ void __launch_bounds__(32 * TS_W)
 // with Knuth's TwoSum, whose rounding errors are gathered with the e in a second FP32 word, so
 // the result is as accurate as if summed in twice the working precision (about 2^-48 relative to
 // sum |q x|) and then rounded.  The GB300 issues FP64 at a small fraction of the FP32 rate, so this
-// is the fast route to a residual whose FP32 rounding matches the FP64 one.  Every step uses the
-// _rn intrinsics so that no product is contracted into an FMA.  Layout as k_resid64; each warp
-// takes two rows per pass so that each solution read serves both.
+// is the fast route to a residual whose FP32 rounding matches the FP64 one.  Every step uses
+// explicitly rounded operations so that no product is contracted into an FMA.
+//
+// (A sum kept on a fixed grid by its first word needs 4 operations per product instead of 10 but
+// loses the low bits of the second word: 2^-40 against 2^-50 of |q||x|, simulated; not used.)
 // ---------------------------------------------------------------------------------------------
-__device__ __forceinline__ void dot2_add(float& s, float& c, float a, float b) {
-  const float p = __fmul_rn(a, b);
-  const float e = __fmaf_rn(a, b, -p);
-  const float t = __fadd_rn(s, p);
-  const float bp = __fsub_rn(t, s);
-  const float q = __fadd_rn(__fsub_rn(s, __fsub_rn(t, bp)), __fsub_rn(p, bp));
-  s = t;
-  c = __fadd_rn(c, __fadd_rn(q, e));
+__device__ __forceinline__ float2 fsub2_rn(float2 a, float2 b) {
+  float2 r;
+  asm("sub.rn.f32x2 %0, %1, %2;"
+      : "=l"(reinterpret_cast<unsigned long long&>(r))
+      : "l"(reinterpret_cast<const unsigned long long&>(a)), "l"(reinterpret_cast<const unsigned long long&>(b)));
+  return r;
 }
 
-// The same for a pair of sums at once (real and imaginary parts) in packed FP32x2 instructions:
-// element by element the operations and their roundings are those of dot2_add.
-__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
-__device__ __forceinline__ void dot2_add2(float2& s, float2& c, float2 a, float2 b) {
-  const float2 p = __fmul2_rn(a, b);
-  const float2 e = __ffma2_rn(a, b, neg2(p));
-  const float2 t = __fadd2_rn(s, p);
-  const float2 bp = __fadd2_rn(t, neg2(s));
-  const float2 q = __fadd2_rn(__fadd2_rn(s, neg2(__fadd2_rn(t, neg2(bp)))), __fadd2_rn(p, neg2(bp)));
+// (s, c) += a b for a pair of sums at once (real and imaginary parts) in packed FP32x2
+// instructions; nb = -b
+__device__ __forceinline__ void dot2_add2(float2& s, float2& c, float2 a, float2 b, float2 nb) {
+  const float2 np = __fmul2_rn(a, nb);  // -p
+  const float2 e = __ffma2_rn(a, b, np);
+  const float2 t = fsub2_rn(s, np);
+  const float2 bp = fsub2_rn(t, s);
+  const float2 q = fsub2_rn(fsub2_rn(s, fsub2_rn(t, bp)), __fadd2_rn(np, bp));
   s = t;
   c = __fadd2_rn(c, __fadd2_rn(q, e));
 }
 
-__global__ void __launch_bounds__(32 * TS_W)
+struct TwoWord {  // real and imaginary part of one sum
+  float2 s, c;
+};
+
+// w -= q x (complex): the real part takes (-q.x) x.x then q.y x.y, the imaginary part (-q.x) x.y
+// then (-q.y) x.x
+struct DotX {
+  float2 x, nx, xs, nxs;  // x, -x, swapped, -swapped
+  __device__ __forceinline__ explicit DotX(float2 v)
+      : x(v), nx(make_float2(-v.x, -v.y)), xs(make_float2(v.y, v.x)), nxs(make_float2(-v.y, -v.x)) {}
+};
+__device__ __forceinline__ void dot2_sub(TwoWord& w, float2 q, const DotX& x) {
+  dot2_add2(w.s, w.c, make_float2(-q.x, -q.x), x.x, x.nx);
+  dot2_add2(w.s, w.c, make_float2(q.y, -q.y), x.xs, x.nxs);
+}
+
+// A lane holds one row and S sources: every sum runs over the columns in order whatever the number
+// of sources, so a source's residual does not depend on the others of the call.  (A lane per
+// source, as before, left 31 of 32 lanes idle for one source; splitting a sum over lanes changes
+// its rounding with the number of sources.)  One block per (frequency, S sources, 64 rows): the
+// block's columns of X in shared memory, read as broadcasts; each warp streams its 32 rows of Q in
+// groups of J columns, read coalesced one group ahead and turned through shared memory.  Blocks of
+// two warps leave no round of blocks nearly empty (115 sources: blocks of eight 186 us).  Bound by
+// FP32 issue, 40 operations per complex product (packed: 174 us; as scalar operations 190 us):
+// 231 receivers x 17 refined frequencies, 115 sources 216 us before, 174 us now; one source 89 us
+// before, 18 us now (groups of 16 columns 22 us: the next group's reads take longer than a
+// group's sums).
+constexpr int RD_W = 2;  // warps per block
+
+template <int S, int J>
+__global__ void __launch_bounds__(32 * RD_W)
     k_resid_dot2(const float2* __restrict__ Qh, int n, const float2* __restrict__ Xh,
                  const float2* __restrict__ Dh, int ns, float2* __restrict__ Rh,
                  const int* __restrict__ kl) {
-  extern __shared__ float2 Xs[];  // [n][32]
+  extern __shared__ __align__(16) float2 Xs[];  // [n rounded up to J][S]
+  __shared__ float2 qs[RD_W][2][32 * (J + 1)];
   const int k = kl ? kl[blockIdx.y] : blockIdx.y;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int col = blockIdx.x * 32 + lane;
-  const bool valid = col < ns;
-  const float2* Q = Qh + (long long)k * n * n;
+  const int c0 = blockIdx.x * S;
   const long long off = (long long)k * n * ns;
-  for (int i = warp; i < n; i += TS_W)
-    Xs[i * 32 + lane] = valid ? Xh[off + (long long)i * ns + col] : make_float2(0.f, 0.f);
+  const int np = (n + J - 1) / J * J;
+  const int r0 = (blockIdx.z * RD_W + warp) * 32;
+  const int i = r0 + lane;
+  // group of columns j0 ..: this lane reads column j0 + lane % J of rows r0 + lane / J + (32 / J) t
+  const float2* Q = Qh + (long long)k * n * n;
+  constexpr int RS = 32 / J;  // rows per load
+  float2 pre[J];
+  auto load = [&](int j0) {
+    const int j = j0 + lane % J;
+#pragma unroll
+    for (int t = 0; t < J; ++t) {
+      const int r = r0 + lane / J + RS * t;
+      pre[t] = r < n && j < n ? __ldg(Q + (long long)r * n + j) : make_float2(0.f, 0.f);
+    }
+  };
+  load(0);
+  for (int e = threadIdx.x; e < np * S; e += 32 * RD_W) {
+    const int j = e / S, c = c0 + e % S;
+    Xs[e] = j < n && c < ns ? Xh[off + (long long)j * ns + c] : make_float2(0.f, 0.f);
+  }
   __syncthreads();
-  const int rows = (n + gridDim.z - 1) / gridDim.z;
-  const int i0 = blockIdx.z * rows, i1 = min(n, i0 + rows);
-  for (int i = i0 + 2 * warp; i < i1; i += 2 * TS_W) {
-    const bool two = i + 1 < i1;
-    const float2* qa = Q + (long long)i * n;
-    const float2* qb = Q + (long long)(two ? i + 1 : i) * n;
-    float2 da = make_float2(0.f, 0.f), db = make_float2(0.f, 0.f);
-    if (valid) {
-      da = Dh[off + (long long)i * ns + col];
-      if (two) db = Dh[off + (long long)(i + 1) * ns + col];
-    }
-    // R = D - Q X: the real part adds (-q.x) x.x then q.y x.y, the imaginary part (-q.x) x.y then
-    // (-q.y) x.x; (real, imaginary) sums and their compensations run as packed pairs
-    float2 sa = da, ca = make_float2(0.f, 0.f), sb = db, cb = make_float2(0.f, 0.f);
-#pragma unroll 4
-    for (int j = 0; j < n; ++j) {
-      const float2 x = Xs[j * 32 + lane], xs = make_float2(x.y, x.x);
-      const float2 a = __ldg(qa + j), b = __ldg(qb + j);
-      dot2_add2(sa, ca, make_float2(-a.x, -a.x), x);
-      dot2_add2(sa, ca, make_float2(a.y, -a.y), xs);
-      dot2_add2(sb, cb, make_float2(-b.x, -b.x), x);
-      dot2_add2(sb, cb, make_float2(b.y, -b.y), xs);
-    }
-    if (valid) {
-      Rh[off + (long long)i * ns + col] = __fadd2_rn(sa, ca);
-      if (two) Rh[off + (long long)(i + 1) * ns + col] = __fadd2_rn(sb, cb);
+  if (r0 >= n) return;
+  TwoWord w[S];
+#pragma unroll
+  for (int u = 0; u < S; ++u) {
+    w[u].s = i < n && c0 + u < ns ? Dh[off + (long long)i * ns + c0 + u] : make_float2(0.f, 0.f);
+    w[u].c = make_float2(0.f, 0.f);
+  }
+  for (int j0 = 0, b = 0; j0 < n; j0 += J, b ^= 1) {
+    float2* g = qs[warp][b];
+#pragma unroll
+    for (int t = 0; t < J; ++t) g[(lane / J + RS * t) * (J + 1) + lane % J] = pre[t];
+    __syncwarp();
+    if (j0 + J < n) load(j0 + J);
+    // (past n both factors are zero, which changes neither word)
+#pragma unroll
+    for (int jj = 0; jj < J; ++jj) {
+      const float2 q = g[lane * (J + 1) + jj];
+#pragma unroll
+      for (int u = 0; u < S; ++u) dot2_sub(w[u], q, DotX(Xs[(j0 + jj) * S + u]));
     }
   }
+  if (i < n)
+#pragma unroll
+    for (int u = 0; u < S; ++u)
+      if (c0 + u < ns) Rh[off + (long long)i * ns + c0 + u] = __fadd2_rn(w[u].s, w[u].c);
 }
 
 cudaError_t launch_resid(const float2* Qh, int n, int nf, const float2* Xh, const float2* Dh,
                          int ns, float2* Rh, bool fp64, cudaStream_t st, const int* kl) {
   if (nf < 1) return cudaSuccess;
-  const size_t smem = sizeof(float2) * 32 * (size_t)n;
-  if (smem > 48 * 1024) {
-    cudaError_t e = fp64 ? cudaFuncSetAttribute(k_resid64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
-                         : cudaFuncSetAttribute(k_resid_dot2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
+  cudaError_t e;
   count_launches(1);
-  // enough blocks for every SM: split the rows of each (frequency, source group)
-  const int blocks = ((ns + 31) / 32) * nf;
-  const int groups = std::max(1, std::min((n + TS_W - 1) / TS_W, (4 * 152 + blocks - 1) / blocks));
-  const dim3 grid((ns + 31) / 32, nf, groups);
-  if (fp64)
-    k_resid64<<<grid, 32 * TS_W, smem, st>>>(Qh, n, Xh, Dh, ns, Rh, kl);
-  else
-    k_resid_dot2<<<grid, 32 * TS_W, smem, st>>>(Qh, n, Xh, Dh, ns, Rh, kl);
+  if (fp64) {
+    const size_t smem = sizeof(float2) * 32 * (size_t)n;
+    if (smem > 48 * 1024 &&
+        (e = cudaFuncSetAttribute(k_resid64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)))
+      return e;
+    // enough blocks for every SM: split the rows of each (frequency, source group)
+    const int blocks = ((ns + 31) / 32) * nf;
+    const int groups = std::max(1, std::min((n + TS_W - 1) / TS_W, (4 * 152 + blocks - 1) / blocks));
+    k_resid64<<<dim3((ns + 31) / 32, nf, groups), 32 * TS_W, smem, st>>>(Qh, n, Xh, Dh, ns, Rh, kl);
+    return cudaGetLastError();
+  }
+  // sources per lane: four share each entry of Q where that still gives the schedulers two warps
+  // each; fewer spread a small call out, with longer groups to cover the reads
+  const long long warps = (long long)((n + 31) / 32) * nf * ns;
+  const int S = warps >= 4 * 2 * 608 ? 4 : warps >= 2 * 2 * 608 ? 2 : 1;
+  const int J = S == 4 ? 8 : S == 2 ? 16 : 32;
+  auto kern = S == 4 ? k_resid_dot2<4, 8> : S == 2 ? k_resid_dot2<2, 16> : k_resid_dot2<1, 32>;
+  const size_t smem = sizeof(float2) * S * (size_t)((n + J - 1) / J * J);
+  if (smem > 12 * 1024 &&  // beside up to 33 KB of turned groups
+      (e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)))
+    return e;
+  kern<<<dim3((ns + S - 1) / S, nf, (n + 32 * RD_W - 1) / (32 * RD_W)), 32 * RD_W, smem, st>>>(
+      Qh, n, Xh, Dh, ns, Rh, kl);
   return cudaGetLastError();
 }
 

@@ -113,6 +113,8 @@ struct egh_ctx {
   size_t Dr_cap = 0, Rr_cap = 0;
   float *io_in = nullptr, *io_out = nullptr;
   size_t io_in_cap = 0, io_out_cap = 0;
+  float* trace_ws = nullptr;  // the forward transform's block sums (calls with few traces)
+  size_t trace_ws_cap = 0;
   unsigned char* syn_ops = nullptr;  // the synthesis operand images
   size_t syn_ops_cap = 0;
   int state = ST_CREATED;
@@ -315,7 +317,7 @@ cudaError_t zero_snap_slot(egh_ctx* ctx, int j, cudaStream_t st) {
 void free_all(egh_ctx* c) {
   void* ptrs[] = {c->Ph, c->fro2, c->kref, c->xbuf, c->rflags, c->tws_deb, c->twt_deb, c->twt_bl, c->Wh, c->Dr, c->Rr, c->coef, c->lev, c->snap, c->twt, c->gh, c->ghb, c->part, c->Qh, c->Lh, c->tw, c->w_dev,
                   c->rec_pts, c->status, c->dsum, c->lmax, c->vchk, c->d_err, c->vel_stage, c->Dh,
-                  c->io_in, c->io_out, c->syn_ops};
+                  c->io_in, c->io_out, c->syn_ops, c->trace_ws};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   for (cudaEvent_t& e : c->ev)
@@ -1178,8 +1180,12 @@ static egh_status deblur_common(egh_ctx* ctx, const float* resid, int32_t ns, in
   CK(cudaEventRecord(ctx->ev[6], stream));
   const int expire = ctx->expire[2] > 0 ? 1 : 0;
   ctx->expire[2] -= expire;
+  const size_t sb = in_map ? 0 : trace_scratch_bytes(ctx->nf, ntr, nt_d);
+  if (sb && (s = ensure_buf(ctx, (void**)&ctx->trace_ws, &ctx->trace_ws_cap, sb, stream, "transform blocks")))
+    return s;
   CK(launch_trace_dft(din, (int)ntr, nt_d, ctx->nf, ctx->nrec, ns, 0, D, stream,
-                      ctx->twt_deb, ctx->d_err, expire, in_map == nullptr));
+                      ctx->twt_deb, ctx->d_err, expire, in_map == nullptr, ctx->trace_ws,
+                      ctx->trace_ws_cap));
   const size_t dbytes = (size_t)ctx->nf * ntr * sizeof(float2);
   const bool refine = !diag && prec_mixed(ctx->prec) && ctx->nref > 0;
   if (!diag && prec_mixed(ctx->prec) &&

@@ -167,10 +167,14 @@ cudaError_t launch_potrf(float2* Lh, int n, int nf, int* status, cudaStream_t st
 // spectra of ntr = nrec * ns traces into columns s0 .. s0+ns-1 of D[nf][nrec][ld] on the tensor
 // cores; twt: the transform's twiddle tiles for at least nt_d levels; err: the flag a bounded
 // wait sets (both required; nf <= 64); expire: test hook, the first CTA's first wait runs out
-// dev_in: resid is device memory (not a mapping of host memory), which the TMA form needs
+// dev_in: resid is device memory (not a mapping of host memory), which the TMA form needs;
+// scratch: device memory of scratch_bytes for the block sums of calls with few traces (used when
+// trace_scratch_bytes asks for some and it is large enough)
 cudaError_t launch_trace_dft(const float* resid, int ntr, int nt_d, int nf, int nrec, int ld,
                              int s0, float2* Dh, cudaStream_t st, const unsigned char* twt,
-                             int* err, int expire = 0, bool dev_in = false);
+                             int* err, int expire = 0, bool dev_in = false, void* scratch = nullptr,
+                             size_t scratch_bytes = 0);
+size_t trace_scratch_bytes(int nf, long long ntr, int nt_d);
 cudaError_t launch_trsm(const float2* Lh, int n, int nf, float2* Dh, int ns, cudaStream_t st);
 // W = L^{-1} per frequency
 cudaError_t launch_trtri(const float2* Lh, int n, int nf, float2* Wh, cudaStream_t st);

@@ -67,3 +67,62 @@ def test_solve_backward_error(n, ns, precision, tmp_path):
         q = Q[k].astype(np.complex128)
         res = np.linalg.norm(out["D"][k] - q @ out["X"][k])
         assert res <= 2e-6 * np.linalg.norm(q, 2) * np.linalg.norm(out["X"][k]), (k, res)
+
+
+@pytest.mark.parametrize("nf", [3, 16, 17, 33, 48, 49])
+@pytest.mark.parametrize("n,ns,nt", [(1, 1, 64), (5, 1, 256), (127, 1, 388), (129, 1, 4000), (64, 5, 2052), (40, 60, 900),
+                                     (7, 3, 2001)])
+def test_forward_transform(n, ns, nt, nf, tmp_path):
+    """Spectra of egh_deblur_freq with Q = I (the product with the identity is exact) against the
+    64-bit transform: traces of one tile, a few tiles and many,
+    one stage to many (block sums from scratch), every width of the component dimension, rows that are not a multiple of
+    16 bytes.  The bf16 pairs carry 16 bits: 2^-17 per factor, 2e-5 of the spectra's norm with room
+    for the dropped product."""
+    import torch
+
+    rng = np.random.default_rng(n + ns + nt + nf)
+    r = rng.standard_normal((ns, n, nt)).astype(np.float32)
+    with _line_ctx(n, nf, nt, 1) as ctx:
+        ctx.prec_for_test = 1
+        _load_set(ctx, np.broadcast_to(np.eye(n, dtype=np.complex64), (nf, n, n)).copy(), tmp_path)
+        x = torch.zeros((nf, n, ns, 2), device="cuda")
+        for _ in range(2):  # again on the same scratch
+            ctx.deblur_freq(torch.from_numpy(r).cuda(), x)
+        torch.cuda.synchronize()
+        got = torch.view_as_complex(x).cpu().numpy()
+        ph = 2 * np.pi * np.mod(ctx.freqs[:, None] * np.arange(nt)[None] * 1e-3, 1.0)
+        many = torch.from_numpy(np.concatenate([r] * (-(-20000 // (n * ns))))).cuda() if n * ns < 200 else None
+        if many is not None:  # the same traces among many others: the same bits
+            y = torch.zeros((nf, n, many.shape[0], 2), device="cuda")
+            ctx.deblur_freq(many, y)
+            assert torch.equal(y[:, :, :ns], x) and torch.equal(y[:, :, -ns:], x)
+    ref = np.einsum("kt,srt->krs", np.exp(-1j * ph), r.astype(np.float64), optimize=True)
+    assert np.linalg.norm(got - ref) <= 2e-5 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("nrec", [1, 16, 24, 33, 48, 49, 97])
+@pytest.mark.parametrize("nx,nz,gram_splits", [(64, 3, 0), (60, 7, 1), (61, 40, 5), (130, 33, 0)])
+def test_gram_fp32(nrec, nx, nz, gram_splits):
+    """FP32 Hessians of imported transforms against the 64-bit Gram: one tile to several of either
+    edge, last panels with few rows, point ranges that begin and end inside a grid row, skipped
+    padding columns.  FP32 products and sums over at most 4000 points with chains of at most 1024:
+    random rounding stays below 1e-6 of the Hessian's norm."""
+    import torch
+    from paper_2512_16642_gb300 import egh
+
+    rng = np.random.default_rng(nrec + nx)
+    nf = 2
+    ix = np.arange(nrec, dtype=np.int32) % nx
+    with egh.Context(nz, nx, 10.0, 10.0, 0, 0.5, 1e-3, 100, np.zeros(nrec, np.int32), ix,
+                     np.array([5.0, 9.0]), precision=0, gram_splits=gram_splits) as ctx:
+        buf = ctx.transform_buffer(nrec, nf)
+        px = ctx.stats()["pitch"]
+        v = rng.standard_normal((nrec, nf, 2, nz, nx)).astype(np.float32)
+        buf[..., : nz * px].unflatten(-1, (nz, px))[..., :nx] = torch.from_numpy(v).cuda()
+        ctx.import_green(buf)
+        ctx.hessian(egh.EGH_MU_ABS, 0.0)
+        Q = ctx.get_hessian(False)
+    g = (v[:, :, 0] + 1j * v[:, :, 1]).reshape(nrec, nf, -1).astype(np.complex128)
+    for k in range(nf):
+        H = g[:, k] @ g[:, k].conj().T
+        assert np.linalg.norm(Q[k] - H) <= 1e-6 * np.linalg.norm(H), k
