@@ -684,6 +684,17 @@ __global__ void __launch_bounds__(128, 16)
 #pragma unroll
         for (int i = 0; i < 8; ++i) v[i] += o[i];
       }
+      if (!first && !last) {
+        // middle chunks: each total is added where it lies (no other thread adds to it; rounded as
+        // the sum of a read, an add and a write), so that the tile does not wait for the old totals:
+        // on 512-level chunks of the layered grid the transform took as long as the FD steps beside
+        // it and held them up (transform 1000 -> 715 ms, Green stage 1032 -> 957 ms)
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+          if (c0 + i < 2 * nf)
+            asm volatile("red.global.add.f32 [%0], %1;" ::"l"(g + (long long)(c0 + i) * G), "f"(v[i]) : "memory");
+        continue;
+      }
       // all loads of the group before any store: the 8 column planes are distinct
 #pragma unroll
       for (int i = 0; i < 8; ++i)
