@@ -114,8 +114,12 @@ cudaError_t launch_build_coef(const float* vel, const Layout& L, double dz, doub
 // (fully unrolled, so the z-window rotates through registers).  The u^n rows stream through a
 // per-warp ring of FD_RING shared-memory rows (64 points + 4 halo points on each side) filled by
 // cp.async FD_D rows ahead of use; the same ring rows give the x-neighbours (five 16-byte loads
-// per lane).  u^{n-1} and the coefficients are prefetched into registers FD_P rows ahead.  Reads
-// of guard rows and padding columns return the zero boundary, so loads need no bounds test.
+// per lane).  The u^{n-1} rows come through a ring of their own, equally far ahead; the
+// coefficients are prefetched into registers FD_P rows ahead.  (Held in registers two rows ahead,
+// u^{n-1} set the pace: a row took half an L2 latency however few warps shared the SM.  Layered
+// update, Green stage: 957 ms before, 886 ms now; decimated update 152 and 140 ms; distances of 4, 6
+// and 7 rows 896, 897 and 982 ms, the last for want of room beside the transform's ring.)
+// Reads of guard rows and padding columns return the zero boundary, so loads need no bounds test.
 //
 // The Laplacian is taken in first differences: with D_j = u_j - u_{j-1} along an axis,
 //   sum_k c_k (u_{+k} + u_{-k} - 2u) = sum_{j=1..4} C_j (D_{+j} - D_{1-j}),  C_j = sum_{k>=j} c_k,
@@ -127,14 +131,19 @@ cudaError_t launch_build_coef(const float* vel, const Layout& L, double dz, doub
 // transform reads.
 // ---------------------------------------------------------------------------------------------
 #ifndef EGH_FD_P
-#define EGH_FD_P 2
+#define EGH_FD_P 4
+#endif
+#ifndef EGH_FD_D
+#define EGH_FD_D 5
 #endif
 #ifndef EGH_FD_MINB
 #define EGH_FD_MINB 1
 #endif
-constexpr int FD_RING = 12;     // ring rows per warp (indices are compile-time: any count)
-constexpr int FD_D = 7;         // u^n rows in flight ahead of the window's leading row
-constexpr int FD_P = EGH_FD_P;  // u^{n-1} / coefficient rows prefetched ahead
+constexpr int FD_D = EGH_FD_D;    // u^n and u^{n-1} rows in flight ahead of the ones in use
+constexpr int FD_RING = FD_D + 5; // u^n ring rows per warp (indices are compile-time: any count)
+constexpr int FD_UP = FD_D + 1;   // u^{n-1} ring rows per warp
+constexpr int FD_P = EGH_FD_P;    // coefficient rows prefetched ahead into registers
+constexpr int FD_WARP4 = FD_RING * 36 + FD_UP * 32;  // float4 of shared memory per warp
 static_assert(FD_D + 5 <= FD_RING && FD_D + 8 >= FD_RING, "ring rows must cover the prefetch distance");
 
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) {
@@ -192,8 +201,10 @@ __global__ void __launch_bounds__(32 * FD_MAXPAIRS, EGH_FD_MINB)
     k_fd_step(const float2* __restrict__ ucur, const float2* __restrict__ uprev,
               float2* __restrict__ unext, const float2* __restrict__ coef, int NZ, int NX, int PX,
               int org, long long pstride, Stencil C, SnapOut so) {
-  extern __shared__ __align__(16) float4 ring_all[];  // [pairs][FD_RING][36]
-  float4 (*ring)[36] = reinterpret_cast<float4 (*)[36]>(ring_all + threadIdx.y * FD_RING * 36);
+  // per pair: u^n rows [FD_RING][36], then u^{n-1} rows [FD_UP][32] (a lane reads what it copied)
+  extern __shared__ __align__(16) float4 ring_all[];
+  float4 (*ring)[36] = reinterpret_cast<float4 (*)[36]>(ring_all + threadIdx.y * FD_WARP4);
+  const float4* upr = ring_all + threadIdx.y * FD_WARP4 + FD_RING * 36 + threadIdx.x;
   const int lane = threadIdx.x;
   const int pair = threadIdx.y;
   const int x0 = blockIdx.x * 64;
@@ -211,6 +222,7 @@ __global__ void __launch_bounds__(32 * FD_MAXPAIRS, EGH_FD_MINB)
   const int hcol = lane < 2 ? (x0 >> 1) - 2 + lane : (x0 >> 1) + 32 + (lane - 30);
   const int hslot = lane < 2 ? lane : 34 + (lane - 30);
   const unsigned ring0 = (unsigned)__cvta_generic_to_shared(&ring[0][0]);
+  const unsigned up0 = ring0 + (unsigned)(FD_RING * 36 + lane) * 16u;
   const bool ok0 = x < NX, ok1 = x + 1 < NX;
   // ring row k holds u^n row z0 - 4 + k; rows z0 - 4 .. z0 + nrows + 3 exist (guard rows included)
   const int nload = nrows + 8;
@@ -225,18 +237,22 @@ __global__ void __launch_bounds__(32 * FD_MAXPAIRS, EGH_FD_MINB)
       // would reach past the level
       if (halo && z >= 0 && z < NZ) cp_async16(dst + (unsigned)hslot * 16u, uc + r + hcol);
     }
+    // row k - 8 of the tile: its u^{n-1} arrives with the last u^n row it needs
+    if (k >= 8 && k - 8 < nrows)
+      cp_async16(up0 + (unsigned)(((k - 8) % FD_UP) * 32) * 16u, up + (z0 + k - 8) * PX2);
     cp_async_commit();  // empty groups keep the group count uniform
   };
+  // Programmatic dependent launch (where the launch asks for it): this block may start while the
+  // previous step's last blocks run.  Its first coefficients are read before the wait for that
+  // step; the next step may start once every block is past it.
+  float4 pc[FD_P];
+#pragma unroll
+  for (int i = 0; i < FD_P; ++i)
+    if (i < nrows) pc[i] = __ldg(cf + (z0 + i) * PX2);
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 #pragma unroll
   for (int k = 0; k < FD_RING; ++k) load_row(k);
-  float4 pu[FD_P], pc[FD_P];
-#pragma unroll
-  for (int i = 0; i < FD_P; ++i) {
-    if (i < nrows) {
-      pu[i] = __ldcg(up + (z0 + i) * PX2);
-      pc[i] = __ldg(cf + (z0 + i) * PX2);
-    }
-  }
   cp_async_wait<FD_RING - 8>();  // rows 0 .. 7 have landed
   __syncwarp();
   // z first differences of both receivers at point p (0: x, 1: x + 1) of the lane:
@@ -274,11 +290,8 @@ __global__ void __launch_bounds__(32 * FD_MAXPAIRS, EGH_FD_MINB)
     load_row(FD_D + 8 + i);
     cp_async_wait<FD_D>();
     __syncwarp();
-    const float4 uo = pu[i % FD_P], cc = pc[i % FD_P];
-    if (i + FD_P < nrows) {
-      pu[i % FD_P] = __ldcg(up + (z0 + i + FD_P) * PX2);
-      pc[i % FD_P] = __ldg(cf + (z0 + i + FD_P) * PX2);
-    }
+    const float4 uo = upr[(i % FD_UP) * 32], cc = pc[i % FD_P];
+    if (i + FD_P < nrows) pc[i % FD_P] = __ldg(cf + (z0 + i + FD_P) * PX2);
     {
       const float4 v = ring[(i + 8) % FD_RING][lane + 2];  // u^n at row z + 4
       const float2 nv[2] = {make_float2(v.x, v.y), make_float2(v.z, v.w)};
@@ -339,7 +352,7 @@ __global__ void __launch_bounds__(32 * FD_MAXPAIRS, EGH_FD_MINB)
 
 int fd_rows_per_warp_default() { return EGH_FD_TZDEF; }
 
-int fd_block_smem(int npairs) { return (int)(sizeof(float4) * FD_RING * 36 * npairs); }
+int fd_block_smem(int npairs) { return (int)(sizeof(float4) * FD_WARP4 * npairs); }
 
 long long fd_sm_smem(int npairs, int tz) {
   int dev = 0, occ = 0, reserved = 0;
@@ -392,7 +405,7 @@ int fd_rows_one_wave(const Layout& L, int npairs) {
 // Raises the dynamic shared-memory limit of every FD and transform kernel instance once per
 // process (outside any stream capture).
 cudaError_t fd_prepare(int nf) {
-  const int fd_smem = (int)(sizeof(float4) * FD_RING * 36 * FD_MAXPAIRS);
+  const int fd_smem = fd_block_smem(FD_MAXPAIRS);
   cudaError_t e;
   if ((e = cudaFuncSetAttribute(k_fd_step<12>, cudaFuncAttributeMaxDynamicSharedMemorySize, fd_smem))) return e;
   if ((e = cudaFuncSetAttribute(k_fd_step<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, fd_smem))) return e;
@@ -429,12 +442,26 @@ cudaError_t launch_fd_step(const float2* ucur, const float2* uprev, float2* unex
   const dim3 blk(32, npairs);
   const size_t smem = fd_block_smem(npairs);
   const int org = (int)L.org;
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.blockDim = blk;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &at;
+  // Programmatic launch hides most of a launch's and a first row's latency, which is much of a small
+  // grid's step (101x101 grid, 21 receivers x 1000 steps: 10.8 -> 9.5 ms), and helps where no
+  // snapshot is written for a transform beside (decimated update 154.7 -> 152.1 ms, modelling of 23
+  // shots 34.4 -> 26.7 ms); beside the transform, a full grid's early blocks take what it would use
+  // (layered: Green stage 957 -> 979 ms).
+  cfg.numAttrs = so.lvl == nullptr || (long long)(L.PX / 64) * ((L.NZ + tz - 1) / tz) < 152 ? 1 : 0;
   switch (tz) {
 #define EGH_FD_CASE(T)                                                                          \
   case T:                                                                                       \
-    k_fd_step<T><<<dim3(L.PX / 64, (L.NZ + T - 1) / T), blk, smem, st>>>(                        \
-        ucur, uprev, unext, coef, L.NZ, L.NX, L.PX, org, L.F, C, so);                           \
-    break;
+    cfg.gridDim = dim3(L.PX / 64, (L.NZ + T - 1) / T);                                           \
+    return cudaLaunchKernelEx(&cfg, k_fd_step<T>, ucur, uprev, unext, coef, L.NZ, L.NX, L.PX,    \
+                              org, L.F, C, so);
     EGH_FD_CASE(12)
     EGH_FD_CASE(16)
     EGH_FD_CASE(18)
