@@ -130,12 +130,14 @@ typedef struct {
                                 egh_green of the context: the smallest count whose tiles fit one
                                 wave of resident blocks is kept unless another is 3% faster */
     int32_t precision;       /* egh_precision of the Hessian stage (0 = EGH_PREC_FP32) */
-    int32_t fd_kernel;       /* FD solver of the Green stage: 0 or 2 = one kernel per time step,
-                                state in global memory (L2-resident), the faster one on a GB300;
-                                1 = resident: the batch's wavefield stays in shared memory for a
+    int32_t fd_kernel;       /* FD solver of the Green stage: 2 = one kernel per time step, state in
+                                global memory (L2-resident); 0 = that one, but on small grids (and
+                                with fd_rows = 0) a cluster of blocks per receiver pair that keeps
+                                the pair's wavefield in shared memory for a transform chunk; 1 =
+                                resident: the batch's wavefield stays in shared memory for a
                                 whole transform chunk, one block per SM in a cooperative launch,
                                 halos exchanged between neighbouring blocks every step (EGH_EINVAL
-                                if it does not fit).  Both give identical levels.  With the
+                                if it does not fit).  All give identical levels.  With the
                                 resident solver, batch_receivers = 0 takes the most receivers whose
                                 state fits (at most 16) and fd_rows does not apply (its rows per
                                 segment are timed on the first egh_green) */
@@ -164,7 +166,7 @@ typedef struct {
     int64_t dft_launches;      /* last egh_green: transform launches */
     double gram_ms;            /* last egh_hessian: device time of the Gram kernel */
     int64_t fd_steps;          /* last egh_green: FD time steps computed (all batches) */
-    int32_t fd_kernel;         /* FD solver in use: 1 resident, 2 per step */
+    int32_t fd_kernel;         /* FD solver in use: 1 resident, 2 per step, 3 clusters */
     int32_t fd_tiles;          /* resident solver: blocks (tiles) per launch, else 0 */
 } egh_stats;
 

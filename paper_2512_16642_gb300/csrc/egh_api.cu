@@ -50,7 +50,12 @@ struct egh_ctx {
   int Bcap = 0;         // receivers the FD state slots hold (>= B)
   bool tune_B = false;  // B is timed on the first egh_green (8, 16 or 32 receivers)
   int fd_tz = 0;  // FD rows per warp of the per-step kernel (0 = library default)
-  int fd_kernel = 2;  // 1: resident solver (fd_resident.cu), 2: one kernel per step (fd.cu)
+  // 1: resident solver (fd_resident.cu), 2: one kernel per step (fd.cu), 3: a cluster per receiver
+  // pair (fd_cluster.cu)
+  int fd_kernel = 2;
+  ClGeom cl{};             // cluster solver
+  float* wav_dev = nullptr;  // cluster solver: the wavelet of a band-limited Green stage
+  size_t wav_cap = 0;
   ResGeom rg{};       // resident solver: tile grid and pairs per block
   int res_sr = 0;     // resident solver: rows per z-march segment (0 = timed on first egh_green)
   float4* xbuf = nullptr;  // resident solver: halo exchange strips
@@ -317,7 +322,7 @@ cudaError_t zero_snap_slot(egh_ctx* ctx, int j, cudaStream_t st) {
 void free_all(egh_ctx* c) {
   void* ptrs[] = {c->Ph, c->fro2, c->kref, c->xbuf, c->rflags, c->tws_deb, c->twt_deb, c->twt_bl, c->Wh, c->Dr, c->Rr, c->coef, c->lev, c->snap, c->twt, c->gh, c->ghb, c->part, c->Qh, c->Lh, c->tw, c->w_dev,
                   c->rec_pts, c->status, c->dsum, c->lmax, c->vchk, c->d_err, c->vel_stage, c->Dh,
-                  c->io_in, c->io_out, c->syn_ops, c->trace_ws};
+                  c->io_in, c->io_out, c->syn_ops, c->trace_ws, c->wav_dev};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   for (cudaEvent_t& e : c->ev)
@@ -548,7 +553,15 @@ egh_status egh_create(const egh_config* cfg, egh_ctx** out) {
                     "block per SM resident (grid too large, or batch_receivers too many)");
       }
     }
-    ctx->fd_kernel = res ? 1 : 2;
+    // by default the cluster solver where a pair's wavefield fits a cluster's shared memory and it is
+    // the faster one (no rows per warp asked for: that is the per-step kernel's)
+    ctx->fd_kernel = 2;
+    if (res) {
+      ctx->fd_kernel = 1;
+    } else if (c.fd_kernel == 0 && c.fd_rows == 0 && fd_cluster_plan(L, &ctx->cl)) {
+      const int b = c.batch_receivers ? c.batch_receivers : 32;
+      if (fd_cluster_faster(ctx->cl, L, c.nrec, b)) ctx->fd_kernel = 3;
+    }
     if (res)
       ctx->B = c.batch_receivers ? std::min(c.batch_receivers, c.nrec) : std::min(c.nrec, 2 * ctx->rg.P);
     else
@@ -749,7 +762,19 @@ egh_status green_run(egh_ctx* ctx, const float* vel, cudaStream_t stream, const 
   ctx->state = ST_CREATED;
   egh_status s = prepare_model(ctx, vel, stream);
   if (s) return s;
+  if (ctx->tune_B && ctx->fd_kernel == 3) {
+    // every pair has a cluster of its own: as many as run at once, at most what the slots hold
+    ctx->B = std::min(ctx->Bcap, 2 * ctx->cl.clusters);
+    ctx->Bp = 2 * ((ctx->B + 1) / 2);
+    ctx->st.batch_receivers = ctx->B;
+    ctx->tune_B = false;
+  }
   if (ctx->tune_B && (s = tune_batch(ctx, stream))) return s;
+  if (wav && ctx->fd_kernel == 3) {
+    if ((s = ensure_buf(ctx, (void**)&ctx->wav_dev, &ctx->wav_cap, nw * sizeof(float), stream, "wavelet")))
+      return s;
+    CK(cudaMemcpyAsync(ctx->wav_dev, wav, nw * sizeof(float), cudaMemcpyHostToDevice, stream));
+  }
   s = ensure_green_buffers(ctx);
   if (s) return s;
   const Layout& L = ctx->L;
@@ -861,7 +886,8 @@ egh_status green_run(egh_ctx* ctx, const float* vel, cudaStream_t stream, const 
       }
       // levels that still take a wavelet sample: a step, then the injection, launched directly
       const int ta = std::max(t0, 2);
-      const int tw = wav ? std::max(ta, std::min(t1, nw + 1)) : ta;
+      // (the cluster solver takes them itself)
+      const int tw = wav && ctx->fd_kernel != 3 ? std::max(ta, std::min(t1, nw + 1)) : ta;
       for (int t = ta; t < tw; ++t) {
         const SnapOut so = level_snap(ctx, t, t0, sbase, D);
         CK(launch_fd_step(slot(ctx, t - 1), slot(ctx, t - 2), slot(ctx, t), ctx->coef, L, ctx->S, np,
@@ -875,11 +901,16 @@ egh_status green_run(egh_ctx* ctx, const float* vel, cudaStream_t stream, const 
           ctx->expire[1] -= expire;
           CK(resident(tw, t0, t1, sbase, np, D, ctx->res_sr, expire));
         }
+      } else if (ctx->fd_kernel == 3) {
+        if (tw < t1)
+          CK(launch_fd_cluster(ctx->cl, ctx->lev, (ctx->Bcap + 1) / 2, L, ctx->coef, ctx->S, nb, tw, t1 - tw,
+                               t0, D, sbase, ctx->snap, per, 2LL * K * per, L.G, wav ? ctx->wav_dev : nullptr,
+                               nw, ctx->rec_pts + b0, src_scale, fs));
       } else if ((s = fd_chunk_steps(ctx, tw, t0, t1, sbase, np, D))) {
         return s;
       }
       fd_steps += std::max(0, t1 - std::max(t0, 2));
-      if (ctx->fd_kernel == 1 && tw < t1) ++fd_kernel_launches;
+      if (ctx->fd_kernel != 2 && tw < t1) ++fd_kernel_launches;
       CK(cudaEventRecord(ctx->ev_fd[2 * g + 1], fs));
       CK(cudaEventRecord(ctx->fd_done[g & 1], fs));
       CK(cudaStreamWaitEvent(ctx->side, ctx->fd_done[g & 1], 0));
@@ -892,11 +923,12 @@ egh_status green_run(egh_ctx* ctx, const float* vel, cudaStream_t stream, const 
       // 40 frequencies on the salt grid, transform 5.9 s against FD steps 5.1 s per patch), so
       // there the transform takes one CTA per tile and fills the SMs between FD launches.
       const bool alone = b0 + B >= ctx->nrec && c == nchunk - 1;
-      const bool slim = dft_ncomp(ctx->nf) <= 64 && ctx->fd_kernel != 1;
+      const bool slim = dft_ncomp(ctx->nf) <= 64 && ctx->fd_kernel == 2;
       const long long beside = fd_sm_smem((std::min(B, ctx->nrec) + 1) / 2, ctx->fd_tz);
       CK(launch_dft_tc(ctx->tmap, twt, ctx->nf, sbase, m1 - m0, m0, L, ctx->gh, ctx->ghb,
                        (m1 == ntd && ctx->ghb) ? 1 : 0, b0, nb, ctx->nrec, ctx->d_err, expire,
-                       alone ? 3 : slim ? 1 : 0, (alone || !slim) ? 0 : beside, ctx->side));
+                       alone || ctx->fd_kernel == 3 ? 3 : slim ? 1 : 0, (alone || !slim) ? 0 : beside,
+                       ctx->side));
       CK(cudaEventRecord(ctx->ev_dft[2 * g + 1], ctx->side));
       CK(cudaEventRecord(ctx->dft_done[g & 1], ctx->side));
     }
@@ -928,7 +960,7 @@ egh_status green_run(egh_ctx* ctx, const float* vel, cudaStream_t stream, const 
     }
     ctx->st.fd_ms = fd;
     ctx->st.dft_ms = dft;
-    ctx->st.fd_launches = ctx->fd_kernel == 1 ? fd_kernel_launches
+    ctx->st.fd_launches = ctx->fd_kernel != 2 ? fd_kernel_launches
                                               : (long long)((ctx->nrec + B - 1) / B) * std::max(0, nt - 2);
     ctx->st.dft_launches = g;
     ctx->st.fd_steps = fd_steps;
@@ -1400,7 +1432,7 @@ egh_status egh_get_stats(egh_ctx* ctx, egh_stats* out) {
       *ms[i] = t;
     }
   ctx->st.kernel_launches = launches_so_far();
-  ctx->st.fd_rows = ctx->fd_kernel == 1 ? ctx->res_sr : ctx->fd_tz;
+  ctx->st.fd_rows = ctx->fd_kernel == 1 ? ctx->res_sr : ctx->fd_kernel == 3 ? ctx->cl.sr : ctx->fd_tz;
   ctx->st.fd_kernel = ctx->fd_kernel;
   ctx->st.fd_tiles = ctx->fd_kernel == 1 ? ctx->rg.TR * ctx->rg.TC : 0;
   *out = ctx->st;

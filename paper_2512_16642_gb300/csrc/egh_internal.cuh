@@ -121,6 +121,28 @@ cudaError_t launch_fd_resident(const ResGeom& g, int sr, float2* lev, int pslot,
                                long long splane, long long srec, float4* xbuf, int* flags,
                                int* err, int expire, cudaStream_t st);
 
+// ---- fd_cluster.cu ----------------------------------------------------------------------------
+// Small grids: a cluster of blocks per receiver pair, both levels of its rows in each block's
+// shared memory.
+struct ClGeom {
+  int rows;        // grid rows per block at most
+  int sr;          // rows per unit
+  int threads;     // per block
+  int clusters;    // clusters that the GPU holds at once
+  bool coef_smem;  // coefficients in shared memory too
+  size_t smem;     // dynamic shared memory per block
+};
+bool fd_cluster_plan(const Layout& L, ClGeom* g);  // false if the grid does not fit
+// whether nrec receivers, at most b in a batch, take less time than with the per-step kernel
+bool fd_cluster_faster(const ClGeom& g, const Layout& L, int nrec, int b);
+// Levels ta .. ta+nsteps-1 (ta >= 2) of nb receivers from the state slots of levels ta-1, ta-2 to
+// the slots of the last two; level t's snapshot to ring slot sbase + (t - t0) / decim when
+// t % decim == 0; wav (device, may be null): level t takes sample t - 1 < nw at the receivers' points
+cudaError_t launch_fd_cluster(const ClGeom& g, float2* lev, int pslot, const Layout& L, const float2* coef,
+                              const Stencil& S, int nb, int ta, int nsteps, int t0, int decim, int sbase,
+                              __nv_bfloat16* snap, long long sslot, long long splane, long long srec,
+                              const float* wav, int nw, const int* pts, float scale, cudaStream_t st);
+
 // ---- gram_tc.cu -------------------------------------------------------------------------------
 // Gram on the tensor cores from the bf16 hi/lo transforms ghb[nrec][nf][re/im][hi/lo][G].
 __host__ __device__ int gram_tc_blocks(int nrec);

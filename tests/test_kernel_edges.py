@@ -126,3 +126,39 @@ def test_gram_fp32(nrec, nx, nz, gram_splits):
     for k in range(nf):
         H = g[:, k] @ g[:, k].conj().T
         assert np.linalg.norm(Q[k] - H) <= 1e-6 * np.linalg.norm(H), k
+
+
+@pytest.mark.parametrize("nz,nx,nsponge,nrec,nt,decim,kw", [
+    (12, 29, 10, 5, 77, 1, {"dft_chunk": 32}),     # 32 rows: four per block, an odd column count
+    (26, 90, 5, 7, 70, 1, {}),                     # uneven rows, one chunk
+    (101, 101, 20, 12, 150, 1, {"dft_chunk": 64}), # the small model's grid, several chunks
+    (101, 101, 20, 3, 131, 4, {"dft_chunk": 32}),  # band-limited, decimated
+    (37, 64, 0, 9, 100, 7, {"batch_receivers": 4, "dft_chunk": 32}),  # no sponge, ragged batches
+    (215, 230, 20, 4, 60, 1, {}),                  # (few receivers on a larger grid: the per-step kernel)
+    (215, 230, 20, 20, 60, 1, {}),                 # the largest slabs: coefficients from global memory
+])
+def test_cluster_solver_equals_per_step_kernel(nz, nx, nsponge, nrec, nt, decim, kw):
+    """Small grids: the cluster solver's transforms are the per-step kernel's bit for bit (the same
+    operations per point in the same order)."""
+    import torch
+    from paper_2512_16642_gb300 import egh
+
+    rng = np.random.default_rng(nz + nx)
+    v = torch.from_numpy((2000.0 + 500.0 * rng.random((nz, nx))).astype(np.float32)).cuda()
+    ix = np.linspace(0, nx - 1, nrec).round().astype(np.int32)
+    iz = (np.arange(nrec) * 3 % nz).astype(np.int32)
+    t = np.arange(40) * 1e-3 - 0.02
+    a = (np.pi * 30.0 * t) ** 2
+    wav = ((1 - 2 * a) * np.exp(-a)).astype(np.float32)
+    out = {}
+    for fk in (0, 2):
+        with egh.Context(nz, nx, 10.0, 10.0, nsponge, 1e-3 if nsponge else 0.5, 1e-3, nt, iz, ix,
+                         np.array([12.0, 25.0]), fd_kernel=fk, **kw) as ctx:
+            for _ in range(2):  # again on used slots
+                if decim == 1:
+                    ctx.green(v)
+                else:
+                    ctx.green_bandlimited(v, wav, decim)
+            out[fk] = ctx.get_green()
+            assert ctx.stats()["fd_kernel"] == (3 if fk == 0 and (nz, nrec) != (215, 4) else 2)
+    assert np.array_equal(out[0], out[2])
