@@ -884,16 +884,14 @@ egh_status green_run(egh_ctx* ctx, const float* vel, cudaStream_t stream, const 
           CK(launch_inject(slot(ctx, 1), L.F, ctx->rec_pts + b0, ctx->coef, nb, wav ? wav[0] : 1.0f,
                            src_scale, L.org, so, fs));
       }
-      // levels that still take a wavelet sample: a step, then the injection, launched directly
+      // levels that still take a wavelet sample: steps with the injection, launched directly
       const int ta = std::max(t0, 2);
       // (the cluster solver takes them itself)
       const int tw = wav && ctx->fd_kernel != 3 ? std::max(ta, std::min(t1, nw + 1)) : ta;
       for (int t = ta; t < tw; ++t) {
-        const SnapOut so = level_snap(ctx, t, t0, sbase, D);
+        const FdAux aux{ctx->rec_pts + b0, nb, wav[t - 1], src_scale, nullptr, 0, nullptr, 0, 0};
         CK(launch_fd_step(slot(ctx, t - 1), slot(ctx, t - 2), slot(ctx, t), ctx->coef, L, ctx->S, np,
-                          so, fs, ctx->fd_tz));
-        CK(launch_inject(slot(ctx, t), L.F, ctx->rec_pts + b0, ctx->coef, nb, wav[t - 1], src_scale,
-                         L.org, so, fs));
+                          level_snap(ctx, t, t0, sbase, D), fs, ctx->fd_tz, &aux));
       }
       if (ctx->fd_kernel == 1) {
         if (tw < t1) {
@@ -1363,16 +1361,19 @@ egh_status egh_forward(egh_ctx* ctx, const float* vel, int32_t nsrc, const int32
     float* tr = dout + (size_t)b0 * nrec * nt;
     CK(cudaMemsetAsync(slot(ctx, 0), 0, (size_t)np * L.F * sizeof(float2), stream));
     CK(cudaMemsetAsync(slot(ctx, 1), 0, (size_t)np * L.F * sizeof(float2), stream));
+    // level 0 is zero and level 1 the first sample; step n computes level n + 1, adds its sample and
+    // records level n; the last level is recorded on its own
+    const int tz = ctx->fd_tz ? ctx->fd_tz : fd_rows_one_wave(L, np);
     CK(launch_record(slot(ctx, 0), L.F, ctx->rec_pts, nrec, nb, tr, nt, 0, stream));
-    for (int n = 0; n + 1 < nt; ++n) {
-      if (n > 0)
-        CK(launch_fd_step(slot(ctx, n), slot(ctx, n - 1), slot(ctx, n + 1), ctx->coef, L, ctx->S,
-                          np, none, stream, ctx->fd_tz));
-      if (wavelet[n] != 0.f)
-        CK(launch_inject(slot(ctx, n + 1), L.F, d_sp + b0, ctx->coef, nb, wavelet[n], scale, L.org,
-                         none, stream));
-      CK(launch_record(slot(ctx, n + 1), L.F, ctx->rec_pts, nrec, nb, tr, nt, n + 1, stream));
+    if (nt > 1 && wavelet[0] != 0.f)
+      CK(launch_inject(slot(ctx, 1), L.F, d_sp + b0, ctx->coef, nb, wavelet[0], scale, L.org, none, stream));
+    for (int n = 1; n + 1 < nt; ++n) {
+      const FdAux aux{wavelet[n] != 0.f ? d_sp + b0 : nullptr, nb, wavelet[n], scale, ctx->rec_pts, nrec, tr,
+                      nt, n};
+      CK(launch_fd_step(slot(ctx, n), slot(ctx, n - 1), slot(ctx, n + 1), ctx->coef, L, ctx->S, np, none,
+                        stream, tz, &aux));
     }
+    if (nt > 1) CK(launch_record(slot(ctx, nt - 1), L.F, ctx->rec_pts, nrec, nb, tr, nt, nt - 1, stream));
   }
   if (!dev_out) CK(cudaMemcpyAsync(data, dout, nbytes, cudaMemcpyDeviceToHost, stream));
   CK(cudaStreamSynchronize(stream));

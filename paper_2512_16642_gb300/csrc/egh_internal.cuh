@@ -62,10 +62,21 @@ struct SnapOut {
 cudaError_t launch_check_velocity(const float* vel, long long n, float* d_vmax_bad, cudaStream_t st);
 cudaError_t launch_build_coef(const float* vel, const Layout& L, double dz, double dx, double dt,
                               double R, const float* d_vmax, float2* coef, cudaStream_t st);
+// What a step does besides: the sample amp into the new level at the points pts (null: none), and the
+// current level's values at rec_pts as sample t of the traces (null: none).
+struct FdAux {
+  const int* pts;
+  int nb;  // receivers (sources) of the batch
+  float amp, scale;
+  const int* rec_pts;
+  int nrec;
+  float* traces;  // [nb][nrec][nt]
+  int nt, t;
+};
 // tz: rows per warp (12, 16, 18, 20, 24 or 32; 0 = default)
 cudaError_t launch_fd_step(const float2* ucur, const float2* uprev, float2* unext,
                            const float2* coef, const Layout& L, const Stencil& S, int npairs,
-                           const SnapOut& so, cudaStream_t st, int tz);
+                           const SnapOut& so, cudaStream_t st, int tz, const FdAux* aux = nullptr);
 int fd_rows_one_wave(const Layout& L, int npairs);
 int fd_rows_per_warp_default();
 cudaError_t fd_prepare(int nf);  // once per context, before any capture

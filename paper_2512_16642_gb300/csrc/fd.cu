@@ -191,16 +191,48 @@ __device__ __forceinline__ float2 lap2(const float2 (&dz)[8], const float2 (&e)[
   return l;
 }
 
+// u[b][p] += c3[p] * amp * scale for receiver b, and its split to the snapshot (see k_inject)
+__device__ __forceinline__ void inject_point(float2* u, long long pstride, int p, int b,
+                                             const float2* __restrict__ coef, float amp, float scale,
+                                             long long org, const SnapOut& so) {
+  float* v = reinterpret_cast<float*>(u + (long long)(b >> 1) * pstride + p) + (b & 1);
+  const float nv = *v + coef[p].y * amp * scale;
+  *v = nv;
+  if (so.lvl) {
+    const __nv_bfloat16 h = __float2bfloat16_rn(nv);
+    const __nv_bfloat16 l = __float2bfloat16_rn(nv - __bfloat162float(h));
+    __nv_bfloat16* s = so.lvl + (long long)b * so.rec + (p - org);
+    s[0] = h;
+    s[so.plane] = l;
+  }
+}
+
 // A CTA holds one warp per receiver pair of the batch (threadIdx.y = pair), all on the same
 // 64-column x TZ-row tile, so the coefficient rows are read from L2 once and served to the other
 // pairs from L1.
 constexpr int FD_MAXPAIRS = 16;
 
-template <int TZ>
+//
+// AUX (modelling, and the wavelet's steps of a band-limited Green stage): the lane that owns a
+// receiver's (source's) point adds the step's wavelet sample to what it has just stored, and one
+// more row of blocks records the current level, so that a step is one launch (three before:
+// modelling of 23 shots 26.6 -> 17.5 ms, a band-limited update 154 -> 147 ms).
+template <int TZ, bool AUX>
 __global__ void __launch_bounds__(32 * FD_MAXPAIRS, EGH_FD_MINB)
     k_fd_step(const float2* __restrict__ ucur, const float2* __restrict__ uprev,
               float2* __restrict__ unext, const float2* __restrict__ coef, int NZ, int NX, int PX,
-              int org, long long pstride, Stencil C, SnapOut so) {
+              int org, long long pstride, Stencil C, SnapOut so, FdAux aux) {
+  if (AUX && blockIdx.y * TZ >= NZ) {  // the recording blocks
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int n = aux.nrec * aux.nb, nthr = gridDim.x * blockDim.x * blockDim.y;
+    for (int i = (blockIdx.x * blockDim.y + threadIdx.y) * blockDim.x + threadIdx.x; i < n; i += nthr) {
+      const int b = i / aux.nrec, r = i % aux.nrec;
+      const float2 v = __ldcg(ucur + (long long)(b >> 1) * pstride + aux.rec_pts[r]);
+      aux.traces[((long long)b * aux.nrec + r) * aux.nt + aux.t] = (b & 1) ? v.y : v.x;
+    }
+    return;
+  }
   // per pair: u^n rows [FD_RING][36], then u^{n-1} rows [FD_UP][32] (a lane reads what it copied)
   extern __shared__ __align__(16) float4 ring_all[];
   float4 (*ring)[36] = reinterpret_cast<float4 (*)[36]>(ring_all + threadIdx.y * FD_WARP4);
@@ -344,6 +376,13 @@ __global__ void __launch_bounds__(32 * FD_MAXPAIRS, EGH_FD_MINB)
     }
   }
   asm volatile("cp.async.wait_all;" ::: "memory");
+  if (AUX && aux.pts)
+    for (int u = 0; u < 2; ++u) {
+      const int b = 2 * pair + u;
+      if (b >= aux.nb) break;
+      const int p = aux.pts[b], z = (p - org) / PX, sx = (p - org) % PX;
+      if (z >= z0 && z < z0 + nrows && (sx >> 1) == xh) inject_point(unext, pstride, p, b, coef, aux.amp, aux.scale, org, so);
+    }
 }
 
 #ifndef EGH_FD_TZDEF
@@ -361,13 +400,13 @@ long long fd_sm_smem(int npairs, int tz) {
     return 0;
   const void* k = nullptr;
   switch (tz) {
-    case 12: k = (const void*)k_fd_step<12>; break;
-    case 16: k = (const void*)k_fd_step<16>; break;
-    case 18: k = (const void*)k_fd_step<18>; break;
-    case 20: k = (const void*)k_fd_step<20>; break;
-    case 24: k = (const void*)k_fd_step<24>; break;
-    case 32: k = (const void*)k_fd_step<32>; break;
-    default: k = (const void*)k_fd_step<EGH_FD_TZDEF>; break;
+    case 12: k = (const void*)k_fd_step<12, false>; break;
+    case 16: k = (const void*)k_fd_step<16, false>; break;
+    case 18: k = (const void*)k_fd_step<18, false>; break;
+    case 20: k = (const void*)k_fd_step<20, false>; break;
+    case 24: k = (const void*)k_fd_step<24, false>; break;
+    case 32: k = (const void*)k_fd_step<32, false>; break;
+    default: k = (const void*)k_fd_step<EGH_FD_TZDEF, false>; break;
   }
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, 32 * npairs, fd_block_smem(npairs)) !=
       cudaSuccess) {
@@ -393,12 +432,12 @@ int fd_rows_one_wave(const Layout& L, int npairs) {
       return false;
     return (long long)(L.PX / 64) * ((L.NZ + tz - 1) / tz) <= (long long)occ * sms;
   };
-  if (fits(k_fd_step<12>, 12)) return 12;
-  if (fits(k_fd_step<16>, 16)) return 16;
-  if (fits(k_fd_step<18>, 18)) return 18;
-  if (fits(k_fd_step<20>, 20)) return 20;
-  if (fits(k_fd_step<24>, 24)) return 24;
-  if (fits(k_fd_step<32>, 32)) return 32;
+  if (fits(k_fd_step<12, false>, 12)) return 12;
+  if (fits(k_fd_step<16, false>, 16)) return 16;
+  if (fits(k_fd_step<18, false>, 18)) return 18;
+  if (fits(k_fd_step<20, false>, 20)) return 20;
+  if (fits(k_fd_step<24, false>, 24)) return 24;
+  if (fits(k_fd_step<32, false>, 32)) return 32;
   return EGH_FD_TZDEF;
 }
 
@@ -407,15 +446,21 @@ int fd_rows_one_wave(const Layout& L, int npairs) {
 cudaError_t fd_prepare(int nf) {
   const int fd_smem = fd_block_smem(FD_MAXPAIRS);
   cudaError_t e;
-  if ((e = cudaFuncSetAttribute(k_fd_step<12>, cudaFuncAttributeMaxDynamicSharedMemorySize, fd_smem))) return e;
-  if ((e = cudaFuncSetAttribute(k_fd_step<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, fd_smem))) return e;
-  if ((e = cudaFuncSetAttribute(k_fd_step<18>, cudaFuncAttributeMaxDynamicSharedMemorySize, fd_smem))) return e;
-  if ((e = cudaFuncSetAttribute(k_fd_step<20>, cudaFuncAttributeMaxDynamicSharedMemorySize, fd_smem))) return e;
-  if ((e = cudaFuncSetAttribute(k_fd_step<24>, cudaFuncAttributeMaxDynamicSharedMemorySize, fd_smem))) return e;
-  if ((e = cudaFuncSetAttribute(k_fd_step<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, fd_smem))) return e;
+  if ((e = cudaFuncSetAttribute(k_fd_step<12, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, fd_smem))) return e;
+  if ((e = cudaFuncSetAttribute(k_fd_step<16, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, fd_smem))) return e;
+  if ((e = cudaFuncSetAttribute(k_fd_step<18, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, fd_smem))) return e;
+  if ((e = cudaFuncSetAttribute(k_fd_step<20, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, fd_smem))) return e;
+  if ((e = cudaFuncSetAttribute(k_fd_step<24, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, fd_smem))) return e;
+  if ((e = cudaFuncSetAttribute(k_fd_step<32, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, fd_smem))) return e;
+  for (const void* f : {(const void*)k_fd_step<12, true>, (const void*)k_fd_step<16, true>, (const void*)k_fd_step<18, true>,
+                        (const void*)k_fd_step<20, true>, (const void*)k_fd_step<24, true>, (const void*)k_fd_step<32, true>})
+    if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, fd_smem)) ||
+        (e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                  (int)cudaSharedmemCarveoutMaxShared)))
+      return e;
   // the FD steps and the transform beside them share each SM's shared memory: ask for all of it
-  for (const void* f : {(const void*)k_fd_step<12>, (const void*)k_fd_step<16>, (const void*)k_fd_step<18>,
-                        (const void*)k_fd_step<20>, (const void*)k_fd_step<24>, (const void*)k_fd_step<32>})
+  for (const void* f : {(const void*)k_fd_step<12, false>, (const void*)k_fd_step<16, false>, (const void*)k_fd_step<18, false>,
+                        (const void*)k_fd_step<20, false>, (const void*)k_fd_step<24, false>, (const void*)k_fd_step<32, false>})
     if ((e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout,
                                   (int)cudaSharedmemCarveoutMaxShared)))
       return e;
@@ -425,7 +470,7 @@ cudaError_t fd_prepare(int nf) {
 
 cudaError_t launch_fd_step(const float2* ucur, const float2* uprev, float2* unext,
                            const float2* coef, const Layout& L, const Stencil& S, int npairs,
-                           const SnapOut& so, cudaStream_t st, int tz) {
+                           const SnapOut& so, cudaStream_t st, int tz, const FdAux* aux) {
   if (L.PX % 64 != 0) return cudaErrorInvalidValue;
   if (tz <= 0) tz = EGH_FD_TZDEF;
   // cumulative weights C_j = sum_{k>=j} c_k of the first-difference form
@@ -459,9 +504,11 @@ cudaError_t launch_fd_step(const float2* ucur, const float2* uprev, float2* unex
   switch (tz) {
 #define EGH_FD_CASE(T)                                                                          \
   case T:                                                                                       \
-    cfg.gridDim = dim3(L.PX / 64, (L.NZ + T - 1) / T);                                           \
-    return cudaLaunchKernelEx(&cfg, k_fd_step<T>, ucur, uprev, unext, coef, L.NZ, L.NX, L.PX,    \
-                              org, L.F, C, so);
+    cfg.gridDim = dim3(L.PX / 64, (L.NZ + T - 1) / T + (aux && aux->traces ? 1 : 0));            \
+    return aux ? cudaLaunchKernelEx(&cfg, k_fd_step<T, true>, ucur, uprev, unext, coef, L.NZ,    \
+                                    L.NX, L.PX, org, L.F, C, so, *aux)                           \
+               : cudaLaunchKernelEx(&cfg, k_fd_step<T, false>, ucur, uprev, unext, coef, L.NZ,   \
+                                    L.NX, L.PX, org, L.F, C, so, FdAux{});
     EGH_FD_CASE(12)
     EGH_FD_CASE(16)
     EGH_FD_CASE(18)
@@ -485,18 +532,7 @@ __global__ void k_inject(float2* __restrict__ u, long long pstride, const int* _
                          const float2* __restrict__ coef, int nb, float amp, float scale,
                          long long org, SnapOut so) {
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= nb) return;
-  const int p = pts[b];
-  float* v = reinterpret_cast<float*>(u + (long long)(b >> 1) * pstride + p) + (b & 1);
-  const float nv = *v + coef[p].y * amp * scale;
-  *v = nv;
-  if (so.lvl) {
-    const __nv_bfloat16 h = __float2bfloat16_rn(nv);
-    const __nv_bfloat16 l = __float2bfloat16_rn(nv - __bfloat162float(h));
-    __nv_bfloat16* s = so.lvl + (long long)b * so.rec + (p - org);
-    s[0] = h;
-    s[so.plane] = l;
-  }
+  if (b < nb) inject_point(u, pstride, pts[b], b, coef, amp, scale, org, so);
 }
 
 cudaError_t launch_inject(float2* u, long long pstride, const int* pts, const float2* coef, int nb,
