@@ -439,72 +439,135 @@ cudaError_t launch_inv_power(const float2* Ph, int n, int nf, double* lam, cudaS
   return cudaGetLastError();
 }
 
-// Largest eigenvalue of each Hermitian H_k by power iteration (fixed 300 iterations, Rayleigh
-// quotient), one block per frequency; d_lmax[k].
-constexpr int PI_ITERS = 300;
+// Largest eigenvalue of each Hermitian H_k by power iteration in FP64 (fixed 300 iterations, Rayleigh
+// quotient of the last), one cluster of blocks per matrix as k_inv_power: the blocks' rows of H_k in
+// shared memory (as doubles where they fit, which saves the conversions), eight lanes per row, the
+// vector handed round through distributed shared memory, the norm taken by one thread.  Bound by the
+// FP64 rate, two lanes a cycle and SM: one block per matrix left it to one SM each and every thread
+// took the root and the quotient, 26 matrices of 100 rows 10.0 ms, a band-limited update of 139 ms was
+// 147 ms.
+constexpr int PI_ITERS = 300, LM_THREADS = 256, LM_L = 8;  // lanes per row
 
-__global__ void k_lambda_max(const float2* __restrict__ Qh, int n, double* d_lmax) {
-  extern __shared__ double sv[];  // v: 2n doubles, y: 2n doubles
-  __shared__ double red[256];
-  const int k = blockIdx.x;
-  const float2* A = Qh + (long long)k * n * n;
-  double* v = sv;
-  double* y = sv + 2 * n;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    v[2 * i] = 1.0 + 0.01 * (i % 7);
-    v[2 * i + 1] = 0.0;
+template <typename T>  // float2 or double2: the rows in shared memory
+__global__ void __cluster_dims__(IP_CL, 1, 1) __launch_bounds__(LM_THREADS)
+    k_lambda_max(const float2* __restrict__ Qh, int n, int cached, double* d_lmax) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
+  extern __shared__ __align__(16) double2 lv[];  // v[2][n], then `cached` rows of H
+  constexpr int NW = LM_THREADS / 32;
+  __shared__ double wred[3][NW];
+  __shared__ double part[2][3][IP_CL];  // the blocks' partial sums, by iteration parity
+  __shared__ double inv_s;
+  const int rank = (int)cluster.block_rank(), tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const float2* A = Qh + (long long)(blockIdx.x / IP_CL) * n * n;
+  const int r0 = (int)((long long)n * rank / IP_CL), r1 = (int)((long long)n * (rank + 1) / IP_CL);
+  const int nr = r1 - r0, nc = min(nr, cached);
+  T* rows = reinterpret_cast<T*>(lv + 2 * n);
+  for (int e = tid; e < nc * n; e += LM_THREADS) {
+    const float2 a = A[(long long)r0 * n + e];
+    rows[e] = T{a.x, a.y};
   }
-  __syncthreads();
-  double lam = 0.0;
+  for (int i = tid; i < n; i += LM_THREADS) lv[i] = make_double2(1.0 + 0.01 * (i % 7), 0.0);
+  double inv = 1.0, lam = 0.0;
+  const int g = tid / LM_L, l = tid % LM_L;
+  cluster.sync();  // every block of the cluster runs before its shared memory is written
   for (int it = 0; it < PI_ITERS; ++it) {
-    // y = A v
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    const double2* v = lv + (it & 1) * n;
+    double2* vn = lv + ((it & 1) ^ 1) * n;
+    const bool last = it == PI_ITERS - 1;
+    double yy = 0.0, num = 0.0, den = 0.0;
+    for (int rb = warp * (32 / LM_L); rb < nr; rb += LM_THREADS / LM_L) {  // warp-uniform
+      const int r = rb + (g & (32 / LM_L - 1));
       double re = 0.0, im = 0.0;
-      for (int j = 0; j < n; ++j) {
-        const float2 a = A[(long long)i * n + j];
-        re += a.x * v[2 * j] - a.y * v[2 * j + 1];
-        im += a.x * v[2 * j + 1] + a.y * v[2 * j];
+      if (r < nc) {
+        const T* row = rows + (size_t)r * n;
+        for (int j = l; j < n; j += LM_L) {
+          const T a = row[j];
+          const double2 b = v[j];
+          re = fma((double)a.x, b.x, fma(-(double)a.y, b.y, re));
+          im = fma((double)a.x, b.y, fma((double)a.y, b.x, im));
+        }
+      } else if (r < nr) {
+        const float2* row = A + (long long)(r0 + r) * n;
+        for (int j = l; j < n; j += LM_L) {
+          const float2 a = row[j];
+          const double2 b = v[j];
+          re = fma((double)a.x, b.x, fma(-(double)a.y, b.y, re));
+          im = fma((double)a.x, b.y, fma((double)a.y, b.x, im));
+        }
       }
-      y[2 * i] = re;
-      y[2 * i + 1] = im;
+      for (int o = LM_L / 2; o > 0; o >>= 1) {
+        re += __shfl_xor_sync(0xffffffffu, re, o);
+        im += __shfl_xor_sync(0xffffffffu, im, o);
+      }
+      if (r < nr) {
+        re *= inv;  // v holds the unscaled product of the iteration before
+        im *= inv;
+        if (l == 0) {
+          yy = fma(re, re, fma(im, im, yy));
+          if (last) {  // Rayleigh quotient v^H y / v^H v
+            const double2 x = make_double2(v[r0 + r].x * inv, v[r0 + r].y * inv);
+            num = fma(x.x, re, fma(x.y, im, num));
+            den = fma(x.x, x.x, fma(x.y, x.y, den));
+          }
+        }
+        cluster.map_shared_rank(vn, l)[r0 + r] = make_double2(re, im);  // lane l to block l
+      }
+    }
+    for (int o = 16; o >= LM_L; o >>= 1) {  // the rows' first lanes
+      yy += __shfl_xor_sync(0xffffffffu, yy, o);
+      if (last) {
+        num += __shfl_xor_sync(0xffffffffu, num, o);
+        den += __shfl_xor_sync(0xffffffffu, den, o);
+      }
+    }
+    if (lane == 0) {
+      wred[0][warp] = yy;
+      wred[1][warp] = num;
+      wred[2][warp] = den;
     }
     __syncthreads();
-    // Rayleigh quotient v^H y / v^H v and the norm of y
-    double num = 0.0, den = 0.0, yy = 0.0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-      num += v[2 * i] * y[2 * i] + v[2 * i + 1] * y[2 * i + 1];
-      den += v[2 * i] * v[2 * i] + v[2 * i + 1] * v[2 * i + 1];
-      yy += y[2 * i] * y[2 * i] + y[2 * i + 1] * y[2 * i + 1];
+    if (tid < 3 * IP_CL && (last || tid < IP_CL)) {
+      const int q = tid / IP_CL, to = tid % IP_CL;
+      double s = 0.0;
+      for (int w = 0; w < NW; ++w) s += wred[q][w];
+      cluster.map_shared_rank(&part[it & 1][0][0], to)[q * IP_CL + rank] = s;
     }
-    double vals[3] = {num, den, yy};
-    for (int q = 0; q < 3; ++q) {
-      red[threadIdx.x] = vals[q];
-      __syncthreads();
-      for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-        __syncthreads();
+    cluster.sync();
+    if (tid == 0) {
+      double s = 0.0;
+      for (int b = 0; b < IP_CL; ++b) s += part[it & 1][0][b];
+      inv_s = s > 0.0 ? 1.0 / sqrt(s) : 0.0;
+      if (last) {
+        double sn = 0.0, sd = 0.0;
+        for (int b = 0; b < IP_CL; ++b) {
+          sn += part[it & 1][1][b];
+          sd += part[it & 1][2][b];
+        }
+        lam = sd > 0.0 ? sn / sd : 0.0;
       }
-      vals[q] = red[0];
-      __syncthreads();
     }
-    lam = vals[1] > 0.0 ? vals[0] / vals[1] : 0.0;
-    const double inv = vals[2] > 0.0 ? 1.0 / sqrt(vals[2]) : 0.0;
-    for (int i = threadIdx.x; i < 2 * n; i += blockDim.x) v[i] = y[i] * inv;
     __syncthreads();
+    inv = inv_s;
   }
-  if (threadIdx.x == 0) d_lmax[k] = lam;
+  if (rank == 0 && tid == 0) d_lmax[blockIdx.x / IP_CL] = lam;
 }
 
 cudaError_t launch_lambda_max(const float2* Qh, int nrec, int nf, double* d_lmax,
                               cudaStream_t st) {
-  const size_t smem = sizeof(double) * 4 * (size_t)nrec;
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(k_lambda_max, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-    if (e != cudaSuccess) return e;
-  }
+  static_assert(LM_L == IP_CL, "lane l of a row's group writes to block l");
+  const size_t vec = 2 * sizeof(double2) * (size_t)nrec, cap = 200 * 1024;
+  const int share = (nrec + IP_CL - 1) / IP_CL;
+  const bool dbl = vec + sizeof(double2) * (size_t)share * nrec <= cap;
+  const size_t el = dbl ? sizeof(double2) : sizeof(float2);
+  const int cached =
+      (int)std::min<size_t>((size_t)share, vec < cap ? (cap - vec) / (el * (size_t)nrec) : 0);
+  const size_t smem = vec + el * (size_t)cached * nrec;
+  auto kern = dbl ? k_lambda_max<double2> : k_lambda_max<float2>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
   count_launches(1);
-  k_lambda_max<<<nf, 256, smem, st>>>(Qh, nrec, d_lmax);
+  kern<<<nf * IP_CL, LM_THREADS, smem, st>>>(Qh, nrec, cached, d_lmax);
   return cudaGetLastError();
 }
 
