@@ -1798,11 +1798,11 @@ size_t synth_tma_smem(int kc) {
   return 1024 + 2 * (size_t)kc * SC_CH + 2 * (size_t)SC_B + 8 * (size_t)sp_nstg(kc) * 4096;
 }
 
-template <int KC>
+template <int KC, bool TMA>
 __global__ void __launch_bounds__(SP_EPI + 32, 1)
-    k_synth_tma(const __grid_constant__ CUtensorMap tm_out, const float2* __restrict__ Dh, int nrec,
-                int ld, int s0, int nf, const float* __restrict__ w,
-                const unsigned char* __restrict__ tws, int nt_d, int ntr,
+    k_synth_tma(const __grid_constant__ CUtensorMap tm_out, float* __restrict__ mult,
+                const float2* __restrict__ Dh, int nrec, int ld, int s0, int nf,
+                const float* __restrict__ w, const unsigned char* __restrict__ tws, int nt_d, int ntr,
                 const unsigned char* __restrict__ aimg, int* __restrict__ err) {
   constexpr int SN = sc_n(KC);         // samples per unit (MMA N)
   constexpr unsigned SA = KC * SC_CH;  // one A plane
@@ -1976,7 +1976,7 @@ __global__ void __launch_bounds__(SP_EPI + 32, 1)
       for (int c0 = 0; c0 < SN / 2; c0 += 32) {
         float v[32];
         tc::tmem_ld32(base + (unsigned)c0, v);
-        if (cnt >= NSTG) {  // the staging tile's previous store has read it
+        if (TMA && cnt >= NSTG) {  // the staging tile's previous store has read it
           if (lane == 0) tc::bulk_wait_read<NSTG - 1>();
           __syncwarp();
         }
@@ -1987,9 +1987,23 @@ __global__ void __launch_bounds__(SP_EPI + 32, 1)
                            sb + lane * 128 + ((k ^ (lane & 7)) << 4)),
                        "f"(v[4 * k]), "f"(v[4 * k + 1]), "f"(v[4 * k + 2]), "f"(v[4 * k + 3])
                        : "memory");
-        tc::fence_proxy_async();
+        if (TMA) tc::fence_proxy_async();
         __syncwarp();
-        if (lane == 0) {
+        if (!TMA) {  // a row of the block per store, 32 adjacent samples
+          const int t = j * SN + hh * (SN / 2) + c0 + lane;
+          const long long q = qt * SC_M + qq * 32;
+          float* out = mult + q * nt_d + t;
+          if (t < nt_d)
+#pragma unroll 8
+            for (int r = 0; r < 32; ++r) {
+              float x;
+              asm volatile("ld.shared.f32 %0, [%1];"
+                           : "=f"(x)
+                           : "r"(sb + r * 128 + (((lane >> 2) ^ (r & 7)) << 4) + (lane & 3) * 4));
+              if (q + r < ntr) __stcs(out + (long long)r * nt_d, x);
+            }
+          __syncwarp();  // the tile has been read before it is filled again
+        } else if (lane == 0) {
           // a box that starts past the last sample or trace writes nothing: not issued (the
           // group is still committed, so that the staging tiles' group count stays in step)
           const int t = j * SN + hh * (SN / 2) + c0, q = (int)(qt * SC_M) + qq * 32;
@@ -2002,7 +2016,7 @@ __global__ void __launch_bounds__(SP_EPI + 32, 1)
       tc::mbar_arrive(tempty(i & 1));
     }
     if (!ok) *fail = 1;
-    if (lane == 0) tc::bulk_wait_all();
+    if (TMA && lane == 0) tc::bulk_wait_all();
   }
   const bool okall = __syncthreads_and(ok) && !*fail;
   if (!okall && tid == 0) atomicExch(err, 1);
@@ -2079,11 +2093,13 @@ cudaError_t launch_synth_tc(const float2* Dh, int nrec, int ns, int ld, int s0, 
   const int kc = sc_kc(nf), sn = sc_n(kc);
   const bool vec = (nt_d & 3) == 0 && (reinterpret_cast<uintptr_t>(mult) & 15) == 0;
   cudaError_t e;
-  if (vec && dev_out && ntr > 0) {
-    // device memory: the persistent kernel with TMA stores, one CTA per SM; its A tiles come
-    // from operand images built first when a scratch buffer of their size is given
-    CUtensorMap tm;
-    if ((e = make_f32_tmap(&tm, mult, ntr, nt_d, 32, 32, true))) return e;
+  if (dev_out && ntr > 0) {
+    // device memory: the persistent kernel, one CTA per SM, with TMA stores where the rows are a
+    // multiple of 16 bytes; its A tiles come from operand images built first when a scratch buffer
+    // of their size is given.  (Rows of other lengths: 161 receivers x 57 sources x 2813 samples,
+    // k_synth_tc, which gathers its A tiles itself, 84 us, this one 34 us.)
+    CUtensorMap tm = {};
+    if (vec && (e = make_f32_tmap(&tm, mult, ntr, nt_d, 32, 32, true))) return e;
     unsigned char* aimg = nullptr;
     if (scratch && scratch_bytes >= synth_operands_bytes(nf, ntr) &&
         (reinterpret_cast<uintptr_t>(scratch) & 15) == 0) {
@@ -2097,7 +2113,8 @@ cudaError_t launch_synth_tc(const float2* Dh, int nrec, int ns, int ld, int s0, 
       if ((e = cudaGetLastError())) return e;
     }
     const size_t smem = synth_tma_smem(kc);
-    auto kern = kc == 1 ? k_synth_tma<1> : k_synth_tma<2>;
+    auto kern = kc == 1 ? (vec ? k_synth_tma<1, true> : k_synth_tma<1, false>)
+                        : (vec ? k_synth_tma<2, true> : k_synth_tma<2, false>);
     if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)))
       return e;
     int dev = 0, sms = 0;
@@ -2106,7 +2123,7 @@ cudaError_t launch_synth_tc(const float2* Dh, int nrec, int ns, int ld, int s0, 
     const long long units = (long long)((ntr + SC_M - 1) / SC_M) * ((nt_d + sn - 1) / sn);
     const int grid = (int)std::min<long long>(units, sms);
     count_launches(1);
-    kern<<<grid, SP_EPI + 32, smem, st>>>(tm, Dh, nrec, ld, s0, nf, w, tws, nt_d, ntr, aimg, err);
+    kern<<<grid, SP_EPI + 32, smem, st>>>(tm, mult, Dh, nrec, ld, s0, nf, w, tws, nt_d, ntr, aimg, err);
     return cudaGetLastError();
   }
   const size_t smem = synth_tc_smem(kc);

@@ -162,3 +162,33 @@ def test_cluster_solver_equals_per_step_kernel(nz, nx, nsponge, nrec, nt, decim,
             out[fk] = ctx.get_green()
             assert ctx.stats()["fd_kernel"] == (3 if fk == 0 and (nz, nrec) != (215, 4) else 2)
     assert np.array_equal(out[0], out[2])
+
+
+@pytest.mark.parametrize("nf", [3, 33, 64])
+@pytest.mark.parametrize("n,ns,nt,off", [(1, 1, 1, 0), (3, 1, 5, 1), (5, 3, 63, 2), (17, 2, 65, 3), (129, 1, 130, 0),
+                                         (43, 3, 1021, 1), (64, 2, 514, 2)])
+def test_ragged_rows(n, ns, nt, off, nf, tmp_path):
+    """Traces that are not a multiple of four samples, in buffers that start 4, 8 or 12 bytes past a
+    16-byte boundary: spectra and multipliers against the 64-bit transform and synthesis (Q = I).
+    Two bf16-pair products in a row: 4e-5 of the multipliers' norm."""
+    import torch
+
+    rng = np.random.default_rng(n * ns + nt)
+    r = rng.standard_normal((ns, n, nt)).astype(np.float32)
+    flat = torch.full((off + r.size + 8,), float("nan"), device="cuda")  # (read past the rows shows)
+    rd = flat[off: off + r.size].view(ns, n, nt)
+    rd.copy_(torch.from_numpy(r))
+    out = torch.full((off + r.size + 8,), 7.0, device="cuda")
+    md = out[off: off + r.size].view(ns, n, nt)
+    with _line_ctx(n, nf, max(nt, 2), 1) as ctx:
+        ctx.prec_for_test = 1
+        _load_set(ctx, np.broadcast_to(np.eye(n, dtype=np.complex64), (nf, n, n)).copy(), tmp_path)
+        ctx.deblur(rd, md)
+        torch.cuda.synchronize()
+        f = ctx.freqs
+    ph = 2 * np.pi * np.mod(f[:, None] * np.arange(nt)[None] * 1e-3, 1.0)
+    X = np.einsum("kt,srt->krs", np.exp(-1j * ph), r.astype(np.float64), optimize=True)
+    w = 2e-3 * np.gradient(f)
+    ref = np.einsum("k,krs,kt->srt", w, X, np.exp(1j * ph), optimize=True).real
+    assert np.linalg.norm(md.cpu().numpy() - ref) <= 4e-5 * np.linalg.norm(ref)
+    assert bool((out[:off] == 7.0).all()) and bool((out[off + r.size:] == 7.0).all())
