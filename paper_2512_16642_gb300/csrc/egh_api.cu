@@ -83,6 +83,7 @@ struct egh_ctx {
   unsigned char* tws_deb = nullptr;  // the synthesis twiddle tiles (tw_len samples)
   float2* Wh = nullptr;  // mixed precision: W = L^{-1} per frequency
   float2* Ph = nullptr;  // mixed precision: Q^{-1} = W^H W per frequency (solves as one product)
+  unsigned char* Pimg = nullptr;  // mixed precision: Ph as operand images of the solve's product
   double* fro2 = nullptr;  // mixed precision: ||Q_k||_F^2 of the last factorisation
   int* kref = nullptr;     // mixed precision: frequencies whose solves are refined (device list)
   int nref = 0;            // their number
@@ -320,7 +321,7 @@ cudaError_t zero_snap_slot(egh_ctx* ctx, int j, cudaStream_t st) {
 }
 
 void free_all(egh_ctx* c) {
-  void* ptrs[] = {c->Ph, c->fro2, c->kref, c->xbuf, c->rflags, c->tws_deb, c->twt_deb, c->twt_bl, c->Wh, c->Dr, c->Rr, c->coef, c->lev, c->snap, c->twt, c->gh, c->ghb, c->part, c->Qh, c->Lh, c->tw, c->w_dev,
+  void* ptrs[] = {c->Ph, c->Pimg, c->fro2, c->kref, c->xbuf, c->rflags, c->tws_deb, c->twt_deb, c->twt_bl, c->Wh, c->Dr, c->Rr, c->coef, c->lev, c->snap, c->twt, c->gh, c->ghb, c->part, c->Qh, c->Lh, c->tw, c->w_dev,
                   c->rec_pts, c->status, c->dsum, c->lmax, c->vchk, c->d_err, c->vel_stage, c->Dh,
                   c->io_in, c->io_out, c->syn_ops, c->trace_ws, c->wav_dev};
   for (void* p : ptrs)
@@ -623,6 +624,7 @@ egh_status egh_create(const egh_config* cfg, egh_ctx** out) {
   if (prec_mixed(ctx->prec)) {
     ALLOC(ctx->Wh, (size_t)c.nfreq * c.nrec * c.nrec * sizeof(float2), "inverse factors");
     ALLOC(ctx->Ph, (size_t)c.nfreq * c.nrec * c.nrec * sizeof(float2), "inverse Hessians");
+    ALLOC(ctx->Pimg, cmm_image_bytes(c.nrec, c.nfreq), "inverse Hessians' operand images");
     ALLOC(ctx->fro2, (size_t)2 * c.nfreq * sizeof(double), "condition estimates");
     ALLOC(ctx->kref, (size_t)c.nfreq * sizeof(int), "refined frequencies");
   }
@@ -1135,6 +1137,7 @@ egh_status egh_factor(egh_ctx* ctx, int32_t* bad_freq, void* stream_) {
   if (ctx->Wh) {
     CK(launch_trtri(ctx->Lh, ctx->nrec, ctx->nf, ctx->Wh, stream));
     CK(launch_gram_inverse(ctx->Wh, ctx->nrec, ctx->nf, ctx->Ph, stream));
+    CK(launch_cmm_images(ctx->Ph, ctx->nrec, ctx->nf, ctx->Pimg, stream));
   }
   if (ctx->Wh) CK(refine_estimates(ctx, stream));
   egh_status rs = refine_fetch(ctx, stream);  // read after the sync
@@ -1231,11 +1234,11 @@ static egh_status deblur_common(egh_ctx* ctx, const float* resid, int32_t ns, in
     // Y = Q^{-1} D, one product on the tensor cores; at the frequencies whose condition bound asks
     // for it, the residual R = D - Q Y to FP64-class accuracy and the correction Y += Q^{-1} R
     float2* Y = ctx->Rr;
-    CK(launch_cmm_tc(ctx->Ph, ctx->nrec, ctx->nf, D, ns, Y, nullptr, ctx->d_err, stream));
+    CK(launch_cmm_tc(ctx->Pimg, ctx->nrec, ctx->nf, D, ns, Y, nullptr, ctx->d_err, stream));
     if (refine) {
       CK(launch_resid(ctx->Qh, ctx->nrec, ctx->nref, Y, D, ns, ctx->Dr,
                       ctx->prec == EGH_PREC_MIXED_FP64, stream, ctx->kref));
-      CK(launch_cmm_tc(ctx->Ph, ctx->nrec, ctx->nref, ctx->Dr, ns, D, ctx->kref, ctx->d_err, stream));
+      CK(launch_cmm_tc(ctx->Pimg, ctx->nrec, ctx->nref, ctx->Dr, ns, D, ctx->kref, ctx->d_err, stream));
       CK(launch_add_correction(Y, D, ntr, ctx->nref, stream, ctx->kref));
     }
     Xs = Y;
@@ -1659,6 +1662,7 @@ static cudaError_t batch_enqueue(egh_batch* b, int threads, cudaStream_t st) {
     if ((e = cudaStreamWaitEvent(s, b->ev_fork, 0))) return e;
     if ((e = launch_trtri(c->Lh, c->nrec, c->nf, c->Wh, s))) return e;
     if ((e = launch_gram_inverse(c->Wh, c->nrec, c->nf, c->Ph, s))) return e;
+    if ((e = launch_cmm_images(c->Ph, c->nrec, c->nf, c->Pimg, s))) return e;
     if ((e = refine_estimates(c, s))) return e;
     if ((e = cudaEventRecord(b->ev_join[i], s))) return e;
     if ((e = cudaStreamWaitEvent(st, b->ev_join[i], 0))) return e;

@@ -213,10 +213,13 @@ cudaError_t launch_trsm(const float2* Lh, int n, int nf, float2* Dh, int ns, cud
 cudaError_t launch_trtri(const float2* Lh, int n, int nf, float2* Wh, cudaStream_t st);
 // Q^{-1}_k = W_k^H W_k (dense) from the inverse factors
 cudaError_t launch_gram_inverse(const float2* Wh, int n, int nf, float2* Ph, cudaStream_t st);
-// C_k = A_k B_k (complex, A_k n x n, B_k and C_k n x ld, row-major; C must not alias B) on the
-// tensor cores with FP32-class products (three-term bf16 splits), for the nk frequencies of the
+// operand images of A_k (n x n complex64 per frequency) for launch_cmm_tc: cmm_image_bytes(n, nf)
+size_t cmm_image_bytes(int n, int nf);
+cudaError_t launch_cmm_images(const float2* A, int n, int nf, unsigned char* img, cudaStream_t st);
+// C_k = A_k B_k (complex, A_k n x n as images, B_k and C_k n x ld, row-major; C must not alias B) on
+// the tensor cores with FP32-class products (three-term bf16 splits), for the nk frequencies of the
 // device list kl (all when null); err: the flag a bounded wait sets (solve_tc.cu)
-cudaError_t launch_cmm_tc(const float2* A, int n, int nk, const float2* B, int ld, float2* C,
+cudaError_t launch_cmm_tc(const unsigned char* Aimg, int n, int nk, const float2* B, int ld, float2* C,
                           const int* kl, int* err, cudaStream_t st);
 // diagonal-Hessian baseline: D_k[r][s] /= Q_k[r][r]
 cudaError_t launch_diag_solve(const float2* Qh, int n, int nf, float2* Dh, int ns, cudaStream_t st);

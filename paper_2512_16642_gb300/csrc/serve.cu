@@ -89,6 +89,7 @@ struct HSet {
   float2 *Qh = nullptr, *Lh = nullptr, *tw = nullptr;
   float2* Wh = nullptr;  // mixed precision: W = L^{-1}
   float2* Ph = nullptr;  // mixed precision: Q^{-1} = W^H W
+  unsigned char* Pimg = nullptr;  // its operand images for the solve's product
   int* kref = nullptr;   // mixed precision: frequencies whose solves are refined (device list)
   int nref = 0;
   unsigned char* twt = nullptr;  // tensor-core transform twiddle tiles (tw_len levels)
@@ -221,12 +222,12 @@ cudaError_t run_batch(Server* sv, Batch* b, const HSet& h, int expire) {
     // residual R = D - Q Y to FP64-class accuracy and the correction Y += Q^{-1} R
     float2* Y = D + dsz;
     float2* R = D + 2 * dsz;
-    if ((e = launch_cmm_tc(h.Ph, h.nrec, h.nf, D, ld, Y, nullptr, err, st))) return e;
+    if ((e = launch_cmm_tc(h.Pimg, h.nrec, h.nf, D, ld, Y, nullptr, err, st))) return e;
     if (h.nref > 0) {
       if ((e = launch_resid(h.Qh, h.nrec, h.nref, Y, D, ld, R, sv->prec == EGH_PREC_MIXED_FP64, st,
                             h.kref)))
         return e;
-      if ((e = launch_cmm_tc(h.Ph, h.nrec, h.nref, R, ld, D, h.kref, err, st))) return e;
+      if ((e = launch_cmm_tc(h.Pimg, h.nrec, h.nref, R, ld, D, h.kref, err, st))) return e;
       if ((e = launch_add_correction(Y, D, (long long)h.nrec * ld, h.nref, st, h.kref))) return e;
     }
     Xs = Y;
@@ -457,6 +458,7 @@ egh_status egh_server_add_set(egh_server* sv, int32_t nrec, int32_t nfreq, const
     cudaFree(d_cond);
     cudaFree(h.kref);
     cudaFree(h.Ph);
+    cudaFree(h.Pimg);
     cudaFree(h.twt);
     cudaFree(h.tws);
     cudaFree(h.Wh);
@@ -493,6 +495,8 @@ egh_status egh_server_add_set(egh_server* sv, int32_t nrec, int32_t nfreq, const
     if (!e) e = launch_trtri(h.Lh, nrec, nfreq, h.Wh, st);
     if (!e) e = cudaMalloc(&h.Ph, qn * sizeof(float2));
     if (!e) e = launch_gram_inverse(h.Wh, nrec, nfreq, h.Ph, st);
+    if (!e) e = cudaMalloc(&h.Pimg, cmm_image_bytes(nrec, nfreq));
+    if (!e) e = launch_cmm_images(h.Ph, nrec, nfreq, h.Pimg, st);
     if (!e) e = cudaMalloc(&d_cond, 2 * nfreq * sizeof(double));
     if (!e) e = launch_fro2(h.Qh, nrec, nfreq, d_cond, st);
     if (!e) e = launch_inv_power(h.Ph, nrec, nfreq, d_cond + nfreq, st);
@@ -690,6 +694,7 @@ void egh_server_destroy(egh_server* sv) {
   for (HSet& h : sv->sets) {
     cudaFree(h.kref);
     cudaFree(h.Ph);
+    cudaFree(h.Pimg);
     cudaFree(h.twt);
     cudaFree(h.tws);
     cudaFree(h.Wh);
