@@ -54,11 +54,12 @@ __device__ __forceinline__ void gram_cp4(unsigned dst, const float* src, bool ok
 //
 // Bound by the FP32 FMA rate: 231 receivers x 26 frequencies x 349 184 points took 75.7 ms with 64 x
 // 64 tiles (4 x 4 entries per thread, two barriers per 16 points and no loads in flight across
-// them), now 67.2 ms: 520 blocks are 1.7 rounds of the 304 that fit, and the sums' fixed ranges of
-// points allow no other split.
+// them), 67.4 ms with these tiles in the order of their index, now 60.4 ms.  520 blocks are 1.7
+// rounds of the 304 that fit, and the sums' fixed ranges of points allow no other split; so the full
+// tiles start first, then those of the last, partial column, then the diagonal with its idle half.
 template <int R>
 __global__ void __launch_bounds__(256, 2)
-    k_gram_partial(const float* __restrict__ gh, int nrec, int nf, long long G, int ntile,
+    k_gram_partial(const float* __restrict__ gh, int nrec, int nf, long long G, int ntile, int nsplit,
                    long long split_len, int px, int xe, float* __restrict__ part) {
   constexpr int T = 16 * R;     // tile edge: 4 x 2 warps of 4 x 8 lanes with R x R entries each
   constexpr int H = R / 4;      // groups of four adjacent rows (columns) per thread
@@ -66,13 +67,13 @@ __global__ void __launch_bounds__(256, 2)
   // the copies, which turn 16 points at a time, then meet two to a bank, and two blocks fit an SM
   extern __shared__ __align__(16) float gsm[];
   float* tot = gsm + GST * 2 * GK * T;
-  const int pair = blockIdx.x, k = blockIdx.y, s = blockIdx.z;
-  int ta = 0, rem = pair;
-  while (rem >= ntile - ta) {
-    rem -= ntile - ta;
-    ++ta;
-  }
-  const int tb = ta + rem;
+  // the tile pair is the slowest index: off the diagonal column by column, then the diagonal
+  const int ks = nf * nsplit, order = blockIdx.x / ks, k = (blockIdx.x - order * ks) % nf,
+            s = (blockIdx.x - order * ks) / nf;
+  int ta = order, tb = 1;
+  while (tb < ntile && ta >= tb) ta -= tb++;
+  if (tb == ntile) tb = ta;
+  const int pair = ta * ntile - ta * (ta - 1) / 2 + (tb - ta);
   const bool diag = ta == tb;  // B is A
   const int rows = 2 * nrec;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -220,9 +221,11 @@ cudaError_t launch_gram_partial(const float* gh, int nrec, int nf, long long G, 
   if ((e = cudaFuncSetAttribute(k_gram_partial<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes(8))) ||
       (e = cudaFuncSetAttribute(k_gram_partial<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes(4))))
     return e;
-  dim3 grid(npairs, nf, splits);
+  const long long blocks = (long long)npairs * nf * splits;
+  if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
   count_launches(1);
-  kern<<<grid, 256, smem, st>>>(gh, nrec, nf, G, nt, split_len, px, (nx + GK - 1) / GK * GK, part);
+  kern<<<(unsigned)blocks, 256, smem, st>>>(gh, nrec, nf, G, nt, splits, split_len, px,
+                                        (nx + GK - 1) / GK * GK, part);
   return cudaGetLastError();
 }
 
@@ -444,8 +447,8 @@ cudaError_t launch_inv_power(const float2* Ph, int n, int nf, double* lam, cudaS
 // shared memory (as doubles where they fit, which saves the conversions), eight lanes per row, the
 // vector handed round through distributed shared memory, the norm taken by one thread.  Bound by the
 // FP64 rate, two lanes a cycle and SM: one block per matrix left it to one SM each and every thread
-// took the root and the quotient, 26 matrices of 100 rows 10.0 ms, a band-limited update of 139 ms was
-// 147 ms.
+// took the root and the quotient (26 matrices of 100 rows 10.0 ms; a band-limited update 147 ms then,
+// 139 ms now).
 constexpr int PI_ITERS = 300, LM_THREADS = 256, LM_L = 8;  // lanes per row
 
 template <typename T>  // float2 or double2: the rows in shared memory
