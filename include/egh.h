@@ -115,9 +115,10 @@ typedef struct {
     const double *freq_hz; /* [nfreq], host */
     int32_t batch_receivers; /* receivers propagated together; 0 = chosen by the library: with
                                 the per-step FD kernel and more than 8 receivers, the first
-                                egh_green times the FD step per receiver for 8, 16 and 32 (at
-                                most nrec) and keeps 16 unless another is 3% faster; else
-                                min(nrec, 16) */
+                                egh_green times the FD steps of all receivers in batches of 8, 16,
+                                32 and min(nrec, 32) and keeps 16 (or nrec, if less) unless another
+                                is 3% faster; with the cluster solver, as many as run at once (at
+                                most 32); else min(nrec, 16) */
     int32_t dft_chunk;       /* levels per transform chunk: 32, 64, ..., 2048; 0 = 512 (the
                                 snapshot ring holds 2 chunks x batch_receivers levels); a
                                 chunk longer than the record is cut to the smallest power of

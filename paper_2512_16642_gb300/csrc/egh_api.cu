@@ -711,53 +711,85 @@ void egh_destroy(egh_ctx* ctx) {
 
 namespace {
 
-// The Green stage.  wav == nullptr: Dirac source (impulse at level 1), every level transformed
-// with the table ctx->twt.  Otherwise the band-limited form: wavelet sample s_n is injected at
-// the receiver into level n + 1, every decim-th level is recorded and transformed with `twt`
-// (which folds in the factor decim and the division by the wavelet's spectrum).
-// Receivers per batch, timed once per context before the ring (sized for the batch) exists: the
-// FD step's time per receiver-step for 8, 16 and 32 receivers (each with its one-wave rows per
-// warp; 24 steps on the state slots, which the run rewrites, best of three passes after a
-// warm-up).  16 is kept unless another is 3% faster per receiver.  The transform's work per
-// receiver does not depend on the batch, and it runs beside the FD steps for every choice.
-egh_status tune_batch(egh_ctx* ctx, cudaStream_t stream) {
-  const Layout& L = ctx->L;
+// Time in ms of 24 FD steps of np receiver pairs with tz rows per warp, with (ring slots 0 .. slots-1)
+// or without snapshots: best of three passes after a warm-up.  As one graph, as the run's chunks are:
+// launched one by one, a step without a programmatic launch costs 2 us more than in the run and one
+// with it nothing, which misled the choice of rows (295x496 grid, 6 receivers: 24 rows at 7.0 us a
+// step taken for faster than 12 rows at 5.4 us).  The run rewrites every state and ring slot it reads.
+egh_status time_fd_steps(egh_ctx* ctx, int np, int tz, int slots, float* best) {
+  constexpr int STEPS = 24;
   cudaStream_t fs = ctx->fdst;
+  CK(cudaStreamBeginCapture(fs, cudaStreamCaptureModeThreadLocal));
+  cudaError_t e = cudaSuccess;
+  for (int t = 2; t < 2 + STEPS && e == cudaSuccess; ++t)
+    e = launch_fd_step(slot(ctx, t - 1), slot(ctx, t - 2), slot(ctx, t), ctx->coef, ctx->L, ctx->S, np,
+                       slots ? snap_slot(ctx, t % slots) : SnapOut{nullptr, 0, 0}, fs, tz);
+  count_launches(-STEPS);  // counted at each replay
+  cudaGraph_t graph = nullptr;
+  const cudaError_t e2 = cudaStreamEndCapture(fs, &graph);
+  if (e == cudaSuccess) e = e2;
+  cudaGraphExec_t exec = nullptr;
+  if (e == cudaSuccess) e = cudaGraphInstantiate(&exec, graph, 0);
+  if (graph) cudaGraphDestroy(graph);
+  *best = 1e30f;
+  for (int rep = 0; rep < 4 && e == cudaSuccess; ++rep) {
+    float ms = 0.f;
+    if ((e = cudaEventRecord(ctx->ev_tune[0], fs)) || (e = cudaGraphLaunch(exec, fs)) ||
+        (e = cudaEventRecord(ctx->ev_tune[1], fs)) || (e = cudaEventSynchronize(ctx->ev_tune[1])) ||
+        (e = cudaEventElapsedTime(&ms, ctx->ev_tune[0], ctx->ev_tune[1])))
+      break;
+    count_launches(STEPS);
+    if (rep > 0) *best = std::min(*best, ms);
+  }
+  if (exec) cudaGraphExecDestroy(exec);
+  if (e != cudaSuccess) return fail(ctx, EGH_ECUDA, std::string("FD step timing: ") + cudaGetErrorString(e));
+  return EGH_OK;
+}
+
+// Receivers per batch, timed once per context before the ring (sized for the batch) exists: the FD
+// steps of all receivers in batches of 8, 16, 32 or all that the state slots hold, the last batch
+// with what is left (each with its one-wave rows per warp).  16 is kept unless another is 3% faster.
+// The transform's work per receiver does not depend on the batch, and it runs beside the FD steps for
+// every choice.  (By the time per receiver
+// alone, 12 receivers ran as 8 and 4: 295x496 grid, 1000 steps, 12.2 ms, now 8.7 ms.)
+egh_status tune_batch(egh_ctx* ctx, cudaStream_t stream) {
   CK(cudaEventRecord(ctx->ev_tune[0], stream));  // after the coefficients
-  CK(cudaStreamWaitEvent(fs, ctx->ev_tune[0], 0));
-  const SnapOut none{nullptr, 0, 0};
+  CK(cudaStreamWaitEvent(ctx->fdst, ctx->ev_tune[0], 0));
+  std::map<int, float> step;  // by pairs
+  egh_status s = EGH_OK;
+  auto time = [&](int b) {
+    const int np = (b + 1) / 2;
+    auto it = step.find(np);
+    if (it != step.end()) return it->second;
+    float ms = 1e30f;
+    if (s == EGH_OK) s = time_fd_steps(ctx, np, fd_rows_one_wave(ctx->L, np), 0, &ms);
+    return step[np] = ms;
+  };
   const int def_b = std::min(ctx->Bcap, 16);
-  float best = 1e30f, def_per = 1e30f;
+  float best = 1e30f, def_ms = 1e30f;
   int best_b = def_b;
-  for (int b : {8, 16, 32}) {
+  for (int b : {8, 16, 32, ctx->Bcap}) {
     if (b > ctx->Bcap) continue;
-    const int np = (b + 1) / 2, tz = fd_rows_one_wave(L, np);
-    float tb = 1e30f;
-    for (int rep = 0; rep < 4; ++rep) {
-      float ms = 0.f;
-      CK(cudaEventRecord(ctx->ev_tune[0], fs));
-      for (int t = 2; t < 26; ++t)
-        CK(launch_fd_step(slot(ctx, t - 1), slot(ctx, t - 2), slot(ctx, t), ctx->coef, L, ctx->S,
-                          np, none, fs, tz));
-      CK(cudaEventRecord(ctx->ev_tune[1], fs));
-      CK(cudaEventSynchronize(ctx->ev_tune[1]));
-      CK(cudaEventElapsedTime(&ms, ctx->ev_tune[0], ctx->ev_tune[1]));
-      if (rep > 0) tb = std::min(tb, ms);
-    }
-    const float per = tb / (float)b;
-    if (per < best) {
-      best = per;
+    const int rest = ctx->nrec % b;
+    const float ms = (float)(ctx->nrec / b) * time(b) + (rest ? time(rest) : 0.f);
+    if (s) return s;
+    if (ms < best) {
+      best = ms;
       best_b = b;
     }
-    if (b == def_b) def_per = per;
+    if (b == def_b) def_ms = ms;
   }
-  ctx->B = best < 0.97f * def_per ? best_b : def_b;
+  ctx->B = best < 0.97f * def_ms ? best_b : def_b;
   ctx->Bp = 2 * ((ctx->B + 1) / 2);
   ctx->st.batch_receivers = ctx->B;
   ctx->tune_B = false;
   return EGH_OK;
 }
 
+// The Green stage.  wav == nullptr: Dirac source (impulse at level 1), every level transformed
+// with the table ctx->twt.  Otherwise the band-limited form: wavelet sample s_n is injected at
+// the receiver into level n + 1, every decim-th level is recorded and transformed with `twt`
+// (which folds in the factor decim and the division by the wavelet's spectrum).
 egh_status green_run(egh_ctx* ctx, const float* vel, cudaStream_t stream, const float* wav, int nw,
                      int decim, const unsigned char* twt) {
   CK(cudaSetDevice(ctx->dev));
@@ -831,30 +863,19 @@ egh_status green_run(egh_ctx* ctx, const float* vel, cudaStream_t stream, const 
   }
   if (ctx->fd_kernel == 2 && ctx->fd_tz == 0) {
     // Rows per warp of the FD step: time each choice on this grid (steps of a full batch that
-    // write their snapshots, as the run does; the run below rewrites every state slot and ring
-    // slot it reads), best of three passes of 24 steps per choice.
+    // write their snapshots, as the run does).
     const int np = (std::min(B, ctx->nrec) + 1) / 2;
     float best = 1e30f, def_ms = 1e30f;
     const int def_tz = fd_rows_one_wave(L, np);
     int best_tz = def_tz;
     for (int tz : {12, 16, 18, 20, 24, 32}) {
-      float tz_best = 1e30f;
-      for (int rep = 0; rep < 4; ++rep) {  // the first pass warms up
-        float ms = 0.f;
-        CK(cudaEventRecord(ctx->ev_tune[0], fs));
-        for (int t = 2; t < 26; ++t)
-          CK(launch_fd_step(slot(ctx, t - 1), slot(ctx, t - 2), slot(ctx, t), ctx->coef, L, ctx->S,
-                            np, snap_slot(ctx, t % (2 * K)), fs, tz));
-        CK(cudaEventRecord(ctx->ev_tune[1], fs));
-        CK(cudaEventSynchronize(ctx->ev_tune[1]));
-        CK(cudaEventElapsedTime(&ms, ctx->ev_tune[0], ctx->ev_tune[1]));
-        if (rep > 0) tz_best = std::min(tz_best, ms);
-      }
-      if (tz_best < best) {
-        best = tz_best;
+      float ms = 0.f;
+      if ((s = time_fd_steps(ctx, np, tz, 2 * K, &ms))) return s;
+      if (ms < best) {
+        best = ms;
         best_tz = tz;
       }
-      if (tz == def_tz) def_ms = tz_best;
+      if (tz == def_tz) def_ms = ms;
     }
     // keep the one-wave choice unless another is clearly faster: the pass runs without the
     // transform beside it, and close calls there have gone either way in the full stage
