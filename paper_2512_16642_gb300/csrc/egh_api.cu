@@ -47,6 +47,7 @@ struct egh_ctx {
   std::vector<double> freqs;
   std::vector<float> wsyn;
   int B = 0, K = 0, splits = 0;
+  bool pad_zero = true;  // the transforms are this context's: zero in the rows' padding columns
   int Bcap = 0;         // receivers the FD state slots hold (>= B)
   bool tune_B = false;  // B is timed on the first egh_green (8, 16 or 32 receivers)
   int fd_tz = 0;  // FD rows per warp of the per-step kernel (0 = library default)
@@ -811,6 +812,7 @@ egh_status green_run(egh_ctx* ctx, const float* vel, cudaStream_t stream, const 
   }
   s = ensure_green_buffers(ctx);
   if (s) return s;
+  ctx->pad_zero = true;
   const Layout& L = ctx->L;
   const int K = ctx->K, B = ctx->B, nt = ctx->nt;
   CK(cudaEventRecord(ctx->ev[0], stream));
@@ -1099,7 +1101,7 @@ egh_status egh_hessian(egh_ctx* ctx, egh_mu_mode mode, double mu_param, double* 
     CK(launch_gram_tc_finish(ctx->part, ctx->nrec, ctx->nf, ctx->splits_tc, ctx->Qh, stream));
   } else {
     CK(launch_gram_partial(ctx->gh, ctx->nrec, ctx->nf, ctx->L.G, ctx->splits, ctx->gram_edge,
-                           ctx->L.PX, ctx->L.NX, ctx->part, stream));
+                           ctx->L.PX, ctx->pad_zero ? ctx->L.NX : ctx->L.PX, ctx->part, stream));
     CK(cudaEventRecord(ctx->ev_gram[1], stream));
     CK(launch_gram_finish(ctx->part, ctx->nrec, ctx->nf, ctx->splits, ctx->gram_edge, ctx->Qh, stream));
   }
@@ -1489,6 +1491,7 @@ egh_status egh_import_green(egh_ctx* ctx, const float* d_in, void* stream_) {
   CK(cudaMemcpyAsync(ctx->gh, d_in, n * sizeof(float), cudaMemcpyDeviceToDevice, stream));
   if (ctx->ghb) CK(launch_gh_to_ghb(ctx->gh, ctx->nrec, ctx->nf, ctx->L.G, ctx->ghb, stream));
   CK(cudaStreamSynchronize(stream));
+  ctx->pad_zero = false;
   ctx->st.pde_solves = 0;
   ctx->st.point_steps = 0;
   ctx->state = ST_GREEN;

@@ -104,7 +104,7 @@ def test_forward_transform(n, ns, nt, nf, tmp_path):
 @pytest.mark.parametrize("nx,nz,gram_splits", [(64, 3, 0), (60, 7, 1), (61, 40, 5), (130, 33, 0)])
 def test_gram_fp32(nrec, nx, nz, gram_splits):
     """FP32 Hessians of imported transforms against the 64-bit Gram: one tile to several of either
-    edge, last panels with few rows, point ranges that begin and end inside a grid row, skipped
+    edge, last panels with few rows, point ranges that begin and end inside a grid row, zero
     padding columns.  FP32 products and sums over at most 4000 points with chains of at most 1024:
     random rounding stays below 1e-6 of the Hessian's norm."""
     import torch
@@ -126,6 +126,33 @@ def test_gram_fp32(nrec, nx, nz, gram_splits):
     for k in range(nf):
         H = g[:, k] @ g[:, k].conj().T
         assert np.linalg.norm(Q[k] - H) <= 1e-6 * np.linalg.norm(H), k
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("nrec", [1, 7, 8, 9, 57, 63, 64, 65, 100, 129, 200])
+def test_gram_of_whole_planes(nrec, precision):
+    """Hessians of imported transforms sum over the whole planes, padding included, for every width of
+    the last panel (one receiver, a multiple of eight, one less and one more) in the first or second
+    half of a block.  Tensor cores: 2^-17 per factor of the bf16 pairs, 2e-5 of the norm with room for
+    the dropped product; FP32 as above."""
+    import torch
+    from paper_2512_16642_gb300 import egh
+
+    nz, nx, nf = 9, 70, 3
+    torch.manual_seed(nrec)
+    ix = np.arange(nrec, dtype=np.int32) % nx
+    with egh.Context(nz, nx, 10.0, 10.0, 4, 0.5, 1e-3, 100, np.zeros(nrec, np.int32), ix,
+                     np.array([5.0, 9.0, 11.0]), precision=precision) as ctx:
+        buf = ctx.transform_buffer(nrec, nf)
+        buf.normal_()
+        ctx.import_green(buf)
+        ctx.hessian(egh.EGH_MU_ABS, 0.0)
+        Q = ctx.get_hessian(False)
+    v = buf.cpu().numpy().astype(np.float64)
+    for k in range(nf):
+        g = v[:, k, 0] + 1j * v[:, k, 1]
+        H = g @ g.conj().T
+        assert np.linalg.norm(Q[k] - H) <= (1e-6, 2e-5)[precision] * np.linalg.norm(H), k
 
 
 @pytest.mark.parametrize("nz,nx,nsponge,nrec,nt,decim,kw", [
