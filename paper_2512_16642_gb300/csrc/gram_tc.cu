@@ -126,7 +126,8 @@ __device__ __forceinline__ void tma_load_5d(unsigned dst, const void* tmap, int 
 // 87 000 points), so the MMAs accumulate into one of two 256-column TMEM buffers for blocks of
 // GC_J stages only, and warps 0..7 (lane quarter w % 4, column half w / 4) drain each finished
 // block into FP32 register totals with round-to-nearest adds while the MMAs fill the other
-// buffer.  Stages of 32 points (48 KB) keep four in the ring, the copies three stages ahead of
+// buffer.  The last panel's columns end with its rows, in the MMA's steps of 16 (7.68 -> 7.56 ms at
+// 231 receivers x 26 frequencies).  Stages of 32 points (48 KB) keep four in the ring, the copies three stages ahead of
 // the MMAs (measured against two 96 KB stages of 64 points: 9.6 -> 8.1 ms at 231 receivers x
 // 26 frequencies).  Every wait is bounded (on expiry: error flag, bounded drain of the copies in
 // flight, TMEM freed, CTA leaves).
@@ -150,7 +151,10 @@ __global__ void __launch_bounds__(288)
   while (ta + 1 < n64 && gram_tc_blocks_before(ta + 1, n64) <= blkid) ++ta;
   const int bp = ta + 2 * (blkid - gram_tc_blocks_before(ta, n64));  // first B panel
   const bool inner = bp == ta;         // the A panel is the first half of the B panels
-  const bool half = bp + 1 >= n64;     // one B panel only: N = 128
+  const bool half = bp + 1 >= n64;     // one B panel only
+  // columns: those of rows that exist, in the MMA's steps of 16 (the last panel is seldom full)
+  const int last = (2 * nrec - GC_M * (n64 - 1) + 15) & ~15;
+  const int N = half ? last : bp + 2 == n64 ? GC_M + last : GC_N;
   const long long p0 = (long long)sp * split_len;
   const long long p1 = min(G, p0 + split_len);
   const int nst = p1 > p0 ? (int)((p1 - p0 + GC_K - 1) / GC_K) : 0;
@@ -177,7 +181,7 @@ __global__ void __launch_bounds__(288)
   auto stage_addr = [&](int b) { return tc::smem_u32(sm + (size_t)b * GC_STAGE); };
   if (warp == 8) {
     if (tid == 256) {
-      const unsigned idesc = tc::idesc_bf16(GC_M, half ? GC_N / 2 : GC_N, 0, 0);
+      const unsigned idesc = tc::idesc_bf16(GC_M, N, 0, 0);
       auto issue = [&](int s) {
         const int b = s % GC_ST;
         const int stg = (int)(p0 / GC_P) + s / (GC_P / GC_K);  // 64-point block
@@ -254,7 +258,7 @@ __global__ void __launch_bounds__(288)
 #pragma unroll
     for (int c = 0; c < 128; ++c) tot[c] = 0.f;
     bool ok = true;
-    const bool idle = half && h == 1;  // columns past the last panel: nothing to drain
+    const int nc = min(128, N - h * 128);  // this warp's columns (none: nothing to drain)
     for (int blk = 0; blk < nblk; ++blk) {
       const bool got = tc::mbar_wait(blockdone(blk & 1), (blk >> 1) & 1);
       if (!__all_sync(0xffffffffu, got && !fail)) {  // warp-uniform: TMEM loads are collective
@@ -262,11 +266,11 @@ __global__ void __launch_bounds__(288)
         break;
       }
       tc::tc_fence_after();
-      if (!idle) {
-        const unsigned base =
-            tmem + ((unsigned)(q * 32) << 16) + (unsigned)((blk & 1) * GC_N + h * 128);
+      const unsigned base =
+          tmem + ((unsigned)(q * 32) << 16) + (unsigned)((blk & 1) * GC_N + h * 128);
 #pragma unroll
-        for (int c0 = 0; c0 < 128; c0 += 32) {
+      for (int c0 = 0; c0 < 128; c0 += 32) {
+        if (c0 < nc) {
           float v[32];
           tc::tmem_ld32(base + (unsigned)c0, v);
 #pragma unroll
@@ -276,15 +280,16 @@ __global__ void __launch_bounds__(288)
       tc::tc_fence_before();
       tc::mbar_arrive(drained(blk & 1));
     }
-    if (ok && !fail && !idle) {
+    if (ok && !fail) {
       const int row = q * 32 + (tid & 31);
       float* out = part +
                    (((long long)sp * nf + k) * gram_tc_blocks(nrec) + blkid) * (GC_M * GC_N) +
                    (long long)row * GC_N + h * 128;
 #pragma unroll
       for (int i = 0; i < 128; i += 4)
-        *reinterpret_cast<float4*>(out + i) = make_float4(tot[i], tot[i + 1], tot[i + 2], tot[i + 3]);
-    } else if (!(ok && !fail) && (tid & 31) == 0) {
+        if (i < nc)
+          *reinterpret_cast<float4*>(out + i) = make_float4(tot[i], tot[i + 1], tot[i + 2], tot[i + 3]);
+    } else if ((tid & 31) == 0) {
       atomicExch(err, 1);
     }
   }
@@ -318,40 +323,36 @@ cudaError_t launch_gram_tc(const CUtensorMap& tmap, int nrec, int nf, long long 
   return cudaGetLastError();
 }
 
-// C[a][b] summed over splits (in double), read from the block that holds (a, b) or, below the
-// diagonal blocks, (b, a) (C is symmetric).
-__device__ inline double ctc_entry(const float* part, int a, int b, int k, int nf, int n64,
-                                   int nblocks, int splits) {
-  if (a / GC_M > b / GC_M) {
-    const int t = a;
-    a = b;
-    b = t;
-  }
-  const int pa = a / GC_M, pb = b / GC_M;
-  const int blk = gram_tc_blocks_before(pa, n64) + (pb - pa) / 2;
-  const long long off = (long long)(a % GC_M) * GC_N + ((pb - pa) & 1) * GC_M + (b % GC_M);
-  double sum = 0.0;
-  for (int s = 0; s < splits; ++s)
-    sum += part[(((long long)s * nf + k) * nblocks + blk) * (GC_M * GC_N) + off];
-  return sum;
-}
-
+// Q_k from the tiles: entry (i, j), i <= j, from the block that holds row 2i and column 2j of C (the
+// panel of i is not past the panel of j), its four values as two 8-byte loads per split, the splits
+// summed in order in double; (j, i) is its conjugate.  Bound by the tiles' bytes (231 receivers x 26
+// frequencies, 16 splits, with the sum of the diagonal after it: 0.44 ms with every entry read at its
+// own place, half of them down a column, now 0.30 ms).
 __global__ void k_gram_tc_finish(const float* __restrict__ part, int nrec, int nf, int splits,
                                  float2* __restrict__ Qh) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   const int i = blockIdx.y;
   const int k = blockIdx.z;
-  if (j >= nrec) return;
+  if (j >= nrec || j < i) return;
   const int n64 = gram_tc_panels64(nrec), nblocks = gram_tc_blocks(nrec);
-  const int a = min(i, j), b = max(i, j);
-  const double rr = ctc_entry(part, 2 * a, 2 * b, k, nf, n64, nblocks, splits);
-  const double ii = ctc_entry(part, 2 * a + 1, 2 * b + 1, k, nf, n64, nblocks, splits);
-  double im = 0.0;
-  if (a != b)
-    im = ctc_entry(part, 2 * a + 1, 2 * b, k, nf, n64, nblocks, splits) -
-         ctc_entry(part, 2 * a, 2 * b + 1, k, nf, n64, nblocks, splits);
-  // entry (a, b) with a <= b; (b, a) is its conjugate
-  Qh[((long long)k * nrec + i) * nrec + j] = make_float2((float)(rr + ii), (float)(i <= j ? im : -im));
+  const int pa = i / 64, pb = j / 64;
+  const int blk = gram_tc_blocks_before(pa, n64) + (pb - pa) / 2;
+  const float* t = part + ((long long)k * nblocks + blk) * (GC_M * GC_N) + (2 * i % GC_M) * GC_N +
+                   ((pb - pa) & 1) * GC_M + 2 * j % GC_M;
+  const long long step = (long long)nf * nblocks * (GC_M * GC_N);
+  double rr = 0.0, ri = 0.0, ir = 0.0, ii = 0.0;
+#pragma unroll 8
+  for (int s = 0; s < splits; ++s) {
+    const float2 re = __ldcs(reinterpret_cast<const float2*>(t + s * step));
+    const float2 im = __ldcs(reinterpret_cast<const float2*>(t + s * step + GC_N));
+    rr += re.x;
+    ri += re.y;
+    ir += im.x;
+    ii += im.y;
+  }
+  const float re = (float)(rr + ii), im = i == j ? 0.f : (float)(ir - ri);
+  Qh[((long long)k * nrec + i) * nrec + j] = make_float2(re, im);
+  if (i != j) Qh[((long long)k * nrec + j) * nrec + i] = make_float2(re, -im);
 }
 
 cudaError_t launch_gram_tc_finish(const float* part, int nrec, int nf, int splits, float2* Qh,
