@@ -77,8 +77,7 @@ struct egh_ctx {
   CUtensorMap tmap{};                        // TMA map of the snapshot ring (64-byte aligned type)
   int Bp = 0;                                // receivers per snapshot slot (B rounded up to even)
   float *gh = nullptr, *part = nullptr;
-  __nv_bfloat16* ghb = nullptr;              // [nf][G/64][hi/lo][nrec x re/im][64] Gram operands
-  CUtensorMap tmap_ghb{};                    // TMA map of ghb
+  __nv_bfloat16* ghb = nullptr;              // [nf][G/32][hi/lo][nrec x re/im][32] Gram operands
   float2 *Qh = nullptr, *Lh = nullptr, *tw = nullptr;
   unsigned char* twt_deb = nullptr;  // the deblur transform's twiddle tiles (tw_len levels)
   unsigned char* tws_deb = nullptr;  // the synthesis twiddle tiles (tw_len samples)
@@ -362,7 +361,6 @@ egh_status ensure_green_buffers(egh_ctx* ctx, bool with_ring = true) {
                   (size_t)ctx->nrec * ctx->nf * 4 * (size_t)L.G * sizeof(__nv_bfloat16),
                   "bf16 transforms")))
     return s;
-  if (ctx->ghb) CK(make_ghb_tmap(&ctx->tmap_ghb, ctx->ghb, L.G, ctx->nf, ctx->nrec));
   return EGH_OK;
 }
 
@@ -1077,7 +1075,7 @@ egh_status egh_hessian(egh_ctx* ctx, egh_mu_mode mode, double mu_param, double* 
       float ms = 0.f;
       for (int rep = 0; rep < 2; ++rep) {  // the first pass warms up
         CK(cudaEventRecord(ctx->ev_gram[0], stream));
-        CK(launch_gram_tc(ctx->tmap_ghb, ctx->nrec, ctx->nf, ctx->L.G, cand, ctx->part,
+        CK(launch_gram_tc(ctx->ghb, ctx->nrec, ctx->nf, ctx->L.G, cand, ctx->part,
                           ctx->d_err, stream));
         CK(launch_gram_tc_finish(ctx->part, ctx->nrec, ctx->nf, cand, ctx->Qh, stream));
         CK(cudaEventRecord(ctx->ev_gram[1], stream));
@@ -1095,7 +1093,7 @@ egh_status egh_hessian(egh_ctx* ctx, egh_mu_mode mode, double mu_param, double* 
   }
   CK(cudaEventRecord(ctx->ev_gram[0], stream));
   if (prec_mixed(ctx->prec)) {
-    CK(launch_gram_tc(ctx->tmap_ghb, ctx->nrec, ctx->nf, ctx->L.G, ctx->splits_tc, ctx->part,
+    CK(launch_gram_tc(ctx->ghb, ctx->nrec, ctx->nf, ctx->L.G, ctx->splits_tc, ctx->part,
                       ctx->d_err, stream));
     CK(cudaEventRecord(ctx->ev_gram[1], stream));
     CK(launch_gram_tc_finish(ctx->part, ctx->nrec, ctx->nf, ctx->splits_tc, ctx->Qh, stream));

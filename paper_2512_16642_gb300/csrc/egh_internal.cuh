@@ -155,12 +155,11 @@ cudaError_t launch_fd_cluster(const ClGeom& g, float2* lev, int pslot, const Lay
                               const float* wav, int nw, const int* pts, float scale, cudaStream_t st);
 
 // ---- gram_tc.cu -------------------------------------------------------------------------------
-// Gram on the tensor cores from the bf16 hi/lo transforms ghb[nrec][nf][re/im][hi/lo][G].
+// Gram on the tensor cores from the bf16 hi/lo transforms ghb[nf][G/32][hi/lo][nrec x re/im][32].
 __host__ __device__ int gram_tc_blocks(int nrec);
 size_t gram_tc_workspace_floats(int nrec, int nf, int splits);
 int gram_tc_splits(int nrec, int nf, long long G);
-cudaError_t make_ghb_tmap(CUtensorMap* tm, void* base, long long G, int nf, int nrec);
-cudaError_t launch_gram_tc(const CUtensorMap& tmap, int nrec, int nf, long long G, int splits,
+cudaError_t launch_gram_tc(const __nv_bfloat16* ghb, int nrec, int nf, long long G, int splits,
                            float* part, int* err, cudaStream_t st);
 cudaError_t launch_gh_to_ghb(const float* gh, int nrec, int nf, long long G, __nv_bfloat16* ghb,
                              cudaStream_t st);

@@ -769,15 +769,16 @@ __global__ void __launch_bounds__(128, 16)
           const float sum = o[i] + v[i];
           __stcs(g + (long long)c * G, sum);
           if (last) {
-            // the Gram's operands: hi = bf16(g), lo = bf16(g - hi), blocked by 64 points as
-            // [freq][G/64][hi|lo][receiver, re/im][64] (each 64-receiver box is contiguous)
+            // the Gram's operands: hi = bf16(g), lo = bf16(g - hi), blocked by 32 points as
+            // [freq][G/32][hi|lo][receiver, re/im][32], the 16-byte runs of a row swapped as the MMA's
+            // 64-byte swizzle wants them (see gram_tc.cu)
             const __nv_bfloat16 h = __float2bfloat16_rn(sum);
             const __nv_bfloat16 l = __float2bfloat16_rn(sum - __bfloat162float(h));
             const long long rows = 2LL * nrec_all;
-            __nv_bfloat16* qp = ghb + (((long long)(c >> 1) * (G >> 6) + (p >> 6)) * 2 * rows +
-                                       2LL * (rec0 + r) + (c & 1)) * 64 + (p & 63);
+            __nv_bfloat16* qp = ghb + (((long long)(c >> 1) * (G >> 5) + (p >> 5)) * 2 * rows +
+                                       2LL * (rec0 + r) + (c & 1)) * 32 + ((p & 31) ^ ((rec0 + r & 3) << 3));
             qp[0] = h;
-            qp[rows * 64] = l;
+            qp[rows * 32] = l;
           }
         }
       }

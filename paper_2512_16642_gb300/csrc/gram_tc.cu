@@ -9,13 +9,12 @@
 // covering exactly the panel pairs on and above the diagonal, by tcgen05 `kind::f16` MMAs in
 // bf16x3: each entry of M_k is stored by the transform's
 // last chunk as hi = bf16(g), lo = bf16(g - hi), and C = Hi Hi^T + Hi Lo^T + Lo Hi^T accumulates in
-// FP32 in TMEM (the dropped Lo Lo^T and the split are ~2^-17 relative).  Operands arrive by 5-D TMA
-// boxes of 32 points x 64 receivers x re/im that land as 128 rows of 64 bytes in the K-major
-// 64-byte-swizzled layout the MMA reads, so the kernel does no conversion.  The grid
+// FP32 in TMEM (the dropped Lo Lo^T and the split are ~2^-17 relative).  Operands arrive by bulk
+// copies of 32 points x up to 128 receivers x re/im, stored so that they land as rows of 64 bytes in
+// the K-major 64-byte-swizzled layout the MMA reads: the kernel does no conversion.  The grid
 // sum is split into `splits` ranges; each CTA writes its FP32 tile to a workspace and a second
 // kernel adds the splits (in double) and forms Q_k.
-#include <cuda.h>
-#include <cudaTypedefs.h>
+#include <cuda_bf16.h>
 
 #include <algorithm>
 
@@ -26,8 +25,8 @@ namespace egh {
 
 constexpr int GC_M = 128;            // block rows of C (64 receivers x re/im)
 constexpr int GC_N = 256;            // block columns of C (128 receivers x re/im)
-constexpr int GC_P = 64;   // points per operand block of the blocked layout
-constexpr int GC_K = 32;   // points per stage: one 64-byte bf16 row (64-byte swizzle)
+constexpr int GC_P = 64;   // point ranges are multiples of it
+constexpr int GC_K = 32;   // points per stage and block of the layout: 64-byte rows (64-byte swizzle)
 constexpr int GC_ST = 4;   // stages in flight (4 x 48 KB: the copies run three stages ahead)
 constexpr unsigned GC_BOX = 128u * GC_K * 2;  // one operand box: 64 receivers x re/im = 128 rows
 constexpr unsigned GC_STAGE = 6 * GC_BOX;  // A hi, A lo (1 box each), B hi, B lo (2 boxes each)
@@ -53,36 +52,11 @@ size_t gram_tc_workspace_floats(int nrec, int nf, int splits) {
 
 size_t gram_tc_smem() { return 1024 + (size_t)GC_ST * GC_STAGE; }
 
-// Tensor map of the bf16 transforms, blocked by 64 points as
-// ghb[nf][G/64][hi/lo][nrec x re/im][64], for boxes {32 points, 128 rows (64 receivers x re/im),
-// 1 plane, 1 block, 1 frequency} with the 64-byte swizzle: every box is 128 runs of 64 bytes
-// 128 bytes apart (one half of a contiguous 16 KB block).
-cudaError_t make_ghb_tmap(CUtensorMap* tm, void* base, long long G, int nf, int nrec) {
-  static PFN_cuTensorMapEncodeTiled_v12000 enc = nullptr;
-  if (!enc) {
-    cudaDriverEntryPointQueryResult q;
-    void* fn = nullptr;
-    cudaError_t e =
-        cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q);
-    if (e != cudaSuccess) return e;
-    if (q != cudaDriverEntryPointSuccess || !fn) return cudaErrorNotSupported;
-    enc = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
-  }
-  const cuuint64_t rows = 2ull * nrec;
-  const cuuint64_t dims[5] = {(cuuint64_t)GC_P, rows, 2, (cuuint64_t)(G / GC_P), (cuuint64_t)nf};
-  const cuuint64_t str[4] = {GC_P * 2, rows * GC_P * 2, 2 * rows * GC_P * 2,
-                             (cuuint64_t)(G / GC_P) * 2 * rows * GC_P * 2};
-  const cuuint32_t box[5] = {GC_K, 128, 1, 1, 1};
-  const cuuint32_t es[5] = {1, 1, 1, 1, 1};
-  const CUresult r = enc(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, base, dims, str, box, es,
-                         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
-                         CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
-}
-
 // The Gram's bf16 operands from FP32 transforms gh[nrec][nf][re/im][G]: hi = bf16(g),
-// lo = bf16(g - hi), blocked by 64 points as ghb[nf][G/64][hi/lo][nrec x re/im][64] (the layout the
-// transform's last chunk writes, from the same values).
+// lo = bf16(g - hi), blocked by 32 points as ghb[nf][G/32][hi/lo][nrec x re/im][32] (the layout the
+// transform's last chunk writes, from the same values).  Within a row the 16-byte runs are swapped as
+// the MMA's 64-byte swizzle has them (run c of row R at c ^ (R / 2 % 4), R / 2 the receiver), so that a
+// panel's rows are one contiguous run that a bulk copy lands as the operand.
 __global__ void k_gh_to_ghb(const float* __restrict__ gh, int nrec, int nf, long long G,
                             __nv_bfloat16* __restrict__ ghb) {
   const long long total = (long long)nrec * nf * 2 * G;
@@ -93,10 +67,10 @@ __global__ void k_gh_to_ghb(const float* __restrict__ gh, int nrec, int nf, long
     const float v = gh[t];
     const __nv_bfloat16 h = __float2bfloat16_rn(v);
     const __nv_bfloat16 l = __float2bfloat16_rn(v - __bfloat162float(h));
-    __nv_bfloat16* q = ghb + (((c2 >> 1) * (G >> 6) + (p >> 6)) * 2 * rows + 2 * r + (c2 & 1)) * 64 +
-                       (p & 63);
+    __nv_bfloat16* q = ghb + (((c2 >> 1) * (G >> 5) + (p >> 5)) * 2 * rows + 2 * r + (c2 & 1)) * 32 +
+                       ((p & 31) ^ ((r & 3) << 3));
     q[0] = h;
-    q[rows * 64] = l;
+    q[rows * 32] = l;
   }
 }
 
@@ -109,35 +83,30 @@ cudaError_t launch_gh_to_ghb(const float* gh, int nrec, int nf, long long G, __n
   return cudaGetLastError();
 }
 
-__device__ __forceinline__ void tma_load_5d(unsigned dst, const void* tmap, int c0, int c1, int c2,
-                                            int c3, int c4, unsigned bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, "
-      "%3, %4, %5, %6}], [%7];" ::"r"(dst),
-      "l"(tmap), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4), "r"(bar)
-      : "memory");
-}
-
 // One CTA: block (ta, tb) of C at frequency k over points [p0, p1), as M128 x N256 MMAs (each
 // A row group read from shared memory serves 256 columns, which halves the operand traffic per
-// product against square 128 x 128 tiles).  Warp 8 (one thread) issues the copies and the MMAs
-// over a GC_ST-stage ring.  The tensor core's FP32 accumulation of a long sum drifts (its
-// rounding is not round-to-nearest: about 2^-24 relative per accumulation, measured 1e-3 over
+// product against square 128 x 128 tiles).  One thread of warp 8 issues the copies of a
+// GC_ST-stage ring, one of warp 9 the MMAs.  The tensor core's FP32 accumulation of a long sum drifts
+// (its rounding is not round-to-nearest: about 2^-24 relative per accumulation, measured 1e-3 over
 // 87 000 points), so the MMAs accumulate into one of two 256-column TMEM buffers for blocks of
 // GC_J stages only, and warps 0..7 (lane quarter w % 4, column half w / 4) drain each finished
 // block into FP32 register totals with round-to-nearest adds while the MMAs fill the other
-// buffer.  The last panel's columns end with its rows, in the MMA's steps of 16 (7.68 -> 7.56 ms at
-// 231 receivers x 26 frequencies).  Stages of 32 points (48 KB) keep four in the ring, the copies three stages ahead of
-// the MMAs (measured against two 96 KB stages of 64 points: 9.6 -> 8.1 ms at 231 receivers x
-// 26 frequencies).  Every wait is bounded (on expiry: error flag, bounded drain of the copies in
-// flight, TMEM freed, CTA leaves).
+// buffer.  Every wait is bounded (on expiry: error flag, the copies in flight awaited, TMEM freed,
+// CTA leaves).
+//
+// Bound by the MMAs (231 receivers x 26 frequencies: 5.09 ms, 7.6e12 issued flop, 1490 TFLOP/s) and
+// their operands in shared memory beside the copies' writes.  There 7.68 ms with tensor boxes of
+// 64-byte rows and one thread for copies and MMAs; 7.56 with the last panel's columns ending with its
+// rows (in the MMA's steps of 16); 6.69 with the operands stored swizzled and copied as contiguous
+// runs; 5.09 with the copies on a thread of their own, which no MMA issue holds up.  Stages of
+// 32 points (48 KB) keep four in the ring (against two 96 KB stages of 64 points: 9.6 -> 8.1 ms).
 constexpr int GC_J = 8 * (GC_P / GC_K);  // stages per TMEM accumulation block (96 accumulations)
 
 // K-major shared-memory descriptor of the 64-byte swizzle (8-row groups 512 bytes apart)
 __device__ __forceinline__ uint64_t gc_desc(unsigned saddr) { return tc::sdesc_sw64(saddr); }
 
-__global__ void __launch_bounds__(288)
-    k_gram_tc(const __grid_constant__ CUtensorMap tmap, int nrec, long long split_len, long long G,
+__global__ void __launch_bounds__(320)
+    k_gram_tc(const __nv_bfloat16* __restrict__ ghb, int nrec, long long split_len, long long G,
               float* __restrict__ part, int* __restrict__ err) {
   extern __shared__ __align__(1024) unsigned char dsm[];
   unsigned char* sm = dsm + ((1024 - (tc::smem_u32(dsm) & 1023)) & 1023);
@@ -181,37 +150,45 @@ __global__ void __launch_bounds__(288)
   auto stage_addr = [&](int b) { return tc::smem_u32(sm + (size_t)b * GC_STAGE); };
   if (warp == 8) {
     if (tid == 256) {
-      const unsigned idesc = tc::idesc_bf16(GC_M, N, 0, 0);
-      auto issue = [&](int s) {
+      // rows of the panels (the last may be partial; rows of a stage past them stay what they were and
+      // reach no entry that is read)
+      const int rows = 2 * nrec;
+      const unsigned ab = (unsigned)min(GC_M, rows - GC_M * ta) * (GC_K * 2);
+      const unsigned bb = (unsigned)min(GC_N, rows - GC_M * bp) * (GC_K * 2);
+      const long long plane = (long long)rows * GC_K;  // elements per point block and plane
+      const __nv_bfloat16* src = ghb + ((long long)k * (G / GC_K) + p0 / GC_K) * 2 * plane;
+      int s = 0;
+      for (; s < nst; ++s) {
         const int b = s % GC_ST;
-        const int stg = (int)(p0 / GC_P) + s / (GC_P / GC_K);  // 64-point block
-        const int xo = GC_K * (s % (GC_P / GC_K));               // its half (64-byte rows)
-        const unsigned base = stage_addr(b);
-        tc::mbar_expect_tx(full(b), (unsigned)((inner ? 0 : 2) + (half ? 2 : 4)) * GC_BOX);
-        for (int hl = 0; hl < 2; ++hl) {
-          if (!inner) tma_load_5d(base + hl * GC_BOX, &tmap, xo, 2 * 64 * ta, hl, stg, k, full(b));
-          for (int h = 0; h < (half ? 1 : 2); ++h)
-            tma_load_5d(base + (2 + 2 * hl + h) * GC_BOX, &tmap, xo, 2 * 64 * (bp + h), hl, stg, k,
-                        full(b));
+        if (s >= GC_ST && !tc::mbar_wait(empty(b), (s / GC_ST - 1) & 1)) {
+          fail = 1;
+          atomicExch(err, 1);
+          break;
         }
-      };
-      int issued = 0, landed = 0;
+        const unsigned base = stage_addr(b);
+        tc::mbar_expect_tx(full(b), 2 * (bb + (inner ? 0 : ab)));
+        for (int hl = 0; hl < 2; ++hl) {
+          const __nv_bfloat16* q = src + (2LL * s + hl) * plane;
+          if (!inner) tc::bulk_g2s(base + hl * GC_BOX, q + GC_M * GC_K * ta, ab, full(b));
+          tc::bulk_g2s(base + (2 + 2 * hl) * GC_BOX, q + GC_M * GC_K * bp, bb, full(b));
+        }
+      }
+      // no copy outlives the block
+      for (int i = max(0, s - GC_ST); i < s; ++i) tc::mbar_wait(full(i % GC_ST), (i / GC_ST) & 1);
+    }
+    __syncwarp();
+  } else if (warp == 9) {
+    if (tid == 288) {
+      const unsigned idesc = tc::idesc_bf16(GC_M, N, 0, 0);
       bool ok = true;
-      for (; issued < min(nst, GC_ST); ++issued) issue(issued);
-      for (int s = 0; s < nst && ok; ++s) {
+      for (int s = 0; s < nst; ++s) {
         const int b = s % GC_ST;
         const int blk = s / GC_J;
         const bool first = s % GC_J == 0;
         // a block reuses the TMEM buffer of block blk - 2 once the drain warps have read it
-        if (first && blk >= 2 && !tc::mbar_wait(drained(blk & 1), ((blk >> 1) - 1) & 1)) {
-          ok = false;
-          break;
-        }
-        if (!tc::mbar_wait(full(b), (s / GC_ST) & 1)) {
-          ok = false;
-          break;
-        }
-        landed = s + 1;
+        ok = !(first && blk >= 2) || tc::mbar_wait(drained(blk & 1), ((blk >> 1) - 1) & 1);
+        ok = ok && tc::mbar_wait(full(b), (s / GC_ST) & 1);
+        if (!ok) break;
         tc::tc_fence_after();
         const unsigned dt = tmem + (unsigned)((blk & 1) * GC_N);
         const unsigned bh = stage_addr(b) + 2 * GC_BOX, bl = stage_addr(b) + 4 * GC_BOX;
@@ -229,22 +206,10 @@ __global__ void __launch_bounds__(288)
         }
         tc::mma_commit(empty(b));
         if (s % GC_J == GC_J - 1 || s == nst - 1) tc::mma_commit(blockdone(blk & 1));
-        // refill the previous stage's buffer (its MMAs were issued one stage earlier, so the
-        // tensor pipe keeps this stage's MMAs queued while the thread waits for them)
-        if (s >= 1 && issued < nst) {
-          const int pb = (s - 1) % GC_ST;
-          if (!tc::mbar_wait(empty(pb), ((s - 1) / GC_ST) & 1)) {
-            ok = false;
-            break;
-          }
-          issue(issued);
-          ++issued;
-        }
       }
       if (!ok) {
         fail = 1;
         atomicExch(err, 1);
-        for (int s = landed; s < issued; ++s) tc::mbar_wait(full(s % GC_ST), (s / GC_ST) & 1);
         // wake the drain warps: every MMA issued so far completes before these arrivals
         tc::mma_commit(blockdone(0));
         tc::mma_commit(blockdone(1));
@@ -308,7 +273,7 @@ int gram_tc_splits(int nrec, int nf, long long G) {
   return (int)s;
 }
 
-cudaError_t launch_gram_tc(const CUtensorMap& tmap, int nrec, int nf, long long G, int splits,
+cudaError_t launch_gram_tc(const __nv_bfloat16* ghb, int nrec, int nf, long long G, int splits,
                            float* part, int* err, cudaStream_t st) {
   if (G % GC_P != 0 || splits < 1) return cudaErrorInvalidValue;
   long long split_len = (G + splits - 1) / splits;
@@ -318,7 +283,7 @@ cudaError_t launch_gram_tc(const CUtensorMap& tmap, int nrec, int nf, long long 
       cudaFuncSetAttribute(k_gram_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   count_launches(1);
-  k_gram_tc<<<dim3(gram_tc_blocks(nrec), nf, splits), 288, smem, st>>>(tmap, nrec, split_len, G,
+  k_gram_tc<<<dim3(gram_tc_blocks(nrec), nf, splits), 320, smem, st>>>(ghb, nrec, split_len, G,
                                                                        part, err);
   return cudaGetLastError();
 }
