@@ -579,7 +579,7 @@ cudaError_t launch_record(const float2* u, long long pstride, const int* rec_pts
 // The kernel is persistent and small so that it runs BESIDE the FD steps of the next chunk: one
 // CTA per SM (a fixed grid of at most one CTA per SM walks the tiles), 128 threads at 32
 // registers and 66.5 KB of shared memory, which fit next to the two FD CTAs an SM holds (2 x 256
-// threads x 120 registers, 2 x 55 KB).  Launched as a grid of thousands of short CTAs, the
+// threads x at most 120 registers, 2 x 70.7 KB).  Launched as a grid of thousands of short CTAs, the
 // transform's CTAs took whole SMs between FD launches and the FD steps waited for them, so that
 // the two ran one after the other; side by side they share the SMs, and the FD steps, which are
 // bound by issue and latency, lose less than the transform's run time.
