@@ -20,12 +20,14 @@ constexpr int GFLUSH = 128;  // stages accumulated before adding into the runnin
 
 // Tile edge of the FP32 Gram: 128 (8 x 8 entries per thread) or 64 (4 x 4).  The larger tile reads
 // each staged value for twice the products; the smaller one computes less past the last receiver,
-// so it is taken where that is a sixth less (231 receivers: 128; up to 32 receivers: 64).  The
+// so it is taken where that is a third less: up to 32 and from 65 to 96 receivers.  Measured with 64
+// and with 128: 30 receivers 0.92 and 1.19 ms, 85 receivers (0.6 of the tiles' entries with 64) 3.21
+// and 3.49 ms, 150 receivers (0.71) 17.0 and 16.3 ms, 212 receivers (0.78) 19.7 and 17.3 ms.  The
 // warps of a 128-row diagonal tile that lie below the diagonal, a quarter of it, compute nothing.
 int gram_tile_edge(int nrec) {
   const long long n64 = (2LL * nrec + 63) / 64, n128 = (2LL * nrec + 127) / 128;
   const long long a64 = n64 * (n64 + 1) / 2, a128 = n128 * (n128 + 1) / 2 * 4 - n128;
-  return 6 * a64 < 5 * a128 ? 64 : 128;
+  return 3 * a64 < 2 * a128 ? 64 : 128;
 }
 
 __host__ __device__ int gram_tiles(int nrec, int edge) { return (2 * nrec + edge - 1) / edge; }
