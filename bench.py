@@ -295,7 +295,9 @@ def gram_roofline(precision, nr, nf, npts, c, ms, peak, kind):
     G = -(-(NZ * PX) // 256) * 256  # padded point count the Gram sums over
     Nx = NZ * NX
     n64 = -(-nr // 64)
-    issued = n64 * (n64 + 1) / 2 * 128 * 128 * 2 * 3 * G * nf
+    # 128-row panels against every column from their own on, the last panel's to the next 16
+    last = -(-(2 * nr - 128 * (n64 - 1)) // 16) * 16
+    issued = sum(128 * (128 * t + last) for t in range(n64)) * 2 * 3 * G * nf
     alg = 8.0 * nf * nr * nr * Nx * (nr + 1) / (2 * nr)
     alg_tf = alg / (ms * 1e-3) / 1e12
     out = {"kernel": "k_gram_tc (bf16x3 tcgen05 Gram)" if precision == "mixed" else "k_gram_partial (FP32)",
