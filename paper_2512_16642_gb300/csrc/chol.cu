@@ -332,10 +332,9 @@ __global__ void __launch_bounds__(THREADS)
 }
 
 cudaError_t potrf_many_prepare(int nmax) {
-  const int smem = (int)potrf_smem(nmax);
-  cudaError_t e;
-  if ((e = cudaFuncSetAttribute(k_potrf_many<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem))) return e;
-  return cudaFuncSetAttribute(k_potrf_many<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (potrf_smem(nmax) > (size_t)kBlockSmem) return cudaErrorInvalidValue;
+  const cudaError_t e = allow_block_smem<k_potrf_many<256>>();
+  return e ? e : allow_block_smem<k_potrf_many<512>>();
 }
 
 cudaError_t launch_potrf_many(const PotrfItem* items, int count, int nmax, int blocks, int threads,
@@ -353,8 +352,7 @@ cudaError_t launch_potrf_many(const PotrfItem* items, int count, int nmax, int b
 cudaError_t launch_potrf(float2* Lh, int n, int nf, int* status, cudaStream_t st, int piv64) {
   const size_t smem = potrf_smem(n);
   if (smem > 32 * 1024) {  // beside the static 8.2 KB
-    cudaError_t e =
-        cudaFuncSetAttribute(k_potrf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_block_smem<k_potrf>();
     if (e != cudaSuccess) return e;
   }
   count_launches(1);

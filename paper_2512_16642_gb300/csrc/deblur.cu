@@ -951,8 +951,7 @@ __global__ void __launch_bounds__(32 * TS_W)
 cudaError_t launch_trsm(const float2* Lh, int n, int nf, float2* Dh, int ns, cudaStream_t st) {
   const size_t smem = sizeof(float2) * TR_C * (size_t)n;
   if (smem > 24 * 1024) {  // beside 16.5 KB of tiles
-    cudaError_t e =
-        cudaFuncSetAttribute(k_trsm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_block_smem<k_trsm>();
     if (e != cudaSuccess) return e;
   }
   dim3 grid((ns + TR_C - 1) / TR_C, nf);
@@ -1177,7 +1176,7 @@ cudaError_t launch_trtri(const float2* Lh, int n, int nf, float2* Wh, cudaStream
   const size_t smem = four ? 4 * one : one;
   auto kern = four ? k_trtri<4> : k_trtri<1>;
   if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = four ? allow_block_smem<k_trtri<4>>() : allow_block_smem<k_trtri<1>>();
     if (e != cudaSuccess) return e;
   }
   const int cb = four ? 4 : 1, warps = 32 * ((groups + cb - 1) / cb);
@@ -1444,9 +1443,7 @@ cudaError_t launch_resid(const float2* Qh, int n, int nf, const float2* Xh, cons
   count_launches(1);
   if (fp64) {
     const size_t smem = sizeof(float2) * 32 * (size_t)n;
-    if (smem > 48 * 1024 &&
-        (e = cudaFuncSetAttribute(k_resid64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)))
-      return e;
+    if (smem > 48 * 1024 && (e = allow_block_smem<k_resid64>())) return e;
     // enough blocks for every SM: split the rows of each (frequency, source group)
     const int blocks = ((ns + 31) / 32) * nf;
     const int groups = std::max(1, std::min((n + TS_W - 1) / TS_W, (4 * 152 + blocks - 1) / blocks));
@@ -1461,7 +1458,9 @@ cudaError_t launch_resid(const float2* Qh, int n, int nf, const float2* Xh, cons
   auto kern = S == 4 ? k_resid_dot2<4, 8> : S == 2 ? k_resid_dot2<2, 16> : k_resid_dot2<1, 32>;
   const size_t smem = sizeof(float2) * S * (size_t)((n + J - 1) / J * J);
   if (smem > 12 * 1024 &&  // beside up to 33 KB of turned groups
-      (e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)))
+      (e = S == 4   ? allow_block_smem<k_resid_dot2<4, 8>>()
+           : S == 2 ? allow_block_smem<k_resid_dot2<2, 16>>()
+                    : allow_block_smem<k_resid_dot2<1, 32>>()))
     return e;
   kern<<<dim3((ns + S - 1) / S, nf, (n + 32 * RD_W - 1) / (32 * RD_W)), 32 * RD_W, smem, st>>>(
       Qh, n, Xh, Dh, ns, Rh, kl);
@@ -2149,8 +2148,7 @@ cudaError_t launch_synth(const float2* Dh, int nrec, int ns, int ld, int s0, int
   const int ntr = nrec * ns;
   const size_t smem = sizeof(float2) * (size_t)nf * SY_TR + 2 * sizeof(float) * (size_t)nf * SY_TP;
   if (smem > 48 * 1024) {
-    cudaError_t e =
-        cudaFuncSetAttribute(k_synth, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_block_smem<k_synth>();
     if (e != cudaSuccess) return e;
   }
   dim3 grid((nt_d + SY_T - 1) / SY_T, (ntr + SY_TR - 1) / SY_TR);

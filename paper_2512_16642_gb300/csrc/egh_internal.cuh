@@ -19,6 +19,7 @@
 
 #include "egh.h"
 
+#include <atomic>
 #include <complex>
 #include <cstdint>
 #include <string>
@@ -33,6 +34,24 @@ void count_launches(int n);
 long long launches_so_far();
 // Message returned by egh_last_error(NULL) for calls that have no context.
 void set_context_free_error(const std::string& msg);
+
+// Lets kernel K take all the dynamic shared memory a block can have (227 KB with its static part).
+// The limit belongs to the kernel in the whole process, not to a call: a launch that set it to its
+// own size would lower it under another host thread's launch, or under a captured one.  So a kernel
+// whose size differs from call to call has this one value set, whatever the call.
+constexpr int kBlockSmem = 227 * 1024;
+template <auto K>
+cudaError_t allow_block_smem() {
+  static std::atomic<int> dynamic{0};
+  int d = dynamic.load(std::memory_order_relaxed);
+  if (d == 0) {
+    cudaFuncAttributes fa;
+    const cudaError_t e = cudaFuncGetAttributes(&fa, K);
+    if (e != cudaSuccess) return e;
+    dynamic.store(d = kBlockSmem - (int)fa.sharedSizeBytes, std::memory_order_relaxed);
+  }
+  return cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, d);
+}
 
 struct Stencil {
   float cx[4];  // c_k / dx^2, k = 1..4

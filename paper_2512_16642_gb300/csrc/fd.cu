@@ -828,7 +828,7 @@ cudaError_t launch_dft_tc(const CUtensorMap& tmap, const unsigned char* twt, int
       if ((long long)dft_smem_ring(nf, 3) <= fit) nring = 3;
     }
   }
-  if ((e = cudaFuncSetAttribute(k_dft_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) ||
+  if ((e = allow_block_smem<k_dft_tc>()) ||
       (e = cudaFuncSetAttribute(k_dft_tc, cudaFuncAttributePreferredSharedMemoryCarveout,
                                 (int)cudaSharedmemCarveoutMaxShared)))
     return e;

@@ -296,7 +296,8 @@ bool fd_cluster_plan(const Layout& L, ClGeom* out) {
     }
   }
   void* k = g.coef_smem ? kernel_of<true>(g.sr) : kernel_of<false>(g.sr);
-  if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem) != cudaSuccess) {
+  // (no static shared memory; one limit for every grid, as allow_block_smem)
+  if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kBlockSmem) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
@@ -370,7 +371,7 @@ cudaError_t launch_fd_cluster(const ClGeom& g, float2* lev, int pslot, const Lay
     a.C.cx[k] = ax;
   }
   void* k = g.coef_smem ? kernel_of<true>(g.sr) : kernel_of<false>(g.sr);
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem);
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kBlockSmem);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute at;

@@ -446,9 +446,7 @@ bool fd_resident_sr_valid(int sr) {
 cudaError_t fd_resident_prepare(const ResGeom& g, int sr, int np) {
   cudaError_t e;
 #define EGH_RES_ATTR(S)                                                                          \
-  if ((e = cudaFuncSetAttribute(k_fd_resident<S>, cudaFuncAttributeMaxDynamicSharedMemorySize,   \
-                                (int)g.smem)))                                                   \
-    return e;
+  if ((e = allow_block_smem<k_fd_resident<S>>())) return e;
   EGH_RES_ATTR(6)
   EGH_RES_ATTR(8)
   EGH_RES_ATTR(11)

@@ -436,8 +436,7 @@ cudaError_t launch_inv_power(const float2* Ph, int n, int nf, double* lam, cudaS
   const int share = (n + IP_CL - 1) / IP_CL;
   const int cached = (int)std::min<size_t>((size_t)share, vec < cap ? (cap - vec) / (sizeof(float2) * (size_t)n) : 0);
   const size_t smem = vec + sizeof(float2) * (size_t)cached * n;
-  cudaError_t e =
-      cudaFuncSetAttribute(k_inv_power, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t e = allow_block_smem<k_inv_power>();
   if (e != cudaSuccess) return e;
   count_launches(1);
   k_inv_power<<<nf * IP_CL, IP_THREADS, smem, st>>>(Ph, n, cached, lam);
@@ -569,7 +568,7 @@ cudaError_t launch_lambda_max(const float2* Qh, int nrec, int nf, double* d_lmax
       (int)std::min<size_t>((size_t)share, vec < cap ? (cap - vec) / (el * (size_t)nrec) : 0);
   const size_t smem = vec + el * (size_t)cached * nrec;
   auto kern = dbl ? k_lambda_max<double2> : k_lambda_max<float2>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t e = dbl ? allow_block_smem<k_lambda_max<double2>>() : allow_block_smem<k_lambda_max<float2>>();
   if (e != cudaSuccess) return e;
   count_launches(1);
   kern<<<nf * IP_CL, LM_THREADS, smem, st>>>(Qh, nrec, cached, d_lmax);

@@ -1,0 +1,138 @@
+"""What a call may rely on whatever other calls do: contexts of different sizes in different host
+threads and in batches, calls under stream capture, and the digits of the smallest steps."""
+import threading
+
+import numpy as np
+import pytest
+
+from test_kernel_edges import _line_ctx
+
+pytestmark = pytest.mark.gpu
+
+
+def _load_set(ctx, Q, tmp_path, mu=0.05):
+    """Puts given Hessians and their penalty into a mixed-precision context (the set-file format)."""
+    import json
+    import struct
+
+    nf, n, _ = Q.shape
+    h = json.dumps({"format": "egh Hessian set", "version": 1, "nrec": n, "nfreq": nf,
+                    "freq_hz": [float(f) for f in ctx.freqs], "dt": 1e-3, "nt": ctx.nt, "precision": 1,
+                    "mu": mu, "rec_iz": [0] * n, "rec_ix": [int(i) % max(64, n) for i in range(n)]}).encode()
+    p = tmp_path / "set.bin"
+    p.write_bytes(b"EGHQSET1" + struct.pack("<Q", len(h)) + h + Q.tobytes() + Q.tobytes())
+    ctx.load(str(p))
+
+
+def _in_threads(*work):
+    """Runs the functions side by side; the first exception of any is raised."""
+    errors = []
+    start = threading.Barrier(len(work))
+
+    def run(f):
+        try:
+            start.wait()
+            f()
+        except BaseException as e:  # noqa: BLE001
+            errors.append(e)
+
+    threads = [threading.Thread(target=run, args=(f,)) for f in work]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    if errors:
+        raise errors[0]
+
+
+def _random_ctx(n, nf, precision):
+    """A context whose transforms are random numbers: Hessians of n receivers over 4 x 512 points."""
+    from paper_2512_16642_gb300 import egh
+
+    ctx = egh.Context(4, 512, 10.0, 10.0, 0, 0.5, 1e-3, 100, np.zeros(n, np.int32),
+                      np.arange(n, dtype=np.int32), np.linspace(5.0, 40.0, nf), precision=precision)
+    buf = ctx.transform_buffer(n, nf)
+    buf.normal_()
+    ctx.import_green(buf)
+    return ctx
+
+
+def test_threads_with_contexts_of_different_sizes():
+    """Distinct contexts are independent: two host threads build penalties and factors of 161 and 341
+    receivers at the same time, again and again; each gets what it got alone."""
+    import torch
+    from paper_2512_16642_gb300 import egh
+
+    torch.manual_seed(5)
+    ctxs = [_random_ctx(n, 2, 1) for n in (161, 341)]
+    try:
+        alone = []
+        for c in ctxs:
+            mu = c.hessian(egh.EGH_MU_REL_MAXEIG, 1e-2)
+            c.factor()
+            alone.append((mu, c.get_hessian(True), c.get_refinement()[0]))
+
+        def loop(c, want):
+            for _ in range(200):
+                assert c.hessian(egh.EGH_MU_REL_MAXEIG, 1e-2) == want[0]
+                c.factor()
+            assert np.array_equal(c.get_hessian(True), want[1])
+            assert np.array_equal(c.get_refinement()[0], want[2])
+
+        _in_threads(*(lambda c=c, w=w: loop(c, w) for c, w in zip(ctxs, alone)))
+    finally:
+        for c in ctxs:
+            c.close()
+
+
+def test_threads_with_grids_of_different_sizes():
+    """As above for the Green stage of small grids and the creation of contexts beside it."""
+    import torch
+    from paper_2512_16642_gb300 import egh
+
+    grids = [(101, 101), (60, 61), (101, 150)]
+
+    def make(nz, nx):
+        return egh.Context(nz, nx, 10.0, 10.0, 10, 1e-3, 1e-3, 40, np.zeros(4, np.int32),
+                           np.arange(4, dtype=np.int32), np.array([12.0, 25.0]), dft_chunk=32)
+
+    vel = [torch.full(g, 2000.0, device="cuda") for g in grids]
+    alone = []
+    for g, v in zip(grids, vel):
+        with make(*g) as c:
+            c.green(v)
+            alone.append(c.get_green())
+    torch.cuda.synchronize()
+
+    def loop(i):
+        for _ in range(8):
+            with make(*grids[i]) as c:
+                for _ in range(10):
+                    c.green(vel[i])
+                assert np.array_equal(c.get_green(), alone[i])
+
+    _in_threads(*(lambda i=i: loop(i) for i in range(len(grids))))
+
+
+def test_small_batch_after_a_large_one(tmp_path):
+    """A batch of small matrices created after one of large matrices takes nothing from it."""
+    from paper_2512_16642_gb300 import egh
+
+    rng = np.random.default_rng(3)
+    ctxs = []
+    try:
+        for n in (200, 9):
+            A = rng.standard_normal((2, n, 2 * n)) + 1j * rng.standard_normal((2, n, 2 * n))
+            Q = (A @ A.conj().transpose(0, 2, 1) / n + 0.1 * np.eye(n)).astype(np.complex64)
+            c = _line_ctx(n, 2, 100, 1)
+            ctxs.append(c)
+            _load_set(c, Q, tmp_path)
+        single = [c.get_hessian(True) for c in ctxs]
+        with egh.Batch(ctxs[:1]) as big, egh.Batch(ctxs[1:]) as small:
+            big.factor()
+            small.factor()
+        for c, L in zip(ctxs, single):
+            assert np.array_equal(c.get_hessian(True), L)
+    finally:
+        for c in ctxs:
+            c.close()
