@@ -758,6 +758,17 @@ size_t trace_scratch_bytes(int nf, long long ntr, int nt_d) {
   return (size_t)ntile * bpt * N * TT_M * sizeof(float) + (size_t)ntile * (TP_EPI / 32) * sizeof(unsigned);
 }
 
+size_t trace_scratch_most(int nf, int nrec, int nt_d) {
+  const int N = tt_ncomp(nf), nst = (nt_d + TT_K - 1) / TT_K, H = nst >= 2 ? 2 : 1;
+  int dev = 0, sms = 0;
+  if (N > TP_NMAX || cudaGetDevice(&dev) ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev))
+    return 0;
+  const int bpt = tp_tile_blocks(H, nst), ntile = sms / (2 * H);  // (as trace_scratch_bytes)
+  if (bpt <= H || (nrec + TT_M - 1) / TT_M > ntile) return 0;
+  return (size_t)ntile * bpt * N * TT_M * sizeof(float) + (size_t)ntile * (TP_EPI / 32) * sizeof(unsigned);
+}
+
 // Persistent transform: one CTA per SM, at most one per unit.  With two parts per tile the
 // spectra of the call's columns are zeroed first (the parts add into them).
 cudaError_t launch_trace_tma(const float* resid, int ntr, int nt_d, const unsigned char* twt,

@@ -119,7 +119,9 @@ struct egh_ctx {
   size_t Dr_cap = 0, Rr_cap = 0;
   float *io_in = nullptr, *io_out = nullptr;
   size_t io_in_cap = 0, io_out_cap = 0;
-  float* trace_ws = nullptr;  // the forward transform's block sums (calls with few traces)
+  float* trace_ws = nullptr;  // the forward transform's block sums (calls with few traces), grown
+                              // with the twiddle tables: a call of fewer sources than an earlier
+                              // one then allocates nothing, and can be captured
   size_t trace_ws_cap = 0;
   unsigned char* syn_ops = nullptr;  // the synthesis operand images
   size_t syn_ops_cap = 0;
@@ -245,6 +247,9 @@ egh_status ensure_twiddles(egh_ctx* ctx, int len, cudaStream_t stream) {
   if (ctx->tw) CK(cudaFree(ctx->tw));
   if (ctx->twt_deb) CK(cudaFree(ctx->twt_deb));
   if (ctx->tws_deb) CK(cudaFree(ctx->tws_deb));
+  if (ctx->trace_ws) CK(cudaFree(ctx->trace_ws));
+  ctx->trace_ws = nullptr;
+  ctx->trace_ws_cap = 0;
   ctx->tw = nullptr;
   ctx->twt_deb = nullptr;
   ctx->tws_deb = nullptr;
@@ -258,6 +263,9 @@ egh_status ensure_twiddles(egh_ctx* ctx, int len, cudaStream_t stream) {
   const std::vector<unsigned char> u = synth_twiddle_tiles(ctx->freqs, ctx->dt, len);
   if ((s = dalloc(ctx, (void**)&ctx->tws_deb, u.size(), "synthesis twiddle tiles"))) return s;
   CK(cudaMemcpy(ctx->tws_deb, u.data(), u.size(), cudaMemcpyHostToDevice));
+  const size_t sb = trace_scratch_most(ctx->nf, ctx->nrec, len);
+  if (sb && (s = dalloc(ctx, (void**)&ctx->trace_ws, sb, "transform blocks"))) return s;
+  ctx->trace_ws_cap = sb;
   ctx->tw_len = len;
   return EGH_OK;
 }
@@ -1234,9 +1242,6 @@ static egh_status deblur_common(egh_ctx* ctx, const float* resid, int32_t ns, in
   CK(cudaEventRecord(ctx->ev[6], stream));
   const int expire = ctx->expire[2] > 0 ? 1 : 0;
   ctx->expire[2] -= expire;
-  const size_t sb = in_map ? 0 : trace_scratch_bytes(ctx->nf, ntr, nt_d);
-  if (sb && (s = ensure_buf(ctx, (void**)&ctx->trace_ws, &ctx->trace_ws_cap, sb, stream, "transform blocks")))
-    return s;
   CK(launch_trace_dft(din, (int)ntr, nt_d, ctx->nf, ctx->nrec, ns, 0, D, stream,
                       ctx->twt_deb, ctx->d_err, expire, in_map == nullptr, ctx->trace_ws,
                       ctx->trace_ws_cap));

@@ -226,6 +226,8 @@ cudaError_t launch_trace_dft(const float* resid, int ntr, int nt_d, int nf, int 
                              int* err, int expire = 0, bool dev_in = false, void* scratch = nullptr,
                              size_t scratch_bytes = 0);
 size_t trace_scratch_bytes(int nf, long long ntr, int nt_d);
+// the most that any call of at most nt_d levels asks for
+size_t trace_scratch_most(int nf, int nrec, int nt_d);
 cudaError_t launch_trsm(const float2* Lh, int n, int nf, float2* Dh, int ns, cudaStream_t st);
 // W = L^{-1} per frequency
 cudaError_t launch_trtri(const float2* Lh, int n, int nf, float2* Wh, cudaStream_t st);

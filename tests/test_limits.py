@@ -136,3 +136,25 @@ def test_small_batch_after_a_large_one(tmp_path):
     finally:
         for c in ctxs:
             c.close()
+
+
+def test_capture_of_a_smaller_deblur(tmp_path):
+    """After one call on device buffers, calls of fewer sources take no device memory (their workspaces
+    stand), so that they can be captured: the replay gives the bits of the call."""
+    import torch
+
+    n, nf, nt = 129, 26, 2000
+    torch.manual_seed(1)
+    r = torch.randn((60, n, nt), device="cuda")
+    big, one, again = torch.empty_like(r), torch.empty_like(r[:1]), torch.empty_like(r[:1])
+    with _line_ctx(n, nf, nt, 1) as ctx:
+        _load_set(ctx, np.broadcast_to(np.eye(n, dtype=np.complex64), (nf, n, n)).copy(), tmp_path)
+        ctx.deblur(r, big)
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, capture_error_mode="thread_local"):
+            ctx.deblur(r[:1], again)
+        g.replay()
+        ctx.deblur(r[:1], one)
+        torch.cuda.synchronize()
+        assert torch.equal(one, big[:1]) and torch.equal(again, one)
