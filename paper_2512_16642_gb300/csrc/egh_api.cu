@@ -23,6 +23,10 @@ const double kC8[5] = {-205.0 / 72.0, 8.0 / 5.0, -1.0 / 5.0, 8.0 / 315.0, -1.0 /
 // Leapfrog stability bound on vmax dt sqrt(1/dx^2 + 1/dz^2) for that stencil:
 // 2 / sqrt(205/72 + 2 (8/5 + 1/5 + 8/315 + 1/560)) = 0.784; kept with a small margin.
 const double kCflMax = 0.78;
+// Factor of the Green transform's twiddles, taken off again when a total is complete (see k_dft_tc).
+// It leaves totals up to 2^104; a transform, a sum of nt levels of a field that the CFL condition
+// bounds over its source's spectrum, stays far below.
+const double kTransformUp = 16777216.0;
 
 thread_local std::string g_create_error;
 std::atomic<long long> g_launches{0};
@@ -618,7 +622,8 @@ egh_status egh_create(const egh_config* cfg, egh_ctx** out) {
     ALLOC(ctx->xbuf, fd_resident_xbuf_float4(ctx->rg) * sizeof(float4), "FD halo exchange");
     ALLOC(ctx->rflags, sizeof(int) * fd_resident_flags(ctx->rg), "FD step counters");
   }
-  std::vector<unsigned char> twt = dft_twiddle_tiles(ctx->freqs, c.dt, c.nt);
+  const std::vector<std::complex<double>> up(c.nfreq, kTransformUp);
+  std::vector<unsigned char> twt = dft_twiddle_tiles(ctx->freqs, c.dt, c.nt, &up);
   ALLOC(ctx->twt, twt.size(), "twiddle tiles");
   ALLOC(ctx->part,
         std::max(gram_workspace_floats(c.nrec, c.nfreq, ctx->splits, ctx->gram_edge),
@@ -798,7 +803,7 @@ egh_status tune_batch(egh_ctx* ctx, cudaStream_t stream) {
 // the receiver into level n + 1, every decim-th level is recorded and transformed with `twt`
 // (which folds in the factor decim and the division by the wavelet's spectrum).
 egh_status green_run(egh_ctx* ctx, const float* vel, cudaStream_t stream, const float* wav, int nw,
-                     int decim, const unsigned char* twt) {
+                     int decim, const unsigned char* twt, float down) {
   CK(cudaSetDevice(ctx->dev));
   ctx->state = ST_CREATED;
   egh_status s = prepare_model(ctx, vel, stream);
@@ -955,9 +960,9 @@ egh_status green_run(egh_ctx* ctx, const float* vel, cudaStream_t stream, const 
       const bool slim = dft_ncomp(ctx->nf) <= 64 && ctx->fd_kernel == 2;
       const long long beside = fd_sm_smem((std::min(B, ctx->nrec) + 1) / 2, ctx->fd_tz);
       CK(launch_dft_tc(ctx->tmap, twt, ctx->nf, sbase, m1 - m0, m0, L, ctx->gh, ctx->ghb,
-                       (m1 == ntd && ctx->ghb) ? 1 : 0, b0, nb, ctx->nrec, ctx->d_err, expire,
+                       m1 == ntd ? 1 : 0, b0, nb, ctx->nrec, ctx->d_err, expire,
                        alone || ctx->fd_kernel == 3 ? 3 : slim ? 1 : 0, (alone || !slim) ? 0 : beside,
-                       ctx->side));
+                       down, ctx->side));
       CK(cudaEventRecord(ctx->ev_dft[2 * g + 1], ctx->side));
       CK(cudaEventRecord(ctx->dft_done[g & 1], ctx->side));
     }
@@ -1008,7 +1013,7 @@ extern "C" {
 
 egh_status egh_green(egh_ctx* ctx, const float* vel, void* stream_) {
   if (!ctx) return fail(nullptr, EGH_EINVAL, "ctx is NULL");
-  return green_run(ctx, vel, (cudaStream_t)stream_, nullptr, 0, 1, ctx->twt);
+  return green_run(ctx, vel, (cudaStream_t)stream_, nullptr, 0, 1, ctx->twt, (float)(1.0 / kTransformUp));
 }
 
 egh_status egh_green_bandlimited(egh_ctx* ctx, const float* vel, const float* wavelet,
@@ -1022,7 +1027,7 @@ egh_status egh_green_bandlimited(egh_ctx* ctx, const float* vel, const float* wa
   // spectral division and the decimation factor, folded into the twiddles:
   // g(w_k) = decim / S(w_k) * sum_m u_{m decim} exp(-i w_k m decim dt), S(w) = sum_n s_n e^{-i w n dt}
   std::vector<std::complex<double>> scale(ctx->nf);
-  double smax = 0.0;
+  double smax = 0.0, wmax = 0.0;
   for (int k = 0; k < ctx->nf; ++k) {
     std::complex<double> S(0.0, 0.0);
     for (int n = 0; n < nw; ++n) {
@@ -1037,7 +1042,11 @@ egh_status egh_green_bandlimited(egh_ctx* ctx, const float* vel, const float* wa
     if (!(std::abs(scale[k]) > 1e-6 * smax))
       return fail(ctx, EGH_EINVAL, "the wavelet's spectrum vanishes at frequency " + std::to_string(k));
     scale[k] = (double)decim / scale[k];
+    wmax = std::max(wmax, std::abs(scale[k]));
   }
+  // (a wavelet so faint that the factor would take the table near the largest float does without)
+  const double up = wmax * kTransformUp < 1e30 ? kTransformUp : 1.0;
+  for (auto& w : scale) w *= up;
   const int ntd = (ctx->nt + decim - 1) / decim;
   const std::vector<unsigned char> twt =
       dft_twiddle_tiles(ctx->freqs, ctx->dt * decim, ntd, &scale);
@@ -1056,7 +1065,7 @@ egh_status egh_green_bandlimited(egh_ctx* ctx, const float* vel, const float* wa
   // the previous Green stage may still read the table
   CK(cudaStreamSynchronize(ctx->side));
   CK(cudaMemcpy(ctx->twt_bl, twt.data(), twt.size(), cudaMemcpyHostToDevice));
-  return green_run(ctx, vel, stream, wavelet, nw, decim, ctx->twt_bl);
+  return green_run(ctx, vel, stream, wavelet, nw, decim, ctx->twt_bl, (float)(1.0 / up));
 }
 
 egh_status egh_hessian(egh_ctx* ctx, egh_mu_mode mode, double mu_param, double* mu_out,

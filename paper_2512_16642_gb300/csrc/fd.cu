@@ -622,7 +622,7 @@ __global__ void __launch_bounds__(128, 16)
     k_dft_tc(const __grid_constant__ CUtensorMap tmap, const unsigned char* __restrict__ twt,
              int N, int nf, int slot0, int kcount, int n0, long long G, float* __restrict__ gh,
              __nv_bfloat16* __restrict__ ghb, int last, int rec0, int nvalid, int nrec_all,
-             int* __restrict__ err, int expire, int nring) {
+             int* __restrict__ err, int expire, int nring, float down) {
   extern __shared__ __align__(1024) unsigned char dsm[];
   unsigned char* sm = dsm + ((1024 - (tc::smem_u32(dsm) & 1023)) & 1023);
   unsigned char* As = sm;                       // [nring][TD_AB]
@@ -739,7 +739,7 @@ __global__ void __launch_bounds__(128, 16)
     const long long p = p0 + tid;
     const long long row0 = (long long)(rec0 + r) * 2 * nf;  // first plane of this receiver
     float* g = gh + row0 * G + p;
-    for (int c0 = 0; c0 < N; c0 += 8) {
+    for (int c0 = 0; c0 < 2 * nf; c0 += 8) {  // (components past 2 nf are padding)
       float v[8], o[8];
       tmem_ld8(tmem + ((unsigned)(warp * 32) << 16) + (unsigned)c0, v);
       if (two) {  // the hi.lo columns, through o before o takes the old totals
@@ -751,7 +751,11 @@ __global__ void __launch_bounds__(128, 16)
         // middle chunks: each total is added where it lies (no other thread adds to it; rounded as
         // the sum of a read, an add and a write), so that the tile does not wait for the old totals:
         // on 512-level chunks of the layered grid the transform took as long as the FD steps beside
-        // it and held them up (transform 1000 -> 715 ms, Green stage 1032 -> 957 ms)
+        // it and held them up (transform 1000 -> 715 ms, Green stage 1032 -> 957 ms).  Such a
+        // reduction flushes operands and sums below 2^-126 to zero, so the twiddles are 2^24 times
+        // theirs (1 / down): every multiple of 2^-149 but zero is then above that.  (The factor
+        // changes no other rounding.  As a product here it took the registers of the copies' loop:
+        // layered update 905 -> 960 ms.)
 #pragma unroll
         for (int i = 0; i < 8; ++i)
           if (c0 + i < 2 * nf)
@@ -766,9 +770,9 @@ __global__ void __launch_bounds__(128, 16)
       for (int i = 0; i < 8; ++i) {
         const int c = c0 + i;
         if (c < 2 * nf) {
-          const float sum = o[i] + v[i];
+          const float sum = last ? (o[i] + v[i]) * down : v[i];
           __stcs(g + (long long)c * G, sum);
-          if (last) {
+          if (last && ghb) {
             // the Gram's operands: hi = bf16(g), lo = bf16(g - hi), blocked by 32 points as
             // [freq][G/32][hi|lo][receiver, re/im][32], the 16-byte runs of a row swapped as the MMA's
             // 64-byte swizzle wants them (see gram_tc.cu)
@@ -796,7 +800,7 @@ __global__ void __launch_bounds__(128, 16)
 cudaError_t launch_dft_tc(const CUtensorMap& tmap, const unsigned char* twt, int nf, int slot0,
                           int kcount, int n0, const Layout& L, float* gh, __nv_bfloat16* ghb,
                           int last, int rec0, int nvalid, int nrec_all, int* err, int expire,
-                          int per_sm, long long beside_smem, cudaStream_t st) {
+                          int per_sm, long long beside_smem, float down, cudaStream_t st) {
   const int N = dft_ncomp(nf);
   if (L.G % TD_M != 0 || N > TD_NMAX || kcount < 1 || slot0 % TD_S != 0 || n0 % TD_S != 0 ||
       nvalid < 1 || per_sm < 0 || per_sm > 3 || beside_smem < 0)
@@ -843,7 +847,7 @@ cudaError_t launch_dft_tc(const CUtensorMap& tmap, const unsigned char* twt, int
                                      : std::min<long long>((long long)sms * std::min(per_sm, occ), ntile));
   count_launches(1);
   k_dft_tc<<<grid, 128, smem, st>>>(tmap, twt, N, nf, slot0, kcount, n0, L.G, gh, ghb, last, rec0,
-                                    nvalid, nrec_all, err, expire, nring);
+                                    nvalid, nrec_all, err, expire, nring, down);
   return cudaGetLastError();
 }
 

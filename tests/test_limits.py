@@ -158,3 +158,24 @@ def test_capture_of_a_smaller_deblur(tmp_path):
         ctx.deblur(r[:1], one)
         torch.cuda.synchronize()
         assert torch.equal(one, big[:1]) and torch.equal(again, one)
+
+
+@pytest.mark.parametrize("fd_kernel", [0, 2])
+def test_transform_totals_below_the_normal_range(fd_kernel):
+    """Sums over several chunks whose totals lie below 2^-126 lose nothing.  A medium so slow that the
+    impulse stays where it is: u(t) = t u(1) with u(1) = 2^-133; at a quarter of the sampling rate the
+    twiddles are 0 and +-1, so that every term and total is an integer times 2^-133 and exact."""
+    import torch
+    from paper_2512_16642_gb300 import egh
+
+    nt = 160
+    v = torch.full((40, 40), float(np.sqrt(2.0 ** -113) / 1e-3), device="cuda")
+    with egh.Context(40, 40, 1024.0, 1024.0, 0, 0.5, 1e-3, nt, np.array([20], np.int32), np.array([7], np.int32),
+                     np.array([250.0]), dft_chunk=32, fd_kernel=fd_kernel) as ctx:
+        ctx.green(v)
+        g = ctx.get_green()[0, 0]
+    t = np.arange(nt)
+    want = np.sum(t * (-1j) ** (t % 4))
+    assert abs(want) < 2.0 ** 7
+    got = g[20, 7].astype(np.complex128) * 2.0 ** 133
+    assert got == want
