@@ -179,3 +179,19 @@ def test_transform_totals_below_the_normal_range(fd_kernel):
     assert abs(want) < 2.0 ** 7
     got = g[20, 7].astype(np.complex128) * 2.0 ** 133
     assert got == want
+
+
+def test_pivot_is_the_rounded_64_bit_root(tmp_path):
+    """Mixed precision's pivots: L22 = float(sqrt(a - x^2)) of [[1, x], [x, a]], the difference and its
+    root in 64 bits, for pairs whose root lies next to the middle between two floats."""
+    pairs = [("0x1.09ed800000000p+1", "0x1.71f6b40000000p-13"), ("0x1.884f1e0000000p+1", "0x1.3b94ee0000000p-12"),
+             ("0x1.6db68c0000000p+1", "0x1.d1c4960000000p-12"), ("0x1.81d2960000000p+0", "0x1.38d3c60000000p-13"),
+             ("0x1.8000000000000p+1", "0x1.0000000000000p-12")]
+    a, x = (np.array([float.fromhex(p[i]) for p in pairs]) for i in (0, 1))
+    Q = np.zeros((len(pairs), 2, 2), np.complex64)
+    Q[:, 0, 0], Q[:, 0, 1], Q[:, 1, 0], Q[:, 1, 1] = 1.0, x, x, a
+    with _line_ctx(2, len(pairs), 100, 1) as ctx:
+        _load_set(ctx, Q, tmp_path)
+        L = ctx.get_hessian(True)
+    assert np.array_equal(L[:, 1, 0].real, x.astype(np.float32))
+    assert np.array_equal(L[:, 1, 1].real, np.sqrt(a - x * x).astype(np.float32))
