@@ -298,60 +298,50 @@ cudaError_t launch_diag_sum(const float2* Qh, int nrec, int nf, double* d_sum, c
   return cudaGetLastError();
 }
 
-// ||Q_k||_F^2 per frequency: one block per frequency.  The squares are summed to FP64-class
-// accuracy in FP32 arithmetic (TwoProd and TwoSum into a two-word sum per thread, Ogita, Rump and
-// Oishi's Dot2) and combined in FP64: the GB300 issues FP64 at a small fraction of the FP32 rate,
-// and two FP64 operations per entry were the kernel's time (40 matrices of 341 rows: 150 us, now
-// 18 us).
-constexpr int FR_THREADS = 1024;
+// ||Q_k||_F^2 per frequency in FP64: one cluster per matrix, the blocks' sums joined by the first one
+// through distributed shared memory, in order.  Bound by the FP64 rate (a conversion and an FMA per real
+// number, two lanes a cycle and SM), so a matrix is spread over FR_CL SMs: 40 matrices of 341 rows took
+// 150 us with a block each, now 54 us.  (Two-word FP32 sums took 28 us, but are off by 1e-12 where the
+// entries' roundings all go one way.)
+constexpr int FR_CL = 8, FR_THREADS = 256;
 
-__device__ __forceinline__ void two_word_square(float a, float& s, float& c) {
-  const float p = __fmul_rn(a, a);
-  const float e = __fmaf_rn(a, a, -p);
-  const float t = __fadd_rn(s, p);
-  const float bp = __fsub_rn(t, s);
-  c = __fadd_rn(c, __fadd_rn(__fadd_rn(__fsub_rn(s, __fsub_rn(t, bp)), __fsub_rn(p, bp)), e));
-  s = t;
-}
-
-__global__ void __launch_bounds__(FR_THREADS)
+__global__ void __cluster_dims__(FR_CL, 1, 1) __launch_bounds__(FR_THREADS)
     k_fro2(const float2* __restrict__ Qh, int n, double* d_out) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
   __shared__ double red[FR_THREADS / 32];
-  __shared__ int emax;
+  __shared__ double part[FR_CL];
+  const int rank = (int)cluster.block_rank(), tid = threadIdx.x;
   const long long n2 = (long long)n * n;
-  const float2* A = Qh + (long long)blockIdx.x * n2;
-  // entries are scaled by the exponent of the largest diagonal one (which bounds every entry of a
-  // positive-definite matrix), so that the FP32 squares neither overflow nor lose their errors
-  if (threadIdx.x == 0) emax = -126;
-  __syncthreads();
-  for (int i = threadIdx.x; i < n; i += FR_THREADS) {
-    const float d = A[(long long)i * n + i].x;
-    if (isfinite(d) && d != 0.f) atomicMax(&emax, ilogbf(d));
-  }
-  __syncthreads();
-  const int ex = max(-126, min(126, emax));
-  const float sc = ldexpf(1.f, -ex);
-  float s[2] = {0.f, 0.f}, c[2] = {0.f, 0.f};
+  const float2* A = Qh + (long long)(blockIdx.x / FR_CL) * n2;
+  double s = 0.0, c = 0.0;
 #pragma unroll 4
-  for (long long t = threadIdx.x; t < n2; t += FR_THREADS) {
+  for (long long t = rank * FR_THREADS + tid; t < n2; t += FR_CL * FR_THREADS) {
     const float2 a = __ldg(A + t);
-    two_word_square(a.x * sc, s[0], c[0]);
-    two_word_square(a.y * sc, s[1], c[1]);
+    const double x = a.x, y = a.y;
+    s = fma(x, x, s);
+    c = fma(y, y, c);
   }
-  double v = ((double)s[0] + c[0]) + ((double)s[1] + c[1]);
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  if (threadIdx.x == 0) {
+  s += c;
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if ((tid & 31) == 0) red[tid >> 5] = s;
+  cluster.sync();  // (every block of the cluster runs before its shared memory is written)
+  if (tid == 0) {
     double sum = 0.0;
     for (int w = 0; w < FR_THREADS / 32; ++w) sum += red[w];
-    d_out[blockIdx.x] = ldexp(sum, 2 * ex);
+    cluster.map_shared_rank(part, 0)[rank] = sum;
+  }
+  cluster.sync();
+  if (rank == 0 && tid == 0) {
+    double sum = 0.0;
+    for (int b = 0; b < FR_CL; ++b) sum += part[b];
+    d_out[blockIdx.x / FR_CL] = sum;
   }
 }
 
 cudaError_t launch_fro2(const float2* Qh, int n, int nf, double* d_out, cudaStream_t st) {
   count_launches(1);
-  k_fro2<<<nf, FR_THREADS, 0, st>>>(Qh, n, d_out);
+  k_fro2<<<nf * FR_CL, FR_THREADS, 0, st>>>(Qh, n, d_out);
   return cudaGetLastError();
 }
 
@@ -364,7 +354,7 @@ cudaError_t launch_fro2(const float2* Qh, int n, int nf, double* d_out, cudaStre
 // and the partial norms go to every block of the cluster through distributed shared memory, in
 // two alternating buffers.  The 40 steps are a serial chain: with one block per matrix reading the
 // two triangular factors from L2 each of them took 10 to 37 us.  Measured on 40 matrices of 341
-// rows: 1471 us before, 166 us now (161 rows: 378 and 105 us).
+// rows: 1471 us before, 304 us now (257 rows: 800 and 166 us, 161 rows: 378 and 105 us).
 constexpr int IP_CL = 8, IP_THREADS = 512, IP_STEPS = 40;
 
 __global__ void __cluster_dims__(IP_CL, 1, 1) __launch_bounds__(IP_THREADS)

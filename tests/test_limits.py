@@ -195,3 +195,19 @@ def test_pivot_is_the_rounded_64_bit_root(tmp_path):
         L = ctx.get_hessian(True)
     assert np.array_equal(L[:, 1, 0].real, x.astype(np.float32))
     assert np.array_equal(L[:, 1, 1].real, np.sqrt(a - x * x).astype(np.float32))
+
+
+@pytest.mark.parametrize("n,v", [(341, 0.32015), (461, 0.39017), (860, 0.5487)])
+def test_frobenius_norm_of_the_condition_bound(n, v, tmp_path):
+    """The condition bound ||Q||_F / mu (mu above the smallest eigenvalue's estimate) of a matrix whose
+    entries are all equal but the diagonal ones, so that every partial sum rounds the same way: FP64
+    sums of at most 2 n^2 / 256 terms, joined in a few steps, are off by at most half of
+    (n^2 / 128 + 40) 2^-53, and the root and the quotient by two roundings."""
+    Q = np.full((1, n, n), np.float32(v), np.complex64)
+    Q[0, np.arange(n), np.arange(n)] = 1.0
+    with _line_ctx(n, 1, 100, 1) as ctx:
+        _load_set(ctx, Q, tmp_path, mu=16.0)
+        got = ctx.get_refinement()[0][0]
+    off = float(np.float32(v)) ** 2  # exact in 64 bits, as are its multiples below
+    want = np.sqrt(n + n * (n - 1) * off) / 16.0
+    assert abs(got / want - 1) <= (n * n / 128 + 40) / 2 * 2.0 ** -53 + 2.0 ** -51
