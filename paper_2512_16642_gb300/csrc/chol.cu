@@ -114,7 +114,6 @@ constexpr int CH_SB = 8;  // columns a thread holds at a time (unrolled code, ru
 struct alignas(16) PotrfShared {
   float2 LT[CH_PB][CH_PB];  // LT[j][c] = the diagonal tile's entry (c, j), c > j
   float inv[CH_PB];         // reciprocal pivots
-  int bad;
 };
 
 // x[q] -= y conj(l[q]) for the CH_SB columns at l
@@ -130,10 +129,10 @@ __device__ __forceinline__ void rank1_sub(float2 (&x)[CH_SB], float2 y, const fl
 }
 
 __device__ void potrf_block_panel(float2* __restrict__ A, int n, int* __restrict__ status_k,
-                                  int piv64, float2* P, double* dg, PotrfShared& sh) {
+                                  int piv64, float2* P, double* dg, PotrfShared& sh, int& bad_s) {
   const int tid = threadIdx.x;
   const int lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
-  if (tid == 0) sh.bad = 0;
+  if (tid == 0) bad_s = 0;
   for (int i = tid; i < n; i += blockDim.x) dg[i] = (double)A[(long long)i * n + i].x;
   __syncthreads();
   for (int p0 = 0; p0 < n; p0 += CH_PB) {
@@ -189,10 +188,10 @@ __device__ void potrf_block_panel(float2* __restrict__ A, int n, int* __restrict
         }
         __syncwarp();
       }
-      if (bad && lane == 0) sh.bad = bad;
+      if (bad && lane == 0) bad_s = bad;
     }
     __syncthreads();
-    if (sh.bad) break;
+    if (bad_s) break;
     // rows below the tile: x L^H = a, CH_SB columns at a time: the earlier columns in order, then
     // each new entry at once subtracted from the later ones (pw = 32 whenever there are rows below)
     for (int r = CH_PB + tid; r < R; r += blockDim.x) {
@@ -286,40 +285,43 @@ __device__ void potrf_block_panel(float2* __restrict__ A, int n, int* __restrict
     }
     __syncthreads();
   }
-  if (tid == 0) *status_k = sh.bad;
-  if (!sh.bad) {
+  if (tid == 0) *status_k = bad_s;
+  if (!bad_s) {
     for (int i = warp; i < n; i += nwarps)
       for (int l = i + 1 + lane; l < n; l += 32) A[(long long)i * n + l] = make_float2(0.f, 0.f);
   }
 }
 
 // shared memory for every matrix size up to nmax: the blocked form for n <= CH_PANEL_NMAX needs
-// the panel, the column form beyond it one column; a batch may hold both kinds (217.6 KB for the
-// panel of an 800-row matrix)
-size_t potrf_smem(int nmax) {
+// the panel and its diagonal tile, the column form beyond it one column; a batch may hold both kinds
+// (225.9 KB for the panel of an 800-row matrix)
+constexpr size_t potrf_smem(int nmax) {
   const size_t np = (size_t)std::min(nmax, CH_PANEL_NMAX);
-  const size_t panel = sizeof(float2) * np * CH_PS + sizeof(double) * np;
+  const size_t panel = sizeof(PotrfShared) + sizeof(float2) * np * CH_PS + sizeof(double) * np;
   if (nmax <= CH_PANEL_NMAX) return panel;
   const size_t column = sizeof(float2) * (size_t)(nmax + (nmax & 1)) + sizeof(double) * (size_t)nmax;
   return std::max(panel, column);
 }
 
-__device__ inline void potrf_any(float2* A, int n, int* status_k, int piv64, float2* buf,
-                                 PotrfShared& sh) {
+// the column form's 14527 rows, and the panel's, fit a block beside the status word
+static_assert(potrf_smem(14527) + sizeof(int) <= kBlockSmem && potrf_smem(CH_PANEL_NMAX) + sizeof(int) <= kBlockSmem);
+
+__device__ inline void potrf_any(float2* A, int n, int* status_k, int piv64, float2* buf, int& bad) {
   if (n <= CH_PANEL_NMAX) {
-    potrf_block_panel(A, n, status_k, piv64, buf, reinterpret_cast<double*>(buf + (size_t)n * CH_PS),
-                      sh);
+    PotrfShared& sh = *reinterpret_cast<PotrfShared*>(buf);
+    float2* P = reinterpret_cast<float2*>(&sh + 1);
+    potrf_block_panel(A, n, status_k, piv64, P, reinterpret_cast<double*>(P + (size_t)n * CH_PS), sh, bad);
   } else {
-    potrf_block(A, n, status_k, piv64, buf, reinterpret_cast<double*>(buf + n + (n & 1)), sh.bad);
+    potrf_block(A, n, status_k, piv64, buf, reinterpret_cast<double*>(buf + n + (n & 1)), bad);
   }
 }
 
 __global__ void __launch_bounds__(CH_THREADS)
     k_potrf(float2* __restrict__ Lh, int n, int* __restrict__ status, int piv64) {
-  extern __shared__ float2 pbuf[];  // panel (or column) cache, then the FP64 diagonal
-  __shared__ PotrfShared sh;
+  extern __shared__ __align__(16) float2 pbuf[];  // panel (or column) cache, then the FP64 diagonal
+  __shared__ int bad;
   const int k = blockIdx.x;
-  potrf_any(Lh + (long long)k * n * n, n, status + k, piv64, pbuf, sh);
+  potrf_any(Lh + (long long)k * n * n, n, status + k, piv64, pbuf, bad);
 }
 
 // Batched form: every matrix of a list (several survey patches x all their frequencies, of
@@ -327,17 +329,17 @@ __global__ void __launch_bounds__(CH_THREADS)
 template <int THREADS>
 __global__ void __launch_bounds__(THREADS)
     k_potrf_many(const PotrfItem* __restrict__ items, int count, int piv64) {
-  extern __shared__ float2 col[];  // sized for the largest matrix
-  __shared__ PotrfShared sh;
+  extern __shared__ __align__(16) float2 col[];  // sized for the largest matrix
+  __shared__ int bad;
   for (int m = blockIdx.x; m < count; m += gridDim.x) {
     const PotrfItem it = items[m];
-    potrf_any(it.A, it.n, it.status, piv64, col, sh);
+    potrf_any(it.A, it.n, it.status, piv64, col, bad);
     __syncthreads();
   }
 }
 
 cudaError_t potrf_many_prepare(int nmax) {
-  if (potrf_smem(nmax) > (size_t)kBlockSmem) return cudaErrorInvalidValue;
+  if (potrf_smem(nmax) + sizeof(int) > (size_t)kBlockSmem) return cudaErrorInvalidValue;
   const cudaError_t e = allow_block_smem<k_potrf_many<256>>();
   return e ? e : allow_block_smem<k_potrf_many<512>>();
 }
@@ -356,7 +358,7 @@ cudaError_t launch_potrf_many(const PotrfItem* items, int count, int nmax, int b
 
 cudaError_t launch_potrf(float2* Lh, int n, int nf, int* status, cudaStream_t st, int piv64) {
   const size_t smem = potrf_smem(n);
-  if (smem > 32 * 1024) {  // beside the static 8.2 KB
+  if (smem > 47 * 1024) {  // (beside the status word)
     const cudaError_t e = allow_block_smem<k_potrf>();
     if (e != cudaSuccess) return e;
   }

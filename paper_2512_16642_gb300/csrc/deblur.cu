@@ -1180,11 +1180,19 @@ __global__ void __launch_bounds__(32 * TRI_WARPS)
   }
 }
 
+// four columns per warp up to 1536 rows; beyond, one
+constexpr bool tri_four(int n) { return n <= 1536; }
+// 32-entry groups of a column, by fours where fewer than TRI_PRE hold it
+constexpr int tri_groups(int n) { return tri_four(n) ? ((n + 31) / 32 + 3) / 4 * 4 : (n + 31) / 32; }
+constexpr size_t tri_smem(int n) {
+  return sizeof(float2) * TRI_WARPS * (tri_four(n) ? 4 : 1) * 32 * (size_t)tri_groups(n);
+}
+static_assert(tri_smem(1536) <= 200 * 1024 && tri_smem(7264) <= kBlockSmem && tri_groups(1537) >= TRI_PRE);
+
 cudaError_t launch_trtri(const float2* Lh, int n, int nf, float2* Wh, cudaStream_t st) {
-  const int groups = ((n + 31) / 32 + 3) / 4 * 4;  // 32-entry groups of a column, by fours
-  const size_t one = sizeof(float2) * TRI_WARPS * 32 * (size_t)groups;  // one column per warp
-  const bool four = 4 * one <= 200 * 1024;  // up to 1536 rows; beyond, a column per warp
-  const size_t smem = four ? 4 * one : one;
+  const int groups = tri_groups(n);
+  const bool four = tri_four(n);
+  const size_t smem = tri_smem(n);
   auto kern = four ? k_trtri<4> : k_trtri<1>;
   if (smem > 48 * 1024) {
     const cudaError_t e = four ? allow_block_smem<k_trtri<4>>() : allow_block_smem<k_trtri<1>>();

@@ -209,7 +209,6 @@ struct PotrfItem {
   int n;
   int* status;  // 0, or the failing pivot + 1
 };
-size_t potrf_smem(int nmax);
 cudaError_t potrf_many_prepare(int nmax);
 cudaError_t launch_potrf_many(const PotrfItem* items, int count, int nmax, int blocks, int threads,
                               int piv64, cudaStream_t st);
