@@ -572,7 +572,7 @@ egh_status egh_create(const egh_config* cfg, egh_ctx** out) {
       ctx->fd_kernel = 1;
     } else if (c.fd_kernel == 0 && c.fd_rows == 0 && fd_cluster_plan(L, &ctx->cl)) {
       const int b = c.batch_receivers ? c.batch_receivers : 32;
-      if (fd_cluster_faster(ctx->cl, L, c.nrec, b)) ctx->fd_kernel = 3;
+      if (fd_cluster_faster(ctx->cl, L, c.nrec, b, c.nfreq)) ctx->fd_kernel = 3;
     }
     if (res)
       ctx->B = c.batch_receivers ? std::min(c.batch_receivers, c.nrec) : std::min(c.nrec, 2 * ctx->rg.P);

@@ -164,8 +164,9 @@ struct ClGeom {
   size_t smem;     // dynamic shared memory per block
 };
 bool fd_cluster_plan(const Layout& L, ClGeom* g);  // false if the grid does not fit
-// whether nrec receivers, at most b in a batch, take less time than with the per-step kernel
-bool fd_cluster_faster(const ClGeom& g, const Layout& L, int nrec, int b);
+// whether nrec receivers, at most b in a batch, and nf frequencies take less time than with the
+// per-step kernel
+bool fd_cluster_faster(const ClGeom& g, const Layout& L, int nrec, int b, int nf);
 // Levels ta .. ta+nsteps-1 (ta >= 2) of nb receivers from the state slots of levels ta-1, ta-2 to
 // the slots of the last two; level t's snapshot to ring slot sbase + (t - t0) / decim when
 // t % decim == 0; wav (device, may be null): level t takes sample t - 1 < nw at the receivers' points

@@ -284,7 +284,10 @@ bool fd_cluster_plan(const Layout& L, ClGeom* out) {
   g.smem = g.coef_smem ? lev + cf : lev;
   if (g.smem > (size_t)optin) return false;
   // rows per unit: the rounds of 512 threads times a unit's length (its rows and the window of
-  // eight rows that it reads first)
+  // eight rows that it reads first, half as dear), and a little for all the units' reads.  Chosen and
+  // best of the six, 20 receivers x 1000 steps, 26 frequencies: 31 x 41 grid 2.02 (2 rows) and 1.98 ms
+  // (3), 101 x 101 3.46 (3) and 3.37 (6), 101 x 301 5.53 (11), 151 x 201 5.22 (6) and 5.11 (8), 201 x 201
+  // 6.03 (8) and 5.98 (11), 101 x 500 8.20 (6); the worst of the six took 1.15 to 1.4 times the best
   long long best = 0;
   for (int sr : kSR) {
     const long long units = (long long)NXH * ((g.rows + sr - 1) / sr);
@@ -319,19 +322,23 @@ bool fd_cluster_plan(const Layout& L, ClGeom* out) {
   return true;
 }
 
-// Time of a step over all batches.  Measured (1000 steps, 26 frequencies): a round of clusters takes
-// 2.1 us on 101 x 121 padded points, 2.7 on 141 x 141, 4.2 on 141 x 341, 4.5 on 241 x 241, 6.1 on 271 x
-// 278, about 1.3 us and 0.52 us per 1000 points of a block; with several rounds a round's transform
-// runs beside the next one, which then takes 1.2 to 1.4 times as long.  The per-step kernel takes 3.8
-// us a batch of 16 receivers on the smallest of these grids and 4.4 on the largest, a launch and a
-// warp's rows.  Whole Green stages, clusters against per-step kernel: 40 receivers on 141 x 341 points
-// 12.1 and 12.9 ms, on 255 x 270 points 17.2 and 14.6 ms; 100 receivers 26.7 and 29.2, 38.3 and 32.0.
-bool fd_cluster_faster(const ClGeom& g, const Layout& L, int nrec, int b) {
-  const int bc = std::min(b, 2 * g.clusters), bs = std::min(b, 16);
-  const double pts = (double)L.NZ * L.NX;
-  const double tc = (double)((nrec + bc - 1) / bc) * (nrec > bc ? 1.3 : 1.0) * (1.3 + 0.52e-3 * pts / CL);
-  const double ts = (double)((nrec + bs - 1) / bs) * (3.75 + 0.88e-5 * pts);
-  return tc < 0.95 * ts;
+// Microseconds per time step of the whole Green stage with either solver, fitted to runs of 1000 steps
+// on nine grids (71 x 81 to 271 x 278 padded points), 2 to 100 receivers, 5, 26 and 60 frequencies, to
+// within 12% for one round of clusters (or one batch), 25% for several; n: receivers, p: points, c:
+// transform components.
+// The clusters leave the transform fewer SMs beside them, so its work counts more than beside the
+// per-step kernel.  The choice was at most 1.06 times the better one's time, and 1.006 times on
+// average, for every level transformed.  Clusters and per-step kernel, ms: 101 x 101 grid, 21 receivers,
+// 5 frequencies 3.3 and 6.5; 151 x 201, 12 and 26: 4.7 and 5.7; 215 x 230, 6 and 26: 6.4 and 4.9, 21 and
+// 26: 7.9 and 8.6; 201 x 201, 40 and 26: 13.4 and 13.5, 100 and 60: 36.5 and 30.5.
+bool fd_cluster_faster(const ClGeom& g, const Layout& L, int nrec, int b, int nf) {
+  const int rounds = (nrec + std::min(b, 2 * g.clusters) - 1) / std::min(b, 2 * g.clusters);
+  const int batches = (nrec + b - 1) / b;
+  const double n = nrec, p = (double)L.NZ * L.NX, w = n * p * dft_ncomp(nf);
+  const double tc = (rounds == 1 ? 1.5 + 0.57e-4 * p : rounds * (1.0 + 0.77e-4 * p)) + 2.2e-8 * w;
+  const double ts = batches == 1 ? 3.65 + 0.10 * n + 0.78e-6 * n * p + 1.2e-8 * w
+                                 : 1.4 + 1.8 * batches + 0.15 * n + 0.63e-6 * n * p + 0.9e-8 * w;
+  return tc < ts;
 }
 
 cudaError_t launch_fd_cluster(const ClGeom& g, float2* lev, int pslot, const Layout& L, const float2* coef,

@@ -211,3 +211,15 @@ def test_frobenius_norm_of_the_condition_bound(n, v, tmp_path):
     off = float(np.float32(v)) ** 2  # exact in 64 bits, as are its multiples below
     want = np.sqrt(n + n * (n - 1) * off) / 16.0
     assert abs(got / want - 1) <= (n * n / 128 + 40) / 2 * 2.0 ** -53 + 2.0 ** -51
+
+
+@pytest.mark.parametrize("nz,nx,nrec,nf,solver", [(101, 101, 21, 5, 3), (151, 201, 12, 26, 3), (215, 230, 6, 26, 2),
+                                                  (201, 201, 100, 60, 2), (231, 238, 24, 60, 2)])
+def test_solver_of_a_small_grid(nz, nx, nrec, nf, solver):
+    """The solver that is clearly the faster one is taken: with many frequencies the clusters leave the
+    transform too few SMs."""
+    from paper_2512_16642_gb300 import egh
+
+    with egh.Context(nz, nx, 10.0, 10.0, 20, 1e-3, 1e-3, 100, np.zeros(nrec, np.int32),
+                     np.arange(nrec, dtype=np.int32), np.linspace(3.0, 15.0, nf)) as ctx:
+        assert ctx.stats()["fd_kernel"] == solver
