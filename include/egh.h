@@ -118,9 +118,11 @@ typedef struct {
                                 egh_green times the FD steps of all receivers in batches of 8, 16,
                                 32 and min(nrec, 32) and keeps 16 (or nrec, if less) unless another
                                 is 3% faster; with the cluster solver, as many as run at once (at
-                                most 32); else min(nrec, 16) */
+                                most 32: its ring below is then up to twice that of 16 receivers,
+                                which a caller short of memory can ask for); else min(nrec, 16) */
     int32_t dft_chunk;       /* levels per transform chunk: 32, 64, ..., 2048; 0 = 512 (the
-                                snapshot ring holds 2 chunks x batch_receivers levels); a
+                                snapshot ring holds 2 chunks x batch_receivers levels of 4 bytes per
+                                point of the padded, pitched grid); a
                                 chunk longer than the record is cut to the smallest power of
                                 two, at least 32, that holds nt levels (the same arithmetic in
                                 one chunk, a smaller ring) */
@@ -130,7 +132,9 @@ typedef struct {
     int32_t fd_rows;         /* FD rows per warp: 12, 16, 18, 20, 24 or 32; 0 = timed on the first
                                 egh_green of the context: the smallest count whose tiles fit one
                                 wave of resident blocks is kept unless another is 3% faster */
-    int32_t precision;       /* egh_precision of the Hessian stage (0 = EGH_PREC_FP32) */
+    int32_t precision;       /* egh_precision of the Hessian stage (0 = EGH_PREC_FP32); the mixed ones
+                                hold the inverse factors, the inverses and the inverses' operand
+                                images (48 KB per 128 rows x 32 columns) beside Q and L */
     int32_t fd_kernel;       /* FD solver of the Green stage: 2 = one kernel per time step, state in
                                 global memory (L2-resident); 0 = that one, but on small grids (and
                                 with fd_rows = 0) a cluster of blocks per receiver pair that keeps
@@ -237,6 +241,8 @@ egh_status egh_factor(egh_ctx *ctx, int32_t *bad_freq, void *stream);
  * bounded device wait of its transforms ran out; with device buffers it returns
  * before the work completes, and such an expiry is reported by the next call
  * that waits for the device (egh_green, egh_hessian, a host-buffer deblur).
+ * A call on device buffers that has no more traces, and no longer ones, than an
+ * earlier one allocates nothing and can be captured into a graph.
  * A source's multipliers do not depend on the other sources of the call, bit
  * for bit.  Device buffers and pageable host buffers (staged through device
  * buffers) give the same bits; page-locked host buffers are read and written
@@ -247,7 +253,7 @@ egh_status egh_deblur(egh_ctx *ctx, const float *resid, int32_t ns, int32_t nt_d
 /* Threshold of the selective refinement of the mixed precisions (the paper has no counterpart:
  * its precision is not stated).  egh_factor bounds each cond(Q_k) by ||Q_k||_F times the smaller
  * of 1/mu (lambda_min >= mu) and 1.25 times a 40-step power estimate of lambda_max(Q_k^{-1})
- * computed with the inverse factor; the solves of the frequencies whose bound exceeds the
+ * of the inverse; the solves of the frequencies whose bound exceeds the
  * threshold get one refinement step.  0 refines every frequency, infinity none.  Applies from the
  * next egh_factor.  EGH_EINVAL if negative or NaN. */
 egh_status egh_set_refinement(egh_ctx *ctx, double threshold);
@@ -340,7 +346,9 @@ egh_status egh_gram_noalloc(const float *gh, int32_t nrec, int32_t nfreq, int64_
 typedef struct egh_server egh_server;
 
 typedef struct {
-    int64_t hbm_budget_bytes;  /* device arena for request buffers (>= 1 MiB) */
+    int64_t hbm_budget_bytes;  /* device arena for request buffers (>= 1 MiB); the sets' own memory is
+                                  not counted: Q and L in FP32, Q and the inverses' operand images (48
+                                  KB per 128 rows x 32 columns and frequency) in mixed precision */
     int32_t slots;             /* batches in flight at once, 1..16 */
     int32_t max_batch_sources; /* sources packed into one batch, >= 1 */
     int32_t precision;         /* egh_precision of the sets' factorisations and solves */

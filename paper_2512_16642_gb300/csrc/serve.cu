@@ -86,10 +86,8 @@ class Arena {
 
 struct HSet {
   int nrec = 0, nf = 0, tw_len = 0;
-  float2 *Qh = nullptr, *Lh = nullptr, *tw = nullptr;
-  float2* Wh = nullptr;  // mixed precision: W = L^{-1}
-  float2* Ph = nullptr;  // mixed precision: Q^{-1} = W^H W
-  unsigned char* Pimg = nullptr;  // its operand images for the solve's product
+  float2 *Qh = nullptr, *Lh = nullptr, *tw = nullptr;  // Lh: not kept in mixed precision
+  unsigned char* Pimg = nullptr;  // mixed precision: operand images of Q^{-1} for the solve's product
   int* kref = nullptr;   // mixed precision: frequencies whose solves are refined (device list)
   int nref = 0;
   unsigned char* twt = nullptr;  // tensor-core transform twiddle tiles (tw_len levels)
@@ -457,11 +455,9 @@ egh_status egh_server_add_set(egh_server* sv, int32_t nrec, int32_t nfreq, const
   auto cleanup = [&]() {
     cudaFree(d_cond);
     cudaFree(h.kref);
-    cudaFree(h.Ph);
     cudaFree(h.Pimg);
     cudaFree(h.twt);
     cudaFree(h.tws);
-    cudaFree(h.Wh);
     cudaFree(h.Qh);
     cudaFree(h.Lh);
     cudaFree(h.tw);
@@ -470,7 +466,8 @@ egh_status egh_server_add_set(egh_server* sv, int32_t nrec, int32_t nfreq, const
   };
   cudaError_t e = cudaSuccess;
   if (!e) e = cudaMalloc(&h.Qh, qn * sizeof(float2));
-  if (!e) e = cudaMalloc(&h.Lh, qn * sizeof(float2));
+  // mixed precision: L, W = L^{-1} and Q^{-1} = W^H W, given back once the images of Q^{-1} are made
+  if (!e) e = cudaMalloc(&h.Lh, (prec_mixed(sv->prec) ? 3 : 1) * qn * sizeof(float2));
   if (!e) e = cudaMalloc(&h.tw, tw.size() * sizeof(float2));
   if (!e) e = cudaMalloc(&h.w, w.size() * sizeof(float));
   if (!e) e = cudaMalloc(&status, nfreq * sizeof(int));
@@ -491,15 +488,14 @@ egh_status egh_server_add_set(egh_server* sv, int32_t nrec, int32_t nfreq, const
   if (!e) e = launch_potrf(h.Lh, nrec, nfreq, status, st, prec_mixed(sv->prec) ? 1 : 0);
   std::vector<double> cond(2 * nfreq, 0.0);
   if (!e && prec_mixed(sv->prec)) {
-    e = cudaMalloc(&h.Wh, qn * sizeof(float2));
-    if (!e) e = launch_trtri(h.Lh, nrec, nfreq, h.Wh, st);
-    if (!e) e = cudaMalloc(&h.Ph, qn * sizeof(float2));
-    if (!e) e = launch_gram_inverse(h.Wh, nrec, nfreq, h.Ph, st);
+    float2 *Wh = h.Lh + qn, *Ph = h.Lh + 2 * qn;
+    e = launch_trtri(h.Lh, nrec, nfreq, Wh, st);
+    if (!e) e = launch_gram_inverse(Wh, nrec, nfreq, Ph, st);
     if (!e) e = cudaMalloc(&h.Pimg, cmm_image_bytes(nrec, nfreq));
-    if (!e) e = launch_cmm_images(h.Ph, nrec, nfreq, h.Pimg, st);
+    if (!e) e = launch_cmm_images(Ph, nrec, nfreq, h.Pimg, st);
     if (!e) e = cudaMalloc(&d_cond, 2 * nfreq * sizeof(double));
     if (!e) e = launch_fro2(h.Qh, nrec, nfreq, d_cond, st);
-    if (!e) e = launch_inv_power(h.Ph, nrec, nfreq, d_cond + nfreq, st);
+    if (!e) e = launch_inv_power(Ph, nrec, nfreq, d_cond + nfreq, st);
     if (!e) e = cudaMemcpyAsync(cond.data(), d_cond, 2 * nfreq * sizeof(double), cudaMemcpyDeviceToHost, st);
   }
   std::vector<int> stv(nfreq, 0);
@@ -527,6 +523,10 @@ egh_status egh_server_add_set(egh_server* sv, int32_t nrec, int32_t nfreq, const
   status = nullptr;
   cudaFree(d_cond);
   d_cond = nullptr;
+  if (prec_mixed(sv->prec)) {
+    cudaFree(h.Lh);
+    h.Lh = nullptr;
+  }
   for (int k = 0; k < nfreq; ++k)
     if (stv[k]) {
       cleanup();
@@ -693,11 +693,9 @@ void egh_server_destroy(egh_server* sv) {
   for (auto& s : sv->streams) cudaStreamDestroy(s);
   for (HSet& h : sv->sets) {
     cudaFree(h.kref);
-    cudaFree(h.Ph);
     cudaFree(h.Pimg);
     cudaFree(h.twt);
     cudaFree(h.tws);
-    cudaFree(h.Wh);
     cudaFree(h.Qh);
     cudaFree(h.Lh);
     cudaFree(h.tw);

@@ -223,3 +223,23 @@ def test_solver_of_a_small_grid(nz, nx, nrec, nf, solver):
     with egh.Context(nz, nx, 10.0, 10.0, 20, 1e-3, 1e-3, 100, np.zeros(nrec, np.int32),
                      np.arange(nrec, dtype=np.int32), np.linspace(3.0, 15.0, nf)) as ctx:
         assert ctx.stats()["fd_kernel"] == solver
+
+
+def test_server_keeps_what_its_solves_read():
+    """A mixed-precision set of a server holds its Hessians and the operand images of their inverses
+    (48 KB per 128 rows x 32 columns), not the factors they were made from."""
+    import torch
+    from paper_2512_16642_gb300 import egh
+
+    n, nf = 257, 40
+    A = np.random.default_rng(1).standard_normal((n, 2 * n))
+    Q = np.broadcast_to((A @ A.T / n + np.eye(n)).astype(np.complex64), (nf, n, n)).copy()
+    with egh.Server(8 << 20, precision=egh.EGH_PREC_MIXED) as sv:
+        f = np.linspace(2.0, 10.0, nf)
+        sv.add_set(Q, f, 1e-3, 500, 500)  # (loads the kernels)
+        free = torch.cuda.mem_get_info()[0]
+        for _ in range(4):
+            sv.add_set(Q, f, 1e-3, 500, 500)
+        held = (free - torch.cuda.mem_get_info()[0]) / 4
+    images = nf * -(-n // 128) * -(-n // 32) * (48 << 10)
+    assert held <= Q.nbytes + images + (6 << 20)  # twiddle tables and the allocator's 2 MB blocks
