@@ -758,40 +758,39 @@ egh_status time_fd_steps(egh_ctx* ctx, int np, int tz, int slots, float* best) {
   return EGH_OK;
 }
 
-// Receivers per batch, timed once per context before the ring (sized for the batch) exists: the FD
-// steps of all receivers in batches of 8, 16, 32 or all that the state slots hold, the last batch
-// with what is left (each with its one-wave rows per warp).  16 is kept unless another is 3% faster.
-// The transform's work per receiver does not depend on the batch, and it runs beside the FD steps for
-// every choice.  (By the time per receiver
-// alone, 12 receivers ran as 8 and 4: 295x496 grid, 1000 steps, 12.2 ms, now 8.7 ms.)
+// Receivers per batch, chosen once per context before the ring (sized for the batch) exists.
+// Fewer than 16 receivers go in one batch while their three levels stay well inside the L2 (40 MB),
+// else eight at a time.  Measured, 400 steps, 26 frequencies, one batch and eight at a time: 295x496
+// grid (28 MB) 12 receivers 4.61 and 5.05 ms, 15 (35 MB) 5.68 and 5.87; 301x921 12 (50 MB) 7.00 and 6.95,
+// 15 (63 MB) 8.96 and 8.29; 600x600 9 (49 MB) 7.33 and 7.04, 15 (81 MB) 11.7 and 10.2; 351x1701 11 (92 MB)
+// 15.7 and 12.3.
+// From 16 on by the time per receiver of 8, 16 and 32 in a batch: 24 FD steps as the run launches them
+// (each with its one-wave rows per warp).  16 is kept unless another is 3% faster.  The transform's work
+// per receiver does not depend on the batch, and it runs beside the FD steps for every choice but the
+// last batch's, which is why a batch of all 17 to 31 receivers is none of them: 295x496, 20 receivers 7.23
+// ms against 6.78 in batches of 16.
 egh_status tune_batch(egh_ctx* ctx, cudaStream_t stream) {
-  CK(cudaEventRecord(ctx->ev_tune[0], stream));  // after the coefficients
-  CK(cudaStreamWaitEvent(ctx->fdst, ctx->ev_tune[0], 0));
-  std::map<int, float> step;  // by pairs
-  egh_status s = EGH_OK;
-  auto time = [&](int b) {
-    const int np = (b + 1) / 2;
-    auto it = step.find(np);
-    if (it != step.end()) return it->second;
-    float ms = 1e30f;
-    if (s == EGH_OK) s = time_fd_steps(ctx, np, fd_rows_one_wave(ctx->L, np), 0, &ms);
-    return step[np] = ms;
-  };
-  const int def_b = std::min(ctx->Bcap, 16);
-  float best = 1e30f, def_ms = 1e30f;
-  int best_b = def_b;
-  for (int b : {8, 16, 32, ctx->Bcap}) {
-    if (b > ctx->Bcap) continue;
-    const int rest = ctx->nrec % b;
-    const float ms = (float)(ctx->nrec / b) * time(b) + (rest ? time(rest) : 0.f);
-    if (s) return s;
-    if (ms < best) {
-      best = ms;
-      best_b = b;
+  if (ctx->nrec < 16) {
+    ctx->B = 3.0 * sizeof(float) * ctx->nrec * (double)ctx->L.F <= 40e6 ? ctx->nrec : 8;
+  } else {
+    CK(cudaEventRecord(ctx->ev_tune[0], stream));  // after the coefficients
+    CK(cudaStreamWaitEvent(ctx->fdst, ctx->ev_tune[0], 0));
+    float best = 1e30f, def = 1e30f;
+    int best_b = 16;
+    for (int b : {8, 16, 32}) {
+      if (b > ctx->Bcap) continue;
+      float ms = 0.f;
+      const egh_status s = time_fd_steps(ctx, b / 2, fd_rows_one_wave(ctx->L, b / 2), 0, &ms);
+      if (s) return s;
+      ms /= (float)b;
+      if (ms < best) {
+        best = ms;
+        best_b = b;
+      }
+      if (b == 16) def = ms;
     }
-    if (b == def_b) def_ms = ms;
+    ctx->B = best < 0.97f * def ? best_b : 16;
   }
-  ctx->B = best < 0.97f * def_ms ? best_b : def_b;
   ctx->Bp = 2 * ((ctx->B + 1) / 2);
   ctx->st.batch_receivers = ctx->B;
   ctx->tune_B = false;
