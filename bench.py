@@ -38,12 +38,12 @@ FALLBACK_HBM_GBS = 6800.0
 # DRAM traffic (read + write bytes) per launch of the FD step and of the transform from the
 # committed ncu capture (profiles/), valid only for the kernel sources it was taken from (sha256
 # of csrc/fd.cu); None until a capture exists.
-KERNEL_TRAFFIC = {"fd_sha256": "8afae4dbb4943cb9c3c79b80b5e97a5bc7d87578b94ef69c01d0f0998c9a03a3",
-                  "k_fd_step": 32.13e6,   # 1.64 MB read + 30.49 MB write per launch (18 rows per warp)
+KERNEL_TRAFFIC = {"fd_sha256": "749bbc0d91603f48cfefceb7f808099e47ece4a0bf37e4a721c0f56cd03a90e0",
+                  "k_fd_step": 31.60e6,   # 1.21 MB read + 30.39 MB write per launch (18 rows per warp)
                   "k_dft_tc": 48.10e9,    # 45.78 GB read + 2.33 GB write per 2048-level launch
-                  "gram_sha256": "f9de315c9b531216c4542c842f967a76ddf97ec6b8c30623a20ace1b44982cd4",
+                  "gram_sha256": "c41f312cc4aec01cca1aab5b9b9c88170b85b5bcb2c7319928b49624b8d12bc0",
                   # per launch at 231 receivers x 26 frequencies, by grid-sum splits (read + write)
-                  "k_gram_tc": {8: 32.98e9, 16: 24.54e9, 32: 18.09e9}}
+                  "k_gram_tc": {8: 24.23e9, 16: 18.59e9, 32: 17.54e9}}
 
 
 def _args():

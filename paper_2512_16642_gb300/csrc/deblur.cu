@@ -335,7 +335,7 @@ __global__ void __cluster_dims__(TD_S, 1, 1) __launch_bounds__(256)
 // TMEM block (TT_J stages of a part) as its unit: the blocks' sums go to the scratch and the last
 // unit of the tile to arrive adds them in the order in which one unit per part adds them, so the
 // spectra have the same bits in both forms.  Used where two parts leave half of the SMs without a
-// unit (34 us for that source before, 24 us now).
+// unit (34 us for that source before, 22.5 us now).
 // ---------------------------------------------------------------------------------------------
 constexpr int TP_EPI = 256;  // threads of warps 0-7
 constexpr int TP_A = 2;  // A tiles in TMEM (the converters fill one while the MMAs read another)
@@ -821,7 +821,7 @@ cudaError_t launch_trace_tma(const float* resid, int ntr, int nt_d, const unsign
 // barriers and a reduction in the row-at-a-time form this replaces); 16 sources per block keep
 // the sums short and give four times the blocks of the 32-source, 64 KB form.  Measured on
 // 161 receivers x 40 frequencies x 57 sources: 605 us for
-// the row form, about 70 us for this one (the FP32 deblur call 0.76 -> 0.23 ms).
+// the row form, 81 us for this one (the FP32 deblur call 0.76 -> 0.19 ms with the ragged synthesis).
 // ---------------------------------------------------------------------------------------------
 constexpr int TS_W = 8;               // warps per block (also of the residual kernels)
 constexpr int TR_B = 32, TR_C = 16;   // block rows, sources per block
