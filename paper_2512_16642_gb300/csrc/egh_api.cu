@@ -267,9 +267,9 @@ egh_status ensure_twiddles(egh_ctx* ctx, int len, cudaStream_t stream) {
   const std::vector<unsigned char> u = synth_twiddle_tiles(ctx->freqs, ctx->dt, len);
   if ((s = dalloc(ctx, (void**)&ctx->tws_deb, u.size(), "synthesis twiddle tiles"))) return s;
   CK(cudaMemcpy(ctx->tws_deb, u.data(), u.size(), cudaMemcpyHostToDevice));
+  // (a device without room for it takes the transform's other form, which gives the same bits)
   const size_t sb = trace_scratch_most(ctx->nf, ctx->nrec, len);
-  if (sb && (s = dalloc(ctx, (void**)&ctx->trace_ws, sb, "transform blocks"))) return s;
-  ctx->trace_ws_cap = sb;
+  if (sb && dalloc(ctx, (void**)&ctx->trace_ws, sb, "transform blocks") == EGH_OK) ctx->trace_ws_cap = sb;
   ctx->tw_len = len;
   return EGH_OK;
 }
