@@ -345,15 +345,12 @@ cudaError_t potrf_many_prepare(int nmax) {
 }
 
 cudaError_t launch_potrf_many(const PotrfItem* items, int count, int nmax, int blocks, int threads,
-                              int piv64, cudaStream_t st) {
+                              int piv64, const Lane& lane) {
   const size_t smem = potrf_smem(nmax);
+  if (threads != 256 && threads != 512) return cudaErrorInvalidValue;
   count_launches(1);
-  switch (threads) {
-    case 256: k_potrf_many<256><<<blocks, 256, smem, st>>>(items, count, piv64); break;
-    case 512: k_potrf_many<512><<<blocks, 512, smem, st>>>(items, count, piv64); break;
-    default: return cudaErrorInvalidValue;
-  }
-  return cudaGetLastError();
+  return launch_on(lane, false, threads == 256 ? k_potrf_many<256> : k_potrf_many<512>, blocks, threads, smem,
+                   items, count, piv64);
 }
 
 cudaError_t launch_potrf(float2* Lh, int n, int nf, int* status, cudaStream_t st, int piv64) {

@@ -1189,7 +1189,7 @@ constexpr size_t tri_smem(int n) {
 }
 static_assert(tri_smem(1536) <= 200 * 1024 && tri_smem(7264) <= kBlockSmem && tri_groups(1537) >= TRI_PRE);
 
-cudaError_t launch_trtri(const float2* Lh, int n, int nf, float2* Wh, cudaStream_t st) {
+cudaError_t launch_trtri(const float2* Lh, int n, int nf, float2* Wh, const Lane& lane) {
   const int groups = tri_groups(n);
   const bool four = tri_four(n);
   const size_t smem = tri_smem(n);
@@ -1200,8 +1200,7 @@ cudaError_t launch_trtri(const float2* Lh, int n, int nf, float2* Wh, cudaStream
   }
   const int cb = four ? 4 : 1, warps = 32 * ((groups + cb - 1) / cb);
   count_launches(1);
-  kern<<<dim3(warps / TRI_WARPS, nf), 32 * TRI_WARPS, smem, st>>>(Lh, n, groups, Wh);
-  return cudaGetLastError();
+  return launch_on(lane, false, kern, dim3(warps / TRI_WARPS, nf), 32 * TRI_WARPS, smem, Lh, n, groups, Wh);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1290,11 +1289,10 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-cudaError_t launch_gram_inverse(const float2* Wh, int n, int nf, float2* Ph, cudaStream_t st) {
+cudaError_t launch_gram_inverse(const float2* Wh, int n, int nf, float2* Ph, const Lane& lane) {
   const int nt = (n + GI_T - 1) / GI_T;
   count_launches(1);
-  k_gram_inverse<<<dim3(nt * (nt + 1) / 2, nf), 256, 0, st>>>(Wh, n, Ph);
-  return cudaGetLastError();
+  return launch_on(lane, false, k_gram_inverse, dim3(nt * (nt + 1) / 2, nf), 256, 0, Wh, n, Ph);
 }
 
 // ---------------------------------------------------------------------------------------------

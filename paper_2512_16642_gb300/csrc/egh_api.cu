@@ -41,6 +41,41 @@ namespace egh {
 void count_launches(int n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
 long long launches_so_far() { return g_launches.load(std::memory_order_relaxed); }
 void set_context_free_error(const std::string& msg) { g_create_error = msg; }
+
+cudaError_t lane_launch(const Lane& lane, const void* kernel, dim3 grid, dim3 block, size_t smem,
+                        void** args, bool early) {
+  if (!lane.graph) {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = lane.stream;
+    cfg.attrs = &at;
+    cfg.numAttrs = early ? 1 : 0;
+    return cudaLaunchKernelExC(&cfg, kernel, args);
+  }
+  cudaGraphNodeParams np = {cudaGraphNodeTypeKernel};
+  np.kernel.func = const_cast<void*>(kernel);
+  np.kernel.gridDim = grid;
+  np.kernel.blockDim = block;
+  np.kernel.sharedMemBytes = (unsigned)smem;
+  np.kernel.kernelParams = args;
+  np.kernel.extra = nullptr;
+  cudaGraphEdgeData edge = {};
+  if (early) {
+    edge.from_port = cudaGraphKernelNodePortProgrammatic;
+    edge.type = cudaGraphDependencyTypeProgrammatic;
+  }
+  const size_t deps = *lane.last ? 1 : 0;
+  cudaGraphNode_t node = nullptr;
+  const cudaError_t e =
+      cudaGraphAddNode(&node, lane.graph, deps ? lane.last : nullptr, deps ? &edge : nullptr, deps, &np);
+  if (e == cudaSuccess) *lane.last = node;
+  return e;
+}
 }  // namespace egh
 
 struct egh_ctx {
@@ -144,15 +179,10 @@ struct egh_batch {
   int dev = 0, nmax = 0, count = 0, piv64 = 0, threads = 0;
   PotrfItem* items = nullptr;  // device list of every (context, frequency) matrix
   int* status = nullptr;       // device, one per item
-  cudaStream_t cap = nullptr;  // capture stream
   cudaGraphExec_t graph = nullptr;
   int graph_launches = 0;      // kernels in one replay of the graph
   cudaEvent_t ev[2] = {};
-  // branches of the contexts' inverses, in order of falling size
-  std::vector<egh_ctx*> by_size;
-  std::vector<cudaStream_t> side;
-  std::vector<cudaEvent_t> ev_join;
-  cudaEvent_t ev_fork = nullptr;
+  std::vector<egh_ctx*> by_size;  // the contexts in order of falling size
   std::string err;
 };
 
@@ -383,7 +413,7 @@ void release_green_buffers(egh_ctx* ctx) {
   ctx->snap = nullptr;
   ctx->gh = nullptr;
   ctx->ghb = nullptr;
-  // graphs captured the ring slots' addresses
+  // the graphs hold the ring slots' addresses
   for (auto& kv : ctx->fd_graphs) cudaGraphExecDestroy(kv.second);
   ctx->fd_graphs.clear();
 }
@@ -395,26 +425,33 @@ SnapOut level_snap(egh_ctx* ctx, int t, int t0, int sbase, int decim) {
   return snap_slot(ctx, sbase + (t - t0) / decim);
 }
 
+// Graph of the FD steps t = ta .. t1-1 of np pairs with tz rows per warp; snap(t): level t's snapshot.
+template <typename F>
+cudaError_t fd_graph(egh_ctx* ctx, int ta, int t1, int np, int tz, F snap, cudaGraphExec_t* exec) {
+  cudaGraph_t graph = nullptr;
+  cudaGraphNode_t last = nullptr;
+  cudaError_t e = cudaGraphCreate(&graph, 0);
+  for (int t = ta; t < t1 && e == cudaSuccess; ++t) {
+    e = launch_fd_step(slot(ctx, t - 1), slot(ctx, t - 2), slot(ctx, t), ctx->coef, ctx->L, ctx->S, np,
+                       snap(t), Lane(graph, &last), tz);
+    count_launches(-1);  // counted at each replay
+  }
+  if (e == cudaSuccess) e = cudaGraphInstantiate(exec, graph, 0);
+  if (graph) cudaGraphDestroy(graph);
+  return e;
+}
+
 // FD steps t = ta .. t1-1 of a chunk whose level t0 sits in ring slot sbase, on the FD stream, as
-// one CUDA graph (captured on first use, then replayed: the kernel nodes' arguments depend only
+// one CUDA graph (built on first use, then replayed: the kernel nodes' arguments depend only
 // on the key, since state slots follow t mod 3 and ring slots follow t - t0).
 egh_status fd_chunk_steps(egh_ctx* ctx, int ta, int t0, int t1, int sbase, int np, int decim) {
   if (ta >= t1) return EGH_OK;
   const auto key = std::make_tuple(ta % 3, ta - t0, t1 - ta, sbase, np, ctx->fd_tz, decim);
   auto it = ctx->fd_graphs.find(key);
   if (it == ctx->fd_graphs.end()) {
-    CK(cudaStreamBeginCapture(ctx->fdst, cudaStreamCaptureModeThreadLocal));
-    cudaError_t e = cudaSuccess;
-    for (int t = ta; t < t1 && e == cudaSuccess; ++t)
-      e = launch_fd_step(slot(ctx, t - 1), slot(ctx, t - 2), slot(ctx, t), ctx->coef, ctx->L,
-                         ctx->S, np, level_snap(ctx, t, t0, sbase, decim), ctx->fdst, ctx->fd_tz);
-    count_launches(-(t1 - ta));  // counted again at each replay
-    cudaGraph_t graph = nullptr;
-    const cudaError_t e2 = cudaStreamEndCapture(ctx->fdst, &graph);
-    if (e == cudaSuccess) e = e2;
     cudaGraphExec_t exec = nullptr;
-    if (e == cudaSuccess) e = cudaGraphInstantiate(&exec, graph, 0);
-    if (graph) cudaGraphDestroy(graph);
+    const cudaError_t e = fd_graph(ctx, ta, t1, np, ctx->fd_tz,
+                                   [&](int t) { return level_snap(ctx, t, t0, sbase, decim); }, &exec);
     if (e != cudaSuccess)
       return fail(ctx, EGH_ECUDA, std::string("FD chunk graph: ") + cudaGetErrorString(e));
     it = ctx->fd_graphs.emplace(key, exec).first;
@@ -426,9 +463,9 @@ egh_status fd_chunk_steps(egh_ctx* ctx, int ta, int t0, int t1, int sbase, int n
 
 // Selective refinement of the mixed precisions, step 1 (queued on `stream` after the inverses):
 // ||Q_k||_F^2 and the power estimate of 1 / lambda_min(Q_k), then their copy to the host buffer.
-cudaError_t refine_estimates(egh_ctx* ctx, cudaStream_t stream) {
-  const cudaError_t e = launch_fro2(ctx->Qh, ctx->nrec, ctx->nf, ctx->fro2, stream);
-  return e ? e : launch_inv_power(ctx->Ph, ctx->nrec, ctx->nf, ctx->fro2 + ctx->nf, stream);
+cudaError_t refine_estimates(egh_ctx* ctx, const Lane& lane) {
+  const cudaError_t e = launch_fro2(ctx->Qh, ctx->nrec, ctx->nf, ctx->fro2, lane);
+  return e ? e : launch_inv_power(ctx->Ph, ctx->nrec, ctx->nf, ctx->fro2 + ctx->nf, lane);
 }
 
 egh_status refine_fetch(egh_ctx* ctx, cudaStream_t stream) {
@@ -731,18 +768,10 @@ namespace {
 egh_status time_fd_steps(egh_ctx* ctx, int np, int tz, int slots, float* best) {
   constexpr int STEPS = 24;
   cudaStream_t fs = ctx->fdst;
-  CK(cudaStreamBeginCapture(fs, cudaStreamCaptureModeThreadLocal));
-  cudaError_t e = cudaSuccess;
-  for (int t = 2; t < 2 + STEPS && e == cudaSuccess; ++t)
-    e = launch_fd_step(slot(ctx, t - 1), slot(ctx, t - 2), slot(ctx, t), ctx->coef, ctx->L, ctx->S, np,
-                       slots ? snap_slot(ctx, t % slots) : SnapOut{nullptr, 0, 0}, fs, tz);
-  count_launches(-STEPS);  // counted at each replay
-  cudaGraph_t graph = nullptr;
-  const cudaError_t e2 = cudaStreamEndCapture(fs, &graph);
-  if (e == cudaSuccess) e = e2;
   cudaGraphExec_t exec = nullptr;
-  if (e == cudaSuccess) e = cudaGraphInstantiate(&exec, graph, 0);
-  if (graph) cudaGraphDestroy(graph);
+  cudaError_t e = fd_graph(ctx, 2, 2 + STEPS, np, tz,
+                           [&](int t) { return slots ? snap_slot(ctx, t % slots) : SnapOut{nullptr, 0, 0}; },
+                           &exec);
   *best = 1e30f;
   for (int rep = 0; rep < 4 && e == cudaSuccess; ++rep) {
     float ms = 0.f;
@@ -1604,12 +1633,6 @@ void egh_batch_destroy(egh_batch* b) {
   cudaSetDevice(b->dev);
   cudaDeviceSynchronize();
   if (b->graph) cudaGraphExecDestroy(b->graph);
-  if (b->cap) cudaStreamDestroy(b->cap);
-  for (cudaStream_t s : b->side)
-    if (s) cudaStreamDestroy(s);
-  for (cudaEvent_t e : b->ev_join)
-    if (e) cudaEventDestroy(e);
-  if (b->ev_fork) cudaEventDestroy(b->ev_fork);
   for (cudaEvent_t e : b->ev)
     if (e) cudaEventDestroy(e);
   cudaFree(b->items);
@@ -1650,17 +1673,11 @@ egh_status egh_batch_create(egh_ctx* const* ctxs, int32_t n, egh_batch** out) {
       for (int k = 0; k < c->nf; ++k, ++o)
         items.push_back(PotrfItem{c->Lh + (size_t)k * c->nrec * c->nrec, c->nrec, b->status + o});
     BCK(cudaMemcpy(b->items, items.data(), sizeof(PotrfItem) * items.size(), cudaMemcpyHostToDevice));
-    BCK(cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking));
     BCK(cudaEventCreate(&b->ev[0]));
     BCK(cudaEventCreate(&b->ev[1]));
     b->by_size = b->ctxs;
     std::stable_sort(b->by_size.begin(), b->by_size.end(),
                      [](const egh_ctx* x, const egh_ctx* y) { return x->nrec > y->nrec; });
-    b->side.assign(b->ctxs.size(), nullptr);
-    b->ev_join.assign(b->ctxs.size(), nullptr);
-    for (cudaStream_t& s : b->side) BCK(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
-    for (cudaEvent_t& e : b->ev_join) BCK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-    BCK(cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming));
     BCK(potrf_many_prepare(b->nmax));
     return EGH_OK;
   };
@@ -1674,35 +1691,47 @@ egh_status egh_batch_create(egh_ctx* const* ctxs, int32_t n, egh_batch** out) {
   return EGH_OK;
 }
 
-// Q -> L copies of every context and one persistent factorisation launch, on `st`, then the
-// contexts' inverses in branches that join `st`.
-static cudaError_t batch_enqueue(egh_batch* b, int threads, cudaStream_t st) {
-  cudaError_t e;
-  for (egh_ctx* c : b->ctxs)
-    if ((e = cudaMemcpyAsync(c->Lh, c->Qh, (size_t)c->nf * c->nrec * c->nrec * sizeof(float2),
-                             cudaMemcpyDeviceToDevice, st)))
+// Graph of the Q -> L copies of every context, one persistent factorisation launch with `threads` per
+// block, and the contexts' inverses.
+static cudaError_t batch_graph(egh_batch* b, int threads, cudaGraphExec_t* exec) {
+  cudaGraph_t g = nullptr;
+  auto build = [&]() -> cudaError_t {
+    cudaError_t e;
+    std::vector<cudaGraphNode_t> copies(b->ctxs.size());
+    for (size_t i = 0; i < b->ctxs.size(); ++i) {
+      const egh_ctx* c = b->ctxs[i];
+      if ((e = cudaGraphAddMemcpyNode1D(&copies[i], g, nullptr, 0, c->Lh, c->Qh,
+                                        (size_t)c->nf * c->nrec * c->nrec * sizeof(float2),
+                                        cudaMemcpyDeviceToDevice)))
+        return e;
+    }
+    cudaGraphNode_t factored = nullptr;
+    if ((e = cudaGraphAddEmptyNode(&factored, g, copies.data(), copies.size())) ||
+        (e = launch_potrf_many(b->items, b->count, b->nmax, std::min(b->count, 2 * 152), threads, b->piv64,
+                               Lane(g, &factored))))
       return e;
-  if ((e = launch_potrf_many(b->items, b->count, b->nmax, std::min(b->count, 2 * 152), threads,
-                             b->piv64, st)))
-    return e;
-  // the mixed precisions' inverse factors, inverses and condition estimates: a branch per context,
-  // largest first (each kernel is a chain of rows or steps that leaves the SMs half idle, so the
-  // contexts' chains run side by side: factor and deblur of patches of 161, 257 and 341 receivers
-  // x 40 frequencies 3.20 ms one after another, 2.70 ms as branches)
-  if ((e = cudaEventRecord(b->ev_fork, st))) return e;
-  for (size_t i = 0; i < b->by_size.size(); ++i) {
-    egh_ctx* c = b->by_size[i];
-    if (!c->Wh) continue;
-    cudaStream_t s = b->side[i];
-    if ((e = cudaStreamWaitEvent(s, b->ev_fork, 0))) return e;
-    if ((e = launch_trtri(c->Lh, c->nrec, c->nf, c->Wh, s))) return e;
-    if ((e = launch_gram_inverse(c->Wh, c->nrec, c->nf, c->Ph, s))) return e;
-    if ((e = launch_cmm_images(c->Ph, c->nrec, c->nf, c->Pimg, s))) return e;
-    if ((e = refine_estimates(c, s))) return e;
-    if ((e = cudaEventRecord(b->ev_join[i], s))) return e;
-    if ((e = cudaStreamWaitEvent(st, b->ev_join[i], 0))) return e;
-  }
-  return cudaSuccess;
+    // the mixed precisions' inverse factors, inverses and condition estimates: a branch per context,
+    // largest first (each kernel is a chain of rows or steps that leaves the SMs half idle, so the
+    // contexts' chains run side by side: factor and deblur of patches of 161, 257 and 341 receivers
+    // x 40 frequencies 3.20 ms one after another, 2.70 ms as branches)
+    for (egh_ctx* c : b->by_size) {
+      if (!c->Wh) continue;
+      cudaGraphNode_t last = factored;
+      const Lane lane(g, &last);
+      if ((e = launch_trtri(c->Lh, c->nrec, c->nf, c->Wh, lane)) ||
+          (e = launch_gram_inverse(c->Wh, c->nrec, c->nf, c->Ph, lane)) ||
+          (e = launch_cmm_images(c->Ph, c->nrec, c->nf, c->Pimg, lane)) || (e = refine_estimates(c, lane)))
+        return e;
+    }
+    return cudaGraphInstantiate(exec, g, 0);
+  };
+  b->graph_launches = 1;
+  for (const egh_ctx* c : b->ctxs) b->graph_launches += c->Wh ? 5 : 0;
+  cudaError_t e = cudaGraphCreate(&g, 0);
+  if (e == cudaSuccess) e = build();
+  count_launches(-b->graph_launches);  // counted at each replay
+  if (g) cudaGraphDestroy(g);
+  return e;
 }
 
 egh_status egh_batch_factor(egh_batch* b, int32_t* bad_ctx, int32_t* bad_freq, void* stream_) {
@@ -1714,36 +1743,27 @@ egh_status egh_batch_factor(egh_batch* b, int32_t* bad_ctx, int32_t* bad_freq, v
   for (egh_ctx* c : b->ctxs)
     if (c->state < ST_HESSIAN) return bfail(b, EGH_ESTATE, "every context needs egh_hessian first");
   if (!b->graph) {
-    // launch shape: time each block size on these matrices and keep the fastest; then capture
-    // the copies and the launch once as a CUDA graph
+    // launch shape: the graph of each block size, timed on these matrices; the fastest is kept
     float best = 1e30f;
-    const long long l0 = launches_so_far();
     for (int th : {256, 512}) {  // (1024 threads leave too few registers for a row per thread)
+      cudaGraphExec_t exec = nullptr;
       float ms = 0.f;
-      for (int rep = 0; rep < 2; ++rep) {
-        BCK(cudaEventRecord(b->ev[0], stream));
-        BCK(batch_enqueue(b, th, stream));
-        BCK(cudaEventRecord(b->ev[1], stream));
-        BCK(cudaEventSynchronize(b->ev[1]));
-        BCK(cudaEventElapsedTime(&ms, b->ev[0], b->ev[1]));
+      cudaError_t e = batch_graph(b, th, &exec);
+      for (int rep = 0; rep < 2 && e == cudaSuccess; ++rep)
+        if (!(e = cudaEventRecord(b->ev[0], stream)) && !(e = cudaGraphLaunch(exec, stream)) &&
+            !(e = cudaEventRecord(b->ev[1], stream)) && !(e = cudaEventSynchronize(b->ev[1])))
+          e = cudaEventElapsedTime(&ms, b->ev[0], b->ev[1]);
+      if (e != cudaSuccess) {
+        if (exec) cudaGraphExecDestroy(exec);
+        return bfail(b, EGH_ECUDA, std::string("batch graph: ") + cudaGetErrorString(e));
       }
       if (ms < best) {
+        std::swap(exec, b->graph);
         best = ms;
         b->threads = th;
       }
+      if (exec) cudaGraphExecDestroy(exec);
     }
-    count_launches(-(int)(launches_so_far() - l0));  // tuning launches are not part of the factorisation
-    const long long l1 = launches_so_far();
-    BCK(cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal));
-    cudaError_t e = batch_enqueue(b, b->threads, b->cap);
-    b->graph_launches = (int)(launches_so_far() - l1);
-    count_launches(-b->graph_launches);  // counted at each replay
-    cudaGraph_t g = nullptr;
-    const cudaError_t e2 = cudaStreamEndCapture(b->cap, &g);
-    if (e == cudaSuccess) e = e2;
-    if (e == cudaSuccess) e = cudaGraphInstantiate(&b->graph, g, 0);
-    if (g) cudaGraphDestroy(g);
-    if (e != cudaSuccess) return bfail(b, EGH_ECUDA, std::string("batch graph: ") + cudaGetErrorString(e));
   }
   BCK(cudaGraphLaunch(b->graph, stream));
   count_launches(b->graph_launches);

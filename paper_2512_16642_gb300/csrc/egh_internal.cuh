@@ -23,6 +23,8 @@
 #include <complex>
 #include <cstdint>
 #include <string>
+#include <tuple>
+#include <utility>
 #include <vector>
 
 namespace egh {
@@ -51,6 +53,32 @@ cudaError_t allow_block_smem() {
     dynamic.store(d = kBlockSmem - (int)fa.sharedSizeBytes, std::memory_order_relaxed);
   }
   return cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, d);
+}
+
+// Where a launch goes: to a stream, or into a graph under construction, after the node *last (if it is
+// not null), which the new one then replaces.  Graphs are built from nodes and not captured: while a
+// stream captures, any host thread's cudaDeviceSynchronize fails and ends the capture, and contexts of
+// different threads are independent.
+struct Lane {
+  Lane(cudaStream_t s) : stream(s) {}
+  Lane(cudaGraph_t g, cudaGraphNode_t* l) : graph(g), last(l) {}
+  cudaStream_t stream = nullptr;
+  cudaGraph_t graph = nullptr;
+  cudaGraphNode_t* last = nullptr;
+};
+// early: programmatic launch, the kernel may start when the one before it allows it (griddepcontrol)
+cudaError_t lane_launch(const Lane& lane, const void* kernel, dim3 grid, dim3 block, size_t smem,
+                        void** args, bool early);
+template <typename... P, typename... A>
+cudaError_t launch_on(const Lane& lane, bool early, void (*kernel)(P...), dim3 grid, dim3 block,
+                      size_t smem, const A&... a) {
+  std::tuple<P...> p(a...);  // converted to the kernel's parameter types
+  return std::apply(
+      [&](auto&... x) {
+        void* args[] = {const_cast<void*>(static_cast<const void*>(&x))...};
+        return lane_launch(lane, (const void*)kernel, grid, block, smem, args, early);
+      },
+      p);
 }
 
 struct Stencil {
@@ -95,7 +123,7 @@ struct FdAux {
 // tz: rows per warp (12, 16, 18, 20, 24 or 32; 0 = default)
 cudaError_t launch_fd_step(const float2* ucur, const float2* uprev, float2* unext,
                            const float2* coef, const Layout& L, const Stencil& S, int npairs,
-                           const SnapOut& so, cudaStream_t st, int tz, const FdAux* aux = nullptr);
+                           const SnapOut& so, const Lane& lane, int tz, const FdAux* aux = nullptr);
 int fd_rows_one_wave(const Layout& L, int npairs);
 int fd_rows_per_warp_default();
 cudaError_t fd_prepare(int nf);  // once per context, before any capture
@@ -212,7 +240,7 @@ struct PotrfItem {
 };
 cudaError_t potrf_many_prepare(int nmax);
 cudaError_t launch_potrf_many(const PotrfItem* items, int count, int nmax, int blocks, int threads,
-                              int piv64, cudaStream_t st);
+                              int piv64, const Lane& lane);
 cudaError_t launch_potrf(float2* Lh, int n, int nf, int* status, cudaStream_t st, int piv64);
 
 // ---- deblur.cu --------------------------------------------------------------------------------
@@ -231,12 +259,12 @@ size_t trace_scratch_bytes(int nf, long long ntr, int nt_d);
 size_t trace_scratch_most(int nf, int nrec, int nt_d);
 cudaError_t launch_trsm(const float2* Lh, int n, int nf, float2* Dh, int ns, cudaStream_t st);
 // W = L^{-1} per frequency
-cudaError_t launch_trtri(const float2* Lh, int n, int nf, float2* Wh, cudaStream_t st);
+cudaError_t launch_trtri(const float2* Lh, int n, int nf, float2* Wh, const Lane& lane);
 // Q^{-1}_k = W_k^H W_k (dense) from the inverse factors
-cudaError_t launch_gram_inverse(const float2* Wh, int n, int nf, float2* Ph, cudaStream_t st);
+cudaError_t launch_gram_inverse(const float2* Wh, int n, int nf, float2* Ph, const Lane& lane);
 // operand images of A_k (n x n complex64 per frequency) for launch_cmm_tc: cmm_image_bytes(n, nf)
 size_t cmm_image_bytes(int n, int nf);
-cudaError_t launch_cmm_images(const float2* A, int n, int nf, unsigned char* img, cudaStream_t st);
+cudaError_t launch_cmm_images(const float2* A, int n, int nf, unsigned char* img, const Lane& lane);
 // C_k = A_k B_k (complex, A_k n x n as images, B_k and C_k n x ld, row-major; C must not alias B) on
 // the tensor cores with FP32-class products (three-term bf16 splits), for the nk frequencies of the
 // device list kl (all when null); err: the flag a bounded wait sets (solve_tc.cu)
@@ -253,9 +281,9 @@ inline bool prec_mixed(int prec) { return prec == EGH_PREC_MIXED || prec == EGH_
 cudaError_t launch_add_correction(float2* X, const float2* R, long long m, int nk, cudaStream_t st,
                                   const int* kl = nullptr);
 // ||Q_k||_F^2 per frequency (FP64 sums) into d_out[nf]
-cudaError_t launch_fro2(const float2* Qh, int n, int nf, double* d_out, cudaStream_t st);
+cudaError_t launch_fro2(const float2* Qh, int n, int nf, double* d_out, const Lane& lane);
 // lambda_max(P_k) = 1 / lambda_min(Q_k), P_k = Q_k^{-1}, by power iteration (from below) into lam[nf]
-cudaError_t launch_inv_power(const float2* Ph, int n, int nf, double* lam, cudaStream_t st);
+cudaError_t launch_inv_power(const float2* Ph, int n, int nf, double* lam, const Lane& lane);
 // Condition bound of a factorisation from ||Q||_F^2, the power estimate of 1/lambda_min (with a
 // margin for its approach from below) and, when known (> 0), mu <= lambda_min.
 inline double cond_bound(double fro2, double inv_lmin, double mu) {

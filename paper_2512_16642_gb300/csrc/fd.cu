@@ -470,7 +470,7 @@ cudaError_t fd_prepare(int nf) {
 
 cudaError_t launch_fd_step(const float2* ucur, const float2* uprev, float2* unext,
                            const float2* coef, const Layout& L, const Stencil& S, int npairs,
-                           const SnapOut& so, cudaStream_t st, int tz, const FdAux* aux) {
+                           const SnapOut& so, const Lane& lane, int tz, const FdAux* aux) {
   if (L.PX % 64 != 0) return cudaErrorInvalidValue;
   if (tz <= 0) tz = EGH_FD_TZDEF;
   // cumulative weights C_j = sum_{k>=j} c_k of the first-difference form
@@ -487,28 +487,18 @@ cudaError_t launch_fd_step(const float2* ucur, const float2* uprev, float2* unex
   const dim3 blk(32, npairs);
   const size_t smem = fd_block_smem(npairs);
   const int org = (int)L.org;
-  cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute at;
-  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at.val.programmaticStreamSerializationAllowed = 1;
-  cfg.blockDim = blk;
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cfg.attrs = &at;
   // Programmatic launch hides most of a launch's and a first row's latency, which is much of a small
   // grid's step (101x101 grid, 21 receivers x 1000 steps: 10.8 -> 9.5 ms), and helps where no
   // snapshot is written for a transform beside (decimated update 154.7 -> 152.1 ms, modelling of 23
   // shots 34.4 -> 26.7 ms); beside the transform, a full grid's early blocks take what it would use
   // (layered: Green stage 957 -> 979 ms).
-  cfg.numAttrs = so.lvl == nullptr || (long long)(L.PX / 64) * ((L.NZ + tz - 1) / tz) < 152 ? 1 : 0;
+  const bool early = so.lvl == nullptr || (long long)(L.PX / 64) * ((L.NZ + tz - 1) / tz) < 152;
+  const dim3 grid(L.PX / 64, (L.NZ + tz - 1) / tz + (aux && aux->traces ? 1 : 0));
   switch (tz) {
-#define EGH_FD_CASE(T)                                                                          \
-  case T:                                                                                       \
-    cfg.gridDim = dim3(L.PX / 64, (L.NZ + T - 1) / T + (aux && aux->traces ? 1 : 0));            \
-    return aux ? cudaLaunchKernelEx(&cfg, k_fd_step<T, true>, ucur, uprev, unext, coef, L.NZ,    \
-                                    L.NX, L.PX, org, L.F, C, so, *aux)                           \
-               : cudaLaunchKernelEx(&cfg, k_fd_step<T, false>, ucur, uprev, unext, coef, L.NZ,   \
-                                    L.NX, L.PX, org, L.F, C, so, FdAux{});
+#define EGH_FD_CASE(T)                                                                                  \
+  case T:                                                                                               \
+    return launch_on(lane, early, aux ? k_fd_step<T, true> : k_fd_step<T, false>, grid, blk, smem, ucur, \
+                     uprev, unext, coef, L.NZ, L.NX, L.PX, org, L.F, C, so, aux ? *aux : FdAux{});
     EGH_FD_CASE(12)
     EGH_FD_CASE(16)
     EGH_FD_CASE(18)
@@ -519,7 +509,6 @@ cudaError_t launch_fd_step(const float2* ucur, const float2* uprev, float2* unex
     default:
       return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------------------------

@@ -339,10 +339,9 @@ __global__ void __cluster_dims__(FR_CL, 1, 1) __launch_bounds__(FR_THREADS)
   }
 }
 
-cudaError_t launch_fro2(const float2* Qh, int n, int nf, double* d_out, cudaStream_t st) {
+cudaError_t launch_fro2(const float2* Qh, int n, int nf, double* d_out, const Lane& lane) {
   count_launches(1);
-  k_fro2<<<nf * FR_CL, FR_THREADS, 0, st>>>(Qh, n, d_out);
-  return cudaGetLastError();
+  return launch_on(lane, false, k_fro2, nf * FR_CL, FR_THREADS, 0, Qh, n, d_out);
 }
 
 // Largest eigenvalue of Q_k^{-1} (the dense inverse P_k) by 40 steps of power iteration in FP32:
@@ -420,7 +419,7 @@ __global__ void __cluster_dims__(IP_CL, 1, 1) __launch_bounds__(IP_THREADS)
   if (rank == 0 && tid == 0) lam[blockIdx.x / IP_CL] = norm;
 }
 
-cudaError_t launch_inv_power(const float2* Ph, int n, int nf, double* lam, cudaStream_t st) {
+cudaError_t launch_inv_power(const float2* Ph, int n, int nf, double* lam, const Lane& lane) {
   // rows of P beside the two vectors in at most 200 KB of a block's shared memory
   const size_t vec = 2 * sizeof(float2) * (size_t)n, cap = 200 * 1024;
   const int share = (n + IP_CL - 1) / IP_CL;
@@ -429,8 +428,7 @@ cudaError_t launch_inv_power(const float2* Ph, int n, int nf, double* lam, cudaS
   const cudaError_t e = allow_block_smem<k_inv_power>();
   if (e != cudaSuccess) return e;
   count_launches(1);
-  k_inv_power<<<nf * IP_CL, IP_THREADS, smem, st>>>(Ph, n, cached, lam);
-  return cudaGetLastError();
+  return launch_on(lane, false, k_inv_power, nf * IP_CL, IP_THREADS, smem, Ph, n, cached, lam);
 }
 
 // Largest eigenvalue of each Hermitian H_k by power iteration in FP64 (fixed 300 iterations, Rayleigh

@@ -317,10 +317,10 @@ size_t cmm_image_bytes(int n, int nf) {
   return (size_t)nf * ((n + CM_M - 1) / CM_M) * ((n + CM_K - 1) / CM_K) * CM_AST;
 }
 
-cudaError_t launch_cmm_images(const float2* A, int n, int nf, unsigned char* img, cudaStream_t st) {
+cudaError_t launch_cmm_images(const float2* A, int n, int nf, unsigned char* img, const Lane& lane) {
   count_launches(1);
-  k_cmm_images<<<dim3((n + CM_K - 1) / CM_K, (n + CM_M - 1) / CM_M, nf), 256, 0, st>>>(A, n, img);
-  return cudaGetLastError();
+  return launch_on(lane, false, k_cmm_images, dim3((n + CM_K - 1) / CM_K, (n + CM_M - 1) / CM_M, nf), 256, 0, A,
+                   n, img);
 }
 
 cudaError_t launch_cmm_tc(const unsigned char* Aimg, int n, int nk, const float2* B, int ld, float2* C,

@@ -258,3 +258,42 @@ def test_batch_of_a_few_receivers(nz, nx, nrec, batch):
                      np.arange(nrec, dtype=np.int32), np.array([8.0]), dft_chunk=32) as ctx:
         ctx.green(torch.full((nz, nx), 2000.0, device="cuda"))
         assert ctx.stats()["batch_receivers"] == batch
+
+
+def test_threads_that_wait_for_the_device():
+    """A host thread that waits for the device and one whose contexts run their first Green stages and
+    batched factorisations (which build their graphs then) leave each other alone."""
+    import torch
+    from paper_2512_16642_gb300 import egh
+
+    done = threading.Event()
+    vel = torch.full((60, 300), 2000.0, device="cuda")
+
+    def wait():
+        while not done.is_set():
+            torch.cuda.synchronize()
+
+    def work():
+        try:
+            first = None
+            for _ in range(8):
+                ctxs = [egh.Context(60, 300, 10.0, 10.0, 10, 1e-3, 1e-3, 200, np.zeros(n, np.int32),
+                                    np.arange(n, dtype=np.int32), np.array([10.0, 20.0]), fd_kernel=2,
+                                    dft_chunk=64, precision=1, gram_splits=2) for n in (12, 33)]
+                try:
+                    for c in ctxs:
+                        c.green(vel)
+                        c.hessian(egh.EGH_MU_REL_MEANDIAG, 1e-2)
+                    with egh.Batch(ctxs) as b:
+                        b.factor()
+                        b.factor()
+                    out = [ctxs[0].get_green()] + [c.get_hessian(True) for c in ctxs]
+                finally:
+                    for c in ctxs:
+                        c.close()
+                first = first or out
+                assert all(np.array_equal(a, w) for a, w in zip(out, first))
+        finally:
+            done.set()
+
+    _in_threads(wait, work)
