@@ -980,17 +980,23 @@ egh_status green_run(egh_ctx* ctx, const float* vel, cudaStream_t stream, const 
       const int expire = ctx->expire[0] > 0 ? 1 : 0;
       ctx->expire[0] -= expire;
       // Beside the next chunk's FD steps the transform takes one CTA per SM (sized to fit next
-      // to two FD CTAs of a full batch); the record's last chunk runs alone and takes three.  With
+      // to two FD CTAs of a full batch); the record's last chunk runs alone and asks for three.  With
       // more than 32 frequencies one CTA per SM no longer keeps pace with the FD steps (measured:
       // 40 frequencies on the salt grid, transform 5.9 s against FD steps 5.1 s per patch), so
       // there the transform takes one CTA per tile and fills the SMs between FD launches.
       const bool alone = b0 + B >= ctx->nrec && c == nchunk - 1;
       const bool slim = dft_ncomp(ctx->nf) <= 64 && ctx->fd_kernel == 2;
+      // the last chunk finishes the totals where it reads them (the Gram's operands) or writes them
+      // first; else they are scaled in a pass of their own
+      const bool finish = m1 == ntd && (ctx->ghb || m0 == 0);
       const long long beside = fd_sm_smem((std::min(B, ctx->nrec) + 1) / 2, ctx->fd_tz);
       CK(launch_dft_tc(ctx->tmap, twt, ctx->nf, sbase, m1 - m0, m0, L, ctx->gh, ctx->ghb,
-                       m1 == ntd ? 1 : 0, b0, nb, ctx->nrec, ctx->d_err, expire,
+                       finish ? 1 : 0, b0, nb, ctx->nrec, ctx->d_err, expire,
                        alone || ctx->fd_kernel == 3 ? 3 : slim ? 1 : 0, (alone || !slim) ? 0 : beside,
                        down, ctx->side));
+      if (m1 == ntd && !finish)
+        CK(launch_scale_totals(ctx->gh + (size_t)b0 * ctx->nf * 2 * L.G, (long long)nb * ctx->nf * 2 * L.G, down,
+                               alone || !slim ? 8 : 1, ctx->side));
       CK(cudaEventRecord(ctx->ev_dft[2 * g + 1], ctx->side));
       CK(cudaEventRecord(ctx->dft_done[g & 1], ctx->side));
     }

@@ -146,6 +146,8 @@ cudaError_t launch_dft_tc(const CUtensorMap& tmap, const unsigned char* twt, int
                           int kcount, int n0, const Layout& L, float* gh, __nv_bfloat16* ghb,
                           int last, int rec0, int nvalid, int nrec_all, int* err, int expire,
                           int per_sm, long long beside_smem, float down, cudaStream_t st);
+// n floats (a multiple of four) times scale, in place
+cudaError_t launch_scale_totals(float* g, long long n, float scale, int per_sm, cudaStream_t st);
 // dynamic shared memory of one k_fd_step CTA for npairs receiver pairs
 int fd_block_smem(int npairs);
 // shared memory (reserved parts included) of the k_fd_step CTAs of npairs pairs and tz rows per
