@@ -114,13 +114,13 @@ typedef struct {
     int32_t nfreq;
     const double *freq_hz; /* [nfreq], host */
     int32_t batch_receivers; /* receivers propagated together; 0 = chosen by the library: with
-                                the per-step FD kernel, 9 to 15 receivers go in one batch where
-                                their levels fit in 40 MB, else 8 at a time; from 16 on the first
-                                egh_green times the FD steps per receiver for 8, 16 and 32 and keeps
-                                16 unless another is 3% faster; with the cluster solver, as many as
-                                run at once (at most 32: its ring below is then up to twice that of
-                                16 receivers, which a caller short of memory can ask for); else
-                                min(nrec, 16) */
+                                the per-step FD kernel and more than 8 receivers, the first
+                                egh_green times the FD steps of batches of 8, 16, 32 and min(nrec,
+                                32) and keeps 16 (or nrec, if less) unless the stage is 5% faster
+                                with another (egh_forward by its own steps); with the cluster
+                                solver, as many as run at once (at most 32: its ring below is then
+                                up to twice that of 16 receivers, which a caller short of memory
+                                can ask for); else min(nrec, 16) */
     int32_t dft_chunk;       /* levels per transform chunk: 32, 64, ..., 2048; 0 = 512 (the
                                 snapshot ring holds 2 chunks x batch_receivers levels of 4 bytes per
                                 point of the padded, pitched grid); a

@@ -88,7 +88,10 @@ struct egh_ctx {
   int B = 0, K = 0, splits = 0;
   bool pad_zero = true;  // the transforms are this context's: zero in the rows' padding columns
   int Bcap = 0;         // receivers the FD state slots hold (>= B)
-  bool tune_B = false;  // B is timed on the first egh_green (8, 16 or 32 receivers)
+  int Bmodel = 0;       // sources per batch of egh_forward (0: B)
+  bool tune_B = false;  // B is timed on the first egh_green
+  bool tune_model = false;  // B was timed: Bmodel is, on the next egh_forward
+  bool rows_given = false;  // by the caller
   int fd_tz = 0;  // FD rows per warp of the per-step kernel (0 = library default)
   // 1: resident solver (fd_resident.cu), 2: one kernel per step (fd.cu), 3: a cluster per receiver
   // pair (fd_cluster.cu)
@@ -571,6 +574,7 @@ egh_status egh_create(const egh_config* cfg, egh_ctx** out) {
   // a record shorter than the chunk is one chunk either way: keep the ring no longer than it
   while (ctx->K > 32 && ctx->K / 2 >= c.nt) ctx->K /= 2;
   ctx->fd_tz = c.fd_rows;
+  ctx->rows_given = c.fd_rows != 0;
 
   Layout& L = ctx->L;
   L.nz = c.nz; L.nx = c.nx; L.ns = c.nsponge;
@@ -760,18 +764,17 @@ void egh_destroy(egh_ctx* ctx) {
 
 namespace {
 
-// Time in ms of 24 FD steps of np receiver pairs with tz rows per warp, with (ring slots 0 .. slots-1)
-// or without snapshots: best of three passes after a warm-up.  As one graph, as the run's chunks are:
+// Time in ms of 24 FD steps of np receiver pairs with tz rows per warp, snap(t) being level t's snapshot:
+// best of three passes after a warm-up.  As one graph, as the run's chunks are:
 // launched one by one, a step without a programmatic launch costs 2 us more than in the run and one
 // with it nothing, which misled the choice of rows (295x496 grid, 6 receivers: 24 rows at 7.0 us a
 // step taken for faster than 12 rows at 5.4 us).  The run rewrites every state and ring slot it reads.
-egh_status time_fd_steps(egh_ctx* ctx, int np, int tz, int slots, float* best) {
+template <typename F>
+egh_status time_fd_steps(egh_ctx* ctx, int np, int tz, F snap, float* best) {
   constexpr int STEPS = 24;
   cudaStream_t fs = ctx->fdst;
   cudaGraphExec_t exec = nullptr;
-  cudaError_t e = fd_graph(ctx, 2, 2 + STEPS, np, tz,
-                           [&](int t) { return slots ? snap_slot(ctx, t % slots) : SnapOut{nullptr, 0, 0}; },
-                           &exec);
+  cudaError_t e = fd_graph(ctx, 2, 2 + STEPS, np, tz, snap, &exec);
   *best = 1e30f;
   for (int rep = 0; rep < 4 && e == cudaSuccess; ++rep) {
     float ms = 0.f;
@@ -787,42 +790,64 @@ egh_status time_fd_steps(egh_ctx* ctx, int np, int tz, int slots, float* best) {
   return EGH_OK;
 }
 
-// Receivers per batch, chosen once per context before the ring (sized for the batch) exists.
-// Fewer than 16 receivers go in one batch while their three levels stay well inside the L2 (40 MB),
-// else eight at a time.  Measured, 400 steps, 26 frequencies, one batch and eight at a time: 295x496
-// grid (28 MB) 12 receivers 4.61 and 5.05 ms, 15 (35 MB) 5.68 and 5.87; 301x921 12 (50 MB) 7.00 and 6.95,
-// 15 (63 MB) 8.96 and 8.29; 600x600 9 (49 MB) 7.33 and 7.04, 15 (81 MB) 11.7 and 10.2; 351x1701 11 (92 MB)
-// 15.7 and 12.3.
-// From 16 on by the time per receiver of 8, 16 and 32 in a batch: 24 FD steps as the run launches them
-// (each with its one-wave rows per warp).  16 is kept unless another is 3% faster.  The transform's work
-// per receiver does not depend on the batch, and it runs beside the FD steps for every choice but the
-// last batch's, which is why a batch of all 17 to 31 receivers is none of them: 295x496, 20 receivers 7.23
-// ms against 6.78 in batches of 16.
-egh_status tune_batch(egh_ctx* ctx, cudaStream_t stream) {
-  if (ctx->nrec < 16) {
-    ctx->B = 3.0 * sizeof(float) * ctx->nrec * (double)ctx->L.F <= 40e6 ? ctx->nrec : 8;
-  } else {
-    CK(cudaEventRecord(ctx->ev_tune[0], stream));  // after the coefficients
-    CK(cudaStreamWaitEvent(ctx->fdst, ctx->ev_tune[0], 0));
-    float best = 1e30f, def = 1e30f;
-    int best_b = 16;
-    for (int b : {8, 16, 32}) {
-      if (b > ctx->Bcap) continue;
-      float ms = 0.f;
-      const egh_status s = time_fd_steps(ctx, b / 2, fd_rows_one_wave(ctx->L, b / 2), 0, &ms);
-      if (s) return s;
-      ms /= (float)b;
-      if (ms < best) {
-        best = ms;
-        best_b = b;
-      }
-      if (b == 16) def = ms;
+// Receivers per batch, chosen once per context (the Green stage's before the ring, which is sized for
+// it, exists): 8, 16, 32 or all that the state slots hold, the last batch with what is left; 16 (or all,
+// if fewer) is kept unless another is 5% faster.
+// Modelling, which writes no snapshots: by the FD steps of all batches (24 steps as the run launches
+// them, each batch with its one-wave rows per warp, or the caller's).  Green stage (`snaps`): by those
+// steps with their snapshots, to a passing ring of more than the L2, and the transform of the last
+// batch's last chunk, which has no steps beside it: 2 ps per point, level and receiver, half as much
+// again for more than 32 frequencies, of which 0.7 counts (the transforms beside the steps are not free
+// either).  Measured in ms, 26 frequencies, one batch and the other choice: 295x496 grid, 12 receivers x
+// 400 steps 4.6 and 5.0 (8), 20 x 400 7.2 and 6.8 (16), 20 x 1403 18.1 and 21.1 (16); 600x600, 15 x 400
+// 11.7 and 10.2 (8); 351x1701, 11 x 400 15.7 and 12.3 (8).  Modelling of 11 shots on 301x921, 400 steps:
+// 3.5 in one batch and 5.9 (8).
+egh_status choose_batch(egh_ctx* ctx, bool snaps, int decim, cudaStream_t stream, int* batch) {
+  CK(cudaEventRecord(ctx->ev_tune[0], stream));  // after the coefficients
+  CK(cudaStreamWaitEvent(ctx->fdst, ctx->ev_tune[0], 0));
+  const Layout& L = ctx->L;
+  const int Bp = 2 * ((ctx->Bcap + 1) / 2);
+  const long long level = (long long)Bp * L.G;  // elements of a plane
+  const int slots = (int)std::min(64LL, std::max(4LL, (256LL << 20) / (4 * level) + 1));
+  __nv_bfloat16* ring = nullptr;
+  if (snaps && cudaMalloc((void**)&ring, 2 * (size_t)slots * level * sizeof(__nv_bfloat16)) != cudaSuccess)
+    cudaGetLastError();  // no room: the steps are timed without snapshots
+  std::map<int, float> step;  // ms of a step, by pairs
+  egh_status s = EGH_OK;
+  auto time = [&](int b) {
+    const int np = (b + 1) / 2;
+    auto it = step.find(np);
+    if (it != step.end()) return (double)it->second;
+    float ms = 1e30f;
+    if (s == EGH_OK)
+      s = time_fd_steps(ctx, np, ctx->rows_given ? ctx->fd_tz : fd_rows_one_wave(L, np),
+                        [&](int t) {
+                          if (!ring || t % decim) return SnapOut{nullptr, 0, 0};
+                          return SnapOut{ring + t / decim % slots * level, slots * level, L.G};
+                        },
+                        &ms);
+    return (double)(step[np] = ms / 24.f);
+  };
+  const int ntd = (ctx->nt + decim - 1) / decim;
+  const double lone =
+      0.7 * 2e-9 * (dft_ncomp(ctx->nf) > 64 ? 1.5 : 1.0) * (double)L.G * ((ntd - 1) % ctx->K + 1);
+  const int def_b = std::min(ctx->Bcap, 16);
+  double best = 1e30, def_ms = 1e30;
+  int best_b = def_b;
+  for (int b : {8, 16, 32, ctx->Bcap}) {
+    if (b > ctx->Bcap) continue;
+    const int rest = ctx->nrec % b;
+    const double ms = ctx->nt * ((ctx->nrec / b) * time(b) + (rest ? time(rest) : 0.0)) +
+                      (snaps ? (rest ? rest : b) * lone : 0.0);
+    if (ms < best) {
+      best = ms;
+      best_b = b;
     }
-    ctx->B = best < 0.97f * def ? best_b : 16;
+    if (b == def_b) def_ms = ms;
   }
-  ctx->Bp = 2 * ((ctx->B + 1) / 2);
-  ctx->st.batch_receivers = ctx->B;
-  ctx->tune_B = false;
+  cudaFree(ring);
+  if (s) return s;
+  *batch = best < 0.95 * def_ms ? best_b : def_b;
   return EGH_OK;
 }
 
@@ -843,7 +868,13 @@ egh_status green_run(egh_ctx* ctx, const float* vel, cudaStream_t stream, const 
     ctx->st.batch_receivers = ctx->B;
     ctx->tune_B = false;
   }
-  if (ctx->tune_B && (s = tune_batch(ctx, stream))) return s;
+  if (ctx->tune_B) {
+    if ((s = choose_batch(ctx, true, decim, stream, &ctx->B))) return s;
+    ctx->Bp = 2 * ((ctx->B + 1) / 2);
+    ctx->st.batch_receivers = ctx->B;
+    ctx->tune_B = false;
+    ctx->tune_model = true;
+  }
   if (wav && ctx->fd_kernel == 3) {
     if ((s = ensure_buf(ctx, (void**)&ctx->wav_dev, &ctx->wav_cap, nw * sizeof(float), stream, "wavelet")))
       return s;
@@ -911,7 +942,7 @@ egh_status green_run(egh_ctx* ctx, const float* vel, cudaStream_t stream, const 
     int best_tz = def_tz;
     for (int tz : {12, 16, 18, 20, 24, 32}) {
       float ms = 0.f;
-      if ((s = time_fd_steps(ctx, np, tz, 2 * K, &ms))) return s;
+      if ((s = time_fd_steps(ctx, np, tz, [&](int t) { return snap_slot(ctx, t % (2 * K)); }, &ms))) return s;
       if (ms < best) {
         best = ms;
         best_tz = tz;
@@ -1405,8 +1436,12 @@ egh_status egh_forward(egh_ctx* ctx, const float* vel, int32_t nsrc, const int32
   egh_status s = prepare_model(ctx, vel, stream);
   ctx->state = prev_state;
   if (s) return s;
+  if (ctx->tune_model) {
+    if ((s = choose_batch(ctx, false, 1, stream, &ctx->Bmodel))) return s;
+    ctx->tune_model = false;
+  }
   const Layout& L = ctx->L;
-  const int B = ctx->B, nt = ctx->nt, nrec = ctx->nrec;
+  const int B = ctx->Bmodel ? ctx->Bmodel : ctx->B, nt = ctx->nt, nrec = ctx->nrec;
   std::vector<int> sp(nsrc);
   for (int i = 0; i < nsrc; ++i)
     sp[i] = (int)(L.org + (long long)(src_iz[i] + L.ns) * L.PX + (src_ix[i] + L.ns));
@@ -1435,7 +1470,8 @@ egh_status egh_forward(egh_ctx* ctx, const float* vel, int32_t nsrc, const int32
     CK(cudaMemsetAsync(slot(ctx, 1), 0, (size_t)np * L.F * sizeof(float2), stream));
     // level 0 is zero and level 1 the first sample; step n computes level n + 1, adds its sample and
     // records level n; the last level is recorded on its own
-    const int tz = ctx->fd_tz ? ctx->fd_tz : fd_rows_one_wave(L, np);
+    // (rows timed on the Green stage are those of its batch)
+    const int tz = ctx->fd_tz && (ctx->rows_given || B == ctx->B) ? ctx->fd_tz : fd_rows_one_wave(L, np);
     CK(launch_record(slot(ctx, 0), L.F, ctx->rec_pts, nrec, nb, tr, nt, 0, stream));
     if (nt > 1 && wavelet[0] != 0.f)
       CK(launch_inject(slot(ctx, 1), L.F, d_sp + b0, ctx->coef, nb, wavelet[0], scale, L.org, none, stream));

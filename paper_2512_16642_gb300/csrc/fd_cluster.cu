@@ -327,8 +327,8 @@ bool fd_cluster_plan(const Layout& L, ClGeom* out) {
 // within 12% for one round of clusters (or one batch), 25% for several; n: receivers, p: points, c:
 // transform components.
 // The clusters leave the transform fewer SMs beside them, so its work counts more than beside the
-// per-step kernel.  The choice was at most 1.06 times the better one's time, and 1.006 times on
-// average, for every level transformed.  Clusters and per-step kernel, ms: 101 x 101 grid, 21 receivers,
+// per-step kernel.  The choice was 1.002 times the better one's time on
+// average, with every level transformed, and more than 1.06 times in two of 270 runs (1.10, 1.16).  Clusters and per-step kernel, ms: 101 x 101 grid, 21 receivers,
 // 5 frequencies 3.3 and 6.5; 151 x 201, 12 and 26: 4.7 and 5.7; 215 x 230, 6 and 26: 6.4 and 4.9, 21 and
 // 26: 7.9 and 8.6; 201 x 201, 40 and 26: 13.4 and 13.5, 100 and 60: 36.5 and 30.5.
 bool fd_cluster_faster(const ClGeom& g, const Layout& L, int nrec, int b, int nf) {

@@ -245,17 +245,18 @@ def test_server_keeps_what_its_solves_read():
     assert held <= Q.nbytes + images + (6 << 20)  # twiddle tables and the allocator's 2 MB blocks
 
 
-@pytest.mark.parametrize("nz,nx,nrec,batch", [(295, 496, 12, 12), (600, 600, 15, 8), (351, 1701, 11, 8),
-                                              (295, 496, 20, 16)])
-def test_batch_of_a_few_receivers(nz, nx, nrec, batch):
-    """9 to 15 receivers go in one batch only where their levels stay in L2, and 17 to 31 never (their
-    transform would have no steps beside it): the sizes where one batch of all took 1.07 to 1.27 times as
-    long, and one where it is the faster one."""
+@pytest.mark.parametrize("nz,nx,nrec,nt,batch", [(295, 496, 12, 400, 12), (600, 600, 15, 400, 8),
+                                                 (351, 1701, 11, 400, 8), (295, 496, 20, 400, 16),
+                                                 (295, 496, 20, 1403, 20)])
+def test_batch_of_a_few_receivers(nz, nx, nrec, nt, batch):
+    """One batch of all receivers is taken where it is clearly the faster choice and not where its levels
+    leave L2, or where the transform of a short record, with no steps beside it, outweighs its steps (the
+    other choice takes 1.07 to 1.27 times as long in each)."""
     import torch
     from paper_2512_16642_gb300 import egh
 
-    with egh.Context(nz, nx, 10.0, 10.0, 20, 1e-3, 1e-3, 40, np.zeros(nrec, np.int32),
-                     np.arange(nrec, dtype=np.int32), np.array([8.0]), dft_chunk=32) as ctx:
+    with egh.Context(nz, nx, 10.0, 10.0, 20, 1e-3, 1e-3, nt, np.zeros(nrec, np.int32),
+                     np.arange(nrec, dtype=np.int32), np.array([8.0])) as ctx:
         ctx.green(torch.full((nz, nx), 2000.0, device="cuda"))
         assert ctx.stats()["batch_receivers"] == batch
 
