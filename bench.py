@@ -38,8 +38,8 @@ FALLBACK_HBM_GBS = 6800.0
 # DRAM traffic (read + write bytes) per launch of the FD step and of the transform from the
 # committed ncu capture (profiles/), valid only for the kernel sources it was taken from (sha256
 # of csrc/fd.cu); None until a capture exists.
-KERNEL_TRAFFIC = {"fd_sha256": "e7df73ae2e26ed56e518dfe476b7609fd9ee8996e813bc820c0373b5a0168efc",
-                  "k_fd_step": 31.63e6,   # 1.22 MB read + 30.42 MB write per launch (18 rows per warp)
+KERNEL_TRAFFIC = {"fd_sha256": "af4de6a8965a7f85c737e0b2d5454954c933d843a3d0dfb36da0df6b5161319f",
+                  "k_fd_step": 31.58e6,   # 1.21 MB read + 30.37 MB write per launch (18 rows per warp)
                   "k_dft_tc": 48.10e9,    # 45.78 GB read + 2.33 GB write per 2048-level launch
                   "gram_sha256": "c41f312cc4aec01cca1aab5b9b9c88170b85b5bcb2c7319928b49624b8d12bc0",
                   # per launch at 231 receivers x 26 frequencies, by grid-sum splits (read + write)
